@@ -109,7 +109,7 @@ __device__ inline M3 m3_mul(const M3& a, const M3& b) {
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) {
       cx<double> v = mk(0.0, 0.0);
-      for (int k = 0; k < 3; ++k) v = v + cmul(a.e[i][k], b.e[k][j]);
+      for (int k = 0; k < 3; ++k) v = cmac(v, a.e[i][k], b.e[k][j]);
       c.e[i][j] = v;
     }
   return c;
@@ -192,8 +192,8 @@ __device__ double inv6(cx<double> a[6][6], cx<double> inv[6][6]) {
       if (r == c) continue;
       cx<double> f = a[r][c];
       for (int j = 0; j < 6; ++j) {
-        a[r][j] = a[r][j] - cmul(f, a[c][j]);
-        inv[r][j] = inv[r][j] - cmul(f, inv[c][j]);
+        a[r][j] = cnmac(a[r][j], f, a[c][j]);
+        inv[r][j] = cnmac(inv[r][j], f, inv[c][j]);
       }
     }
   }

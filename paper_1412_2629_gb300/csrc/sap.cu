@@ -509,8 +509,8 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
     for (int s = 0; s < 4; ++s)
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        x.c[s][c] = x.c[s][c] + cmul(alpha, rho.c[s][c]);
-        rho.c[s][c] = rho.c[s][c] - cmul(alpha, pv.c[s][c]);
+        x.c[s][c] = cmac(x.c[s][c], alpha, rho.c[s][c]);
+        rho.c[s][c] = cnmac(rho.c[s][c], alpha, pv.c[s][c]);
       }
     st_buf(sE, Hd, tid, rho);
     __syncthreads();
@@ -1240,8 +1240,8 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
       for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          x.c[s][c] = x.c[s][c] + cmul(alpha, rho.c[s][c]);
-          rho.c[s][c] = rho.c[s][c] - cmul(alpha, pv.c[s][c]);
+          x.c[s][c] = cmac(x.c[s][c], alpha, rho.c[s][c]);
+          rho.c[s][c] = cnmac(rho.c[s][c], alpha, pv.c[s][c]);
         }
       // the last MR step hands x to the reconstruction phase instead of rho
       st_hbuf(sE, Hd, i, h, ph == nph - 2 ? x : rho);
