@@ -105,7 +105,7 @@ struct dd_ctx {
   double* Ucanon = nullptr;
   double2* U64 = nullptr;
   float2* U32 = nullptr;
-  uint32_t* U16 = nullptr;
+  uint4* U16 = nullptr;
   bool have_gauge = false;
   // clover
   double2* C64 = nullptr;
@@ -297,7 +297,7 @@ extern "C" dd_status dd_load_gauge(dd_ctx* c, const double* U, int where) {
     TRY(dalloc(c, &c->Ucanon, n * 8));
     TRY(dalloc(c, &c->U64, n * 8));
     TRY(dalloc(c, &c->U32, n * 4));
-    TRY(dalloc(c, &c->U16, n * 2));
+    TRY(dalloc(c, &c->U16, (size_t)g.V * LINK16_BYTES_PER_SITE));
   }
   TRY(cuda_check(c, cudaMemcpyAsync(c->Ucanon, U, n * 8, where == DD_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->st),
                  "gauge copy"));
@@ -455,8 +455,8 @@ static SapState sap_state(dd_ctx* c, int prec, const dd_sap_params* p, int nrhs)
   S.u_norm = b.u_norm;
   S.faces = b.faces;
   S.err = c->sap_err;
-  S.mat_in_smem = sap_mat_fits_smem(c->g, prec);
   S.threads_per_site = p->threads_per_site ? p->threads_per_site : 2;
+  S.mat_in_smem = sap_mat_fits_smem(c->g, prec, S.threads_per_site);
   S.inject_wait_timeout = c->inject_wait_timeout;
   S.half_arith = p->storage_prec == DD_PREC_FP16_H2;
   return S;
@@ -1759,7 +1759,7 @@ extern "C" dd_status dd_solve_lattices(dd_ctx** ctxs, int nlat, const double* co
   for (int l = 0; l < nlat; ++l) {
     if (!ctxs[l] || !f[l] || !x[l]) return DD_ERR_INVALID;
     if (!ctxs[l]->have_clover) return fail(c0, DD_ERR_NO_CLOVER, "clover not built on lattice " + std::to_string(l));
-    if (ctxs[l]->g.Vd != c0->g.Vd || sap_mat_fits_smem(ctxs[l]->g, P16) != sap_mat_fits_smem(c0->g, P16))
+    if (ctxs[l]->g.Vd != c0->g.Vd || sap_mat_fits_smem(ctxs[l]->g, P16, 2) != sap_mat_fits_smem(c0->g, P16, 2))
       return fail(c0, DD_ERR_DIMS, "lattices of one launch need the same domain volume");
     for (int q = 0; q < l; ++q)
       if (ctxs[q] == ctxs[l]) return fail(c0, DD_ERR_INVALID, "a context appears twice");
@@ -2371,8 +2371,8 @@ extern "C" dd_status dd_autotune(dd_ctx* c, int storage_prec, int domain_out[4],
     }
     if (c->trace) {
       const long long n = t->g.ND / 2;
-      const bool big = sap_smem_bytes(t->g, sap_prec(storage_prec), sap_mat_fits_smem(t->g, sap_prec(storage_prec))) >
-                       116 * 1024;
+      const int pr = sap_prec(storage_prec);
+      const bool big = sap_smem_bytes(t->g, pr, sap_mat_fits_smem(t->g, pr, cd.tps), cd.tps) > 113 * 1024;
       fprintf(stderr,
               "[dd] autotune b %dx%dx%dx%d I_S %d I_d %d tps %d: %d it, %.3f ms, residual %.3e, %.4f ms/e-fold, "
               "load %.2f\n",
@@ -2517,8 +2517,8 @@ extern "C" dd_status dd_sap_precondition_noalloc(dd_ctx* c, const float* in, flo
   S.u_norm = un_bytes ? (float*)(base + off) : nullptr; off += up(un_bytes);
   S.faces = (float4*)(base + off); off += up(f_bytes);
   S.err = (int*)(base + off);
-  S.mat_in_smem = sap_mat_fits_smem(g, prec);
   S.threads_per_site = p->threads_per_site ? p->threads_per_site : 2;
+  S.mat_in_smem = sap_mat_fits_smem(g, prec, S.threads_per_site);
   S.half_arith = p->storage_prec == DD_PREC_FP16_H2;
   S.inject_wait_timeout = c->inject_wait_timeout;
   // the error word must start at zero; residual, solution and faces are written before

@@ -425,7 +425,20 @@ template <> struct SpinorPtr<__half> {
 template <typename T> struct Arith { typedef float type; };
 template <> struct Arith<double> { typedef double type; };
 
-// Gauge links: [domain][mu][9][r] of (double2 | float2 | half2); entry j = 3 a + b.
+// Gauge links of one domain.  FP64: [mu][9][r] double2, entry 3 a + b.  FP32 and FP16 group
+// the entries by diagonals, D0 = (00, 11, 22), D1 = (01, 12, 20), D2 = (10, 21, 02): the
+// transposed matrix is the same list with D1 and D2 exchanged, so a kernel whose lanes need U
+// or U^dag reads both with the same instructions from two base addresses.
+//   FP32: [mu][9][r] float2 in the order D0, D1, D2.
+//   FP16: [mu][2][r] of 16-byte units (D1, 00) and (D2, 00), then [mu][r] of 8-byte units
+//         (11, 22): three vector loads per link, 40 bytes (00 is held twice so that either
+//         16-byte unit can come first).
+__host__ __device__ constexpr int link_row(int k) { return k < 3 ? k : k < 6 ? k - 3 : (k - 5) % 3; }
+__host__ __device__ constexpr int link_col(int k) { return k < 3 ? k : k < 6 ? (k - 2) % 3 : k - 6; }
+// and back: the place of entry j = 3 a + b in that order (0, 3, 8, 6, 1, 4, 5, 7, 2)
+__host__ __device__ constexpr int link_slot(int j) { return (int)((0x275416830ull >> (4 * j)) & 15); }
+constexpr int LINK16_BYTES_PER_SITE = 4 * 40;
+
 template <typename T> struct LinkPtr;
 template <> struct LinkPtr<double> {
   const double2* p;
@@ -442,16 +455,25 @@ template <> struct LinkPtr<float> {
     long long d = s >> g.lgVd, r = s & (g.Vd - 1);
     const float2* q = p + (((d * 4 + mu) * 9) << g.lgVd) + r;
 #pragma unroll
-    for (int j = 0; j < 9; ++j) { float2 v = __ldg(q + ((long long)j << g.lgVd)); U.e[j / 3][j % 3] = mk(v.x, v.y); }
+    for (int j = 0; j < 9; ++j) {
+      float2 v = __ldg(q + ((long long)link_slot(j) << g.lgVd));
+      U.e[j / 3][j % 3] = mk(v.x, v.y);
+    }
   }
 };
+__device__ inline void link_from_words(uint4 d1, uint4 d2, uint2 d0, Link<float>& U) {
+  const uint32_t w[9] = {d1.w, d0.x, d0.y, d1.x, d1.y, d1.z, d2.x, d2.y, d2.z};
+#pragma unroll
+  for (int k = 0; k < 9; ++k) { float2 v = h2f(w[k]); U.e[link_row(k)][link_col(k)] = mk(v.x, v.y); }
+}
 template <> struct LinkPtr<__half> {
-  const uint32_t* p;
+  const uint4* p;
   __device__ void load(const Geom& g, long long s, int mu, Link<float>& U) const {
     long long d = s >> g.lgVd, r = s & (g.Vd - 1);
-    const uint32_t* q = p + (((d * 4 + mu) * 9) << g.lgVd) + r;
-#pragma unroll
-    for (int j = 0; j < 9; ++j) { float2 v = h2f(__ldg(q + ((long long)j << g.lgVd))); U.e[j / 3][j % 3] = mk(v.x, v.y); }
+    const uint4* q = p + ((d * 10) << g.lgVd);   // 10 16-byte units per site
+    const uint2* q2 = reinterpret_cast<const uint2*>(q + (8 << g.lgVd));
+    link_from_words(__ldg(q + ((2 * mu) << g.lgVd) + r), __ldg(q + ((2 * mu + 1) << g.lgVd) + r),
+                    __ldg(q2 + (mu << g.lgVd) + r), U);
   }
 };
 

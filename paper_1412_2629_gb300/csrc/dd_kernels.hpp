@@ -28,7 +28,7 @@ struct CloverView { const void* m; int prec; };
 void launch_pack_spinor(const Geom& g, const void* canon, int canon_prec, FieldView out, cudaStream_t st);
 void launch_unpack_spinor(const Geom& g, FieldView in, void* canon, int canon_prec, cudaStream_t st);
 void launch_pack_gauge(const Geom& g, const double* canon, int t_antiperiodic, double2* u64, float2* u32,
-                       uint32_t* u16, cudaStream_t st);
+                       uint4* u16, cudaStream_t st);
 // Builds clover (all sites, with the 1/(2 kappa) diagonal) in FP64/FP32/FP16 and the
 // Schwarz matrices (even sites: clover block; odd sites: its inverse) in FP32/FP16.
 // status[0] counts sites with a (near-)singular block.
@@ -86,8 +86,8 @@ int sap_half_sweep(const Geom& g, const SapState& S, int colour, int first, int 
 // Several lattices (same domain shape, FP16 storage) in one launch per half-sweep.
 int sap_half_sweep_lattices(const Geom* gs, const SapState* Ss, int nlat, int colour, int first, int use_faces,
                             int last, const float4* const* v, float4* const* z, int i_domain, cudaStream_t st);
-size_t sap_smem_bytes(const Geom& g, int mat_prec, bool mat_in_smem);
-bool sap_mat_fits_smem(const Geom& g, int mat_prec);
+size_t sap_smem_bytes(const Geom& g, int mat_prec, bool mat_in_smem, int threads_per_site);
+bool sap_mat_fits_smem(const Geom& g, int mat_prec, int threads_per_site);
 int sap_max_domain_sites();
 // Fixed scratch array of the allocation-free Schwarz entry point (size, device address).
 size_t sap_noalloc_scratch_bytes();

@@ -137,7 +137,7 @@ void launch_apply_A(const Geom& g, GaugeView U, CloverView C, FieldView in, Fiel
                                               fi, res);
   } else {
     SpinorPtr<__half> fi{res ? (uint4*)f->data : nullptr, res ? f->norm : nullptr};
-    apply_A_kernel<__half><<<nb, 256, 0, st>>>(g, LinkPtr<__half>{(const uint32_t*)U.links},
+    apply_A_kernel<__half><<<nb, 256, 0, st>>>(g, LinkPtr<__half>{(const uint4*)U.links},
                                                CloverPtr<__half>{(const uint4*)C.m},
                                                SpinorPtr<__half>{(uint4*)in.data, in.norm},
                                                SpinorPtr<__half>{(uint4*)out.data, out.norm}, fi, res);
@@ -244,7 +244,7 @@ void launch_apply_A_multi(const Geom& g, GaugeView U, CloverView C, FieldView in
     // FP16 fields are V * 52 bytes each (values, then the per-site norms) and follow each
     // other: 13 V / 4 uint4 units or 13 V floats apart (V is a multiple of 64)
     apply_A_multi_kernel<__half, NR><<<grid, 128, 0, st>>>(
-        g, LinkPtr<__half>{(const uint32_t*)U.links}, CloverPtr<__half>{(const uint4*)C.m},
+        g, LinkPtr<__half>{(const uint4*)U.links}, CloverPtr<__half>{(const uint4*)C.m},
         SpinorPtr<__half>{(uint4*)in.data, in.norm}, SpinorPtr<__half>{(uint4*)out.data, out.norm}, 13 * g.V / 4,
         13 * g.V, nrhs, nullptr, nullptr);
   }

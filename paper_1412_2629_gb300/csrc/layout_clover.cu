@@ -76,7 +76,7 @@ void launch_unpack_spinor(const Geom& g, FieldView in, void* canon, int canon_pr
   else unpack_dispatch(g, in, (float*)canon, st);
 }
 
-__global__ void pack_gauge_kernel(Geom g, const double* canon, int anti, double2* u64, float2* u32, uint32_t* u16) {
+__global__ void pack_gauge_kernel(Geom g, const double* canon, int anti, double2* u64, float2* u32, uint4* u16) {
   long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (s >= g.V) return;
   Site st = decode(g, s);
@@ -86,17 +86,24 @@ __global__ void pack_gauge_kernel(Geom g, const double* canon, int anti, double2
   long long d = st.d, r = s & (g.Vd - 1);
   for (int mu = 0; mu < 4; ++mu) {
     double sg = (anti && mu == 3 && x[3] == g.L[3] - 1) ? -1.0 : 1.0;
-    for (int j = 0; j < 9; ++j) {
+    uint32_t w[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const int j = 3 * link_row(k) + link_col(k);
       double re = sg * q[18 * mu + 2 * j], im = sg * q[18 * mu + 2 * j + 1];
-      long long a = (((d * 4 + mu) * 9 + j) << g.lgVd) + r;
-      u64[a] = make_double2(re, im);
-      u32[a] = make_float2((float)re, (float)im);
-      u16[a] = f2h((float)re, (float)im);
+      const long long a = ((d * 4 + mu) * 9) << g.lgVd;
+      u64[a + ((long long)j << g.lgVd) + r] = make_double2(re, im);
+      u32[a + ((long long)k << g.lgVd) + r] = make_float2((float)re, (float)im);
+      w[k] = f2h((float)re, (float)im);
     }
+    uint4* b = u16 + ((d * 10) << g.lgVd);
+    b[((2 * mu) << g.lgVd) + r] = make_uint4(w[3], w[4], w[5], w[0]);
+    b[((2 * mu + 1) << g.lgVd) + r] = make_uint4(w[6], w[7], w[8], w[0]);
+    reinterpret_cast<uint2*>(b + (8 << g.lgVd))[(mu << g.lgVd) + r] = make_uint2(w[1], w[2]);
   }
 }
 
-void launch_pack_gauge(const Geom& g, const double* canon, int anti, double2* u64, float2* u32, uint32_t* u16,
+void launch_pack_gauge(const Geom& g, const double* canon, int anti, double2* u64, float2* u32, uint4* u16,
                        cudaStream_t st) {
   pack_gauge_kernel<<<nblk(g.V, 128), 128, 0, st>>>(g, canon, anti, u64, u32, u16);
 }
@@ -270,14 +277,17 @@ __global__ void __launch_bounds__(128) build_clover_kernel(Geom g, const double*
     c32[unit_addr(g, s, 18, u)] = make_float4((float)cl[4 * u], (float)cl[4 * u + 1], (float)cl[4 * u + 2], (float)cl[4 * u + 3]);
     s32[unit_addr(g, s, 18, u)] = make_float4((float)sm[4 * u], (float)sm[4 * u + 1], (float)sm[4 * u + 2], (float)sm[4 * u + 3]);
   }
+  uint32_t v[36];   // Schwarz matrix words: block 0 (18), block 1 (18)
+  for (int k = 0; k < 36; ++k) v[k] = f2h((float)sm[2 * k], (float)sm[2 * k + 1]);
   for (int u = 0; u < 9; ++u) {
-    uint32_t w[4], v[4];
-    for (int e = 0; e < 4; ++e) {
-      w[e] = f2h((float)cl[8 * u + 2 * e], (float)cl[8 * u + 2 * e + 1]);
-      v[e] = f2h((float)sm[8 * u + 2 * e], (float)sm[8 * u + 2 * e + 1]);
-    }
+    uint32_t w[4];
+    for (int e = 0; e < 4; ++e) w[e] = f2h((float)cl[8 * u + 2 * e], (float)cl[8 * u + 2 * e + 1]);
     c16[unit_addr(g, s, 9, u)] = make_uint4(w[0], w[1], w[2], w[3]);
-    s16[unit_addr(g, s, 9, u)] = make_uint4(v[0], v[1], v[2], v[3]);
+    // units 0..3: words 0..15 of block 0, 4..7: of block 1, 8: words 16, 17 of both, so each
+    // block is four 16-byte units and one 8-byte half unit
+    const int k = u < 8 ? 18 * (u >> 2) + 4 * (u & 3) : 16;
+    s16[unit_addr(g, s, 9, u)] = u < 8 ? make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3])
+                                       : make_uint4(v[16], v[17], v[34], v[35]);
   }
 }
 

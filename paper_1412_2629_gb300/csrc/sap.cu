@@ -22,6 +22,7 @@
 // owns even site i and odd site i and keeps x, rho and r_o in registers, so every MR
 // step runs on chip.  The MR inner products are reduced with warp shuffles and one
 // exchange through shared memory.
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -30,47 +31,93 @@
 namespace dd {
 
 // ------------------------------------------------------------------ matrix views
+// Links and Schwarz matrices of one domain, in shared or global memory.  link<...>(mu, r, h)
+// is U_mu of site r for h = 0 and its adjoint for h = 1 (h may differ between lanes: see the
+// diagonal grouping of the link layout); block(r, h) the packed Hermitian 6x6 block of
+// chirality h.
 template <typename MT> struct MatBlock;
 
 template <> struct MatBlock<__half> {
-  const uint32_t* lk;  // [mu][9][Vd] half2
-  const uint4* cm;     // [9][Vd]     8 halves
+  const uint4* l4;     // [mu][2][Vd], then
+  const uint2* l2;     // [mu][Vd]
+  const uint4* cm;     // [8][Vd], then 8-byte halves [Vd][2]
   int Vd;
-  __device__ void link(int mu, int r, Link<float>& U) const {
-#pragma unroll
-    for (int j = 0; j < 9; ++j) { float2 v = h2f(lk[(mu * 9 + j) * Vd + r]); U.e[j / 3][j % 3] = mk(v.x, v.y); }
+  __device__ void set_links(const void* p) {
+    l4 = reinterpret_cast<const uint4*>(p);
+    l2 = reinterpret_cast<const uint2*>(l4 + 8 * Vd);
   }
-  __device__ void mat(int r, float m[72]) const {
+  __device__ void set_mats(const void* p) { cm = reinterpret_cast<const uint4*>(p); }
+  // the nine entries (re, im) in the order D0, D1, D2 of U (h = 0) or U^dag (h = 1)
+  __device__ void words(int mu, int r, int h, uint32_t w[9]) const {
+    const uint4 a = l4[(2 * mu + h) * Vd + r], b = l4[(2 * mu + 1 - h) * Vd + r];
+    const uint2 c = l2[mu * Vd + r];
+    const uint32_t conj = h ? 0x80000000u : 0u;   // the sign of the imaginary halves
+    const uint32_t v[9] = {a.w, c.x, c.y, a.x, a.y, a.z, b.x, b.y, b.z};
 #pragma unroll
-    for (int u = 0; u < 9; ++u) {
-      uint4 v = cm[u * Vd + r];
-      uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    for (int k = 0; k < 9; ++k) w[k] = v[k] ^ conj;
+  }
+  __device__ void link(int mu, int r, int h, Link<float>& U) const {
+    uint32_t w[9];
+    words(mu, r, h, w);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) { float2 f = h2f(w[e]); m[8 * u + 2 * e] = f.x; m[8 * u + 2 * e + 1] = f.y; }
+    for (int k = 0; k < 9; ++k) { float2 v = h2f(w[k]); U.e[link_row(k)][link_col(k)] = mk(v.x, v.y); }
+  }
+  __device__ void block_words(int r, int h, uint32_t w[18]) const {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint4 v = cm[(4 * h + u) * Vd + r];
+      w[4 * u] = v.x;
+      w[4 * u + 1] = v.y;
+      w[4 * u + 2] = v.z;
+      w[4 * u + 3] = v.w;
     }
+    const uint2 v = reinterpret_cast<const uint2*>(cm + 8 * Vd)[2 * r + h];
+    w[16] = v.x;
+    w[17] = v.y;
   }
-  static constexpr int link_bytes_per_site = 4 * 9 * 4;
+  __device__ void block(int r, int h, float m[36]) const {
+    uint32_t w[18];
+    block_words(r, h, w);
+#pragma unroll
+    for (int k = 0; k < 18; ++k) { float2 f = h2f(w[k]); m[2 * k] = f.x; m[2 * k + 1] = f.y; }
+  }
+  static constexpr int link_bytes_per_site = LINK16_BYTES_PER_SITE;
   static constexpr int mat_bytes_per_site = 9 * 16;
 };
 
 template <> struct MatBlock<float> {
-  const float2* lk;    // [mu][9][Vd]
+  const float2* lk;    // [mu][9][Vd], entries in the order D0, D1, D2
   const float4* cm;    // [18][Vd]
   int Vd;
-  __device__ void link(int mu, int r, Link<float>& U) const {
+  __device__ void set_links(const void* p) { lk = reinterpret_cast<const float2*>(p); }
+  __device__ void set_mats(const void* p) { cm = reinterpret_cast<const float4*>(p); }
+  __device__ void link(int mu, int r, int h, Link<float>& U) const {
+    const float2* q = lk + mu * 9 * Vd + r;
+    const float2* q1 = q + 3 * h * Vd;    // h = 1: D2 in the place of D1 and
+    const float2* q2 = q - 3 * h * Vd;    // D1 in the place of D2
+    const uint32_t conj = h ? 0x80000000u : 0u;
 #pragma unroll
-    for (int j = 0; j < 9; ++j) { float2 v = lk[(mu * 9 + j) * Vd + r]; U.e[j / 3][j % 3] = mk(v.x, v.y); }
+    for (int k = 0; k < 9; ++k) {
+      const float2 v = (k < 3 ? q : k < 6 ? q1 : q2)[k * Vd];
+      U.e[link_row(k)][link_col(k)] = mk(v.x, __uint_as_float(__float_as_uint(v.y) ^ conj));
+    }
   }
-  __device__ void mat(int r, float m[72]) const {
+  __device__ void block(int r, int h, float m[36]) const {
 #pragma unroll
-    for (int u = 0; u < 18; ++u) {
-      float4 v = cm[u * Vd + r];
+    for (int u = 0; u < 9; ++u) {
+      const float4 v = cm[(9 * h + u) * Vd + r];
       m[4 * u] = v.x; m[4 * u + 1] = v.y; m[4 * u + 2] = v.z; m[4 * u + 3] = v.w;
     }
   }
   static constexpr int link_bytes_per_site = 4 * 9 * 8;
   static constexpr int mat_bytes_per_site = 18 * 16;
 };
+
+template <typename MT>
+__device__ inline void site_mat(const MatBlock<MT>& M, int r, float m[72]) {
+  M.block(r, 0, m);
+  M.block(r, 1, m + 36);
+}
 
 // ------------------------------------------------------------------ work buffers
 __device__ inline void ld_buf(const float4* buf, int Hd, int i, Spinor<float>& v) {
@@ -160,7 +207,7 @@ __device__ inline void inside_hop_mu(const Geom& g, const int l[4], int lex, int
     int j = (lex + g.bstride[MU]) >> 1;
     ld_buf(src, g.Hd, j, psi);
     project<MU, -1>(psi, h);
-    M.link(MU, r_self, L);
+    M.link(MU, r_self, 0, L);
     su3_mul(L, h, uh);
     accum_recon<MU, -1>(acc, uh);
   }
@@ -168,7 +215,7 @@ __device__ inline void inside_hop_mu(const Geom& g, const int l[4], int lex, int
     int j = (lex - g.bstride[MU]) >> 1;
     ld_buf(src, g.Hd, j, psi);
     project<MU, +1>(psi, h);
-    M.link(MU, (1 - p) * g.Hd + j, L);
+    M.link(MU, (1 - p) * g.Hd + j, 0, L);
     su3_dag_mul(L, h, uh);
     accum_recon<MU, +1>(acc, uh);
   }
@@ -214,7 +261,7 @@ __device__ inline void face_hop_mu(const Geom& g, int d, const int n[4], const i
     const float4* q = faces + (dn * g.face_block + g.face_off[2 * MU] + face_index(g, l, MU)) * 3;
     ld_half(q, h);
     Link<float> L;
-    M.link(MU, r_self, L);
+    M.link(MU, r_self, 0, L);
     su3_mul(L, h, uh);
     accum_recon<MU, -1>(acc, uh);
   }
@@ -246,7 +293,7 @@ __device__ inline void face_write_mu(const Geom& g, long long d, const int l[4],
   if (l[MU] == g.b[MU] - 1) {
     project<MU, +1>(dl, h);
     Link<float> L;
-    M.link(MU, r_self, L);
+    M.link(MU, r_self, 0, L);
     su3_dag_mul(L, h, uh);
     st_half(faces + (d * g.face_block + g.face_off[2 * MU + 1] + face_index(g, l, MU)) * 3, uh);
   }
@@ -286,7 +333,7 @@ __device__ inline unsigned long long globaltimer_ns() {
 // Wait for the given phase parity of the barrier, for at most limit_ns nanoseconds;
 // returns false if the limit ran out.
 __device__ inline bool mbar_wait(uint64_t* bar, uint32_t phase, unsigned long long limit_ns) {
-  const unsigned long long t0 = globaltimer_ns();
+  unsigned long long t0 = 0;
   while (true) {
     uint32_t ok = 0;
     asm volatile(
@@ -295,7 +342,9 @@ __device__ inline bool mbar_wait(uint64_t* bar, uint32_t phase, unsigned long lo
         : "r"(smem_u32(bar)), "r"(phase)
         : "memory");
     if (ok) return true;
-    if (globaltimer_ns() - t0 > limit_ns) return false;
+    const unsigned long long now = globaltimer_ns();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > limit_ns) return false;
   }
 }
 
@@ -353,20 +402,17 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
   const long long d = n[0] + (long long)g.dstride[1] * n[1] + (long long)g.dstride[2] * n[2] +
                       (long long)g.dstride[3] * n[3];
 
-  const size_t lk_elems = (size_t)4 * 9 * Vd;
   const size_t lk_bytes = (size_t)MatBlock<MT>::link_bytes_per_site * Vd;
   const size_t cm_bytes = (size_t)MatBlock<MT>::mat_bytes_per_site * Vd;
   char* sbase = reinterpret_cast<char*>(smem);
   MatBlock<MT> M;
   M.Vd = Vd;
-  typedef typename std::remove_const<typename std::remove_pointer<decltype(M.lk)>::type>::type LkT;
-  typedef typename std::remove_const<typename std::remove_pointer<decltype(M.cm)>::type>::type CmT;
-  const LkT* glk = reinterpret_cast<const LkT*>(a.links) + d * lk_elems;
-  const CmT* gcm = reinterpret_cast<const CmT*>(a.smat) + d * (cm_bytes / sizeof(CmT));
+  const char* glk = reinterpret_cast<const char*>(a.links) + d * (long long)lk_bytes;
+  const char* gcm = reinterpret_cast<const char*>(a.smat) + d * (long long)cm_bytes;
   float4* sE;
   if (MSMEM) {
-    M.lk = reinterpret_cast<const LkT*>(sbase);
-    M.cm = reinterpret_cast<const CmT*>(sbase + lk_bytes);
+    M.set_links(sbase);
+    M.set_mats(sbase + lk_bytes);
     sE = reinterpret_cast<float4*>(sbase + lk_bytes + cm_bytes);
     if (tid == 0) {
       mbar_init(&mbar, 1);
@@ -381,8 +427,8 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
       if (a.extra_tx) mbar_expect_tx(&mbar_inj, a.extra_tx);
     }
   } else {
-    M.lk = glk;
-    M.cm = gcm;
+    M.set_links(glk);
+    M.set_mats(gcm);
     sE = smem;
   }
   float4* sO = sE + 6 * Hd;
@@ -446,7 +492,7 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
   // 2. even-odd preparation
   float m[72];
   Spinor<float> t, acc, rho, x;
-  M.mat(r_o, m);
+  site_mat(M, r_o, m);
   clover_mul(m, ro, t);
   st_buf(sO, Hd, tid, t);
   __syncthreads();
@@ -468,7 +514,7 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
     // odd sites: t = A_oo^{-1} H_oe rho
     zero(acc);
     inside_hops(g, lo, lex_o, 1, r_o, sE, M, acc);
-    M.mat(r_o, m);
+    site_mat(M, r_o, m);
     clover_mul(m, acc, t);
     st_buf(sO, Hd, tid, t);
     __syncthreads();
@@ -476,7 +522,7 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
     zero(acc);
     inside_hops(g, le, lex_e, 0, r_e, sO, M, acc);
     Spinor<float> pv;
-    M.mat(r_e, m);
+    site_mat(M, r_e, m);
     clover_mul(m, rho, pv);
     float pr_re = 0.f, pr_im = 0.f, pp = 0.f;
 #pragma unroll
@@ -526,7 +572,7 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc.c[s][c] = ro.c[s][c] + 0.5f * acc.c[s][c];
   Spinor<float> dlo;
-  M.mat(r_o, m);
+  site_mat(M, r_o, m);
   clover_mul(m, acc, dlo);
 
   // solution and residual
@@ -563,256 +609,152 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
 }
 
 // ------------------------------------------------------------------ two threads per site
-// Same algorithm with 2 Hd threads per domain.  In the MR phases thread (h, i) works on
-// even site i and odd site i: h = 0 computes the hops along x and y, h = 1 along z and t,
-// and each keeps chirality half h (spins 2h, 2h+1) of x, rho and r_o.  Because the clover
-// block and its inverse act within one chirality, the only exchange is of the two
-// threads' partial hop sums, half by half, through the shared work buffer that the phase
-// does not otherwise read.  Prologue and epilogue run one thread per site (h = parity).
+// Same algorithm with 2 Hd threads per domain.  Lanes l and l + 16 of a warp (h = 0, 1) work
+// on even site i and odd site i: h = 0 takes the four forward hops of a site, h = 1 the four
+// backward hops, and each keeps chirality half h (spins 2h, 2h+1) of x, rho and the odd
+// solution.  The clover block and its inverse act within one chirality, so the only exchange
+// is of the two lanes' partial hop sums: one shuffle per number.
+//
+// Both lanes run the same instructions.  In lane h's frame the own spins are 2h, 2h+1 and
+// the others follow; with gamma_mu = [[0, B], [B^dag, 0]] a forward hop (1 - gamma) projects to
+// own - B other and adds -B^dag U h to the other spins, a backward hop (1 + gamma) in the frame
+// of h = 1 to own + B^dag other and +B U^dag h.  B_k^dag = -B_k in space, so the two agree; in
+// time B = 1 and they differ by a sign, which is a register.  The adjoint link comes from
+// the same loads (MatBlock).
+//
+// Hops that leave the domain read a zero spinor (eight zero slots behind every unit of the
+// work buffers, one per 16-byte bank group), so no hop is conditional and the loads of
+// one hop overlap the arithmetic of another.
+//
+// Measured against the form with the hop directions split over two warps (masked hops, the
+// partial sums exchanged through shared memory, faces read site by site from global memory):
+// half-sweep of 32^3x64 (8x4x4x4 domains, I_domain 4, FP16 storage) 571 -> 430 us, of 24^3x48
+// (4^4, I_domain 3) 162 -> 112 us, FP32 storage 32^3x64 679 -> 474 us; 12.0k -> 10.0k cycles and
+// 2029 -> 1860 instructions per warp and MR step, 28k -> 21k cycles a visit outside them.
+// Bound by instruction issue (74 % in the MR steps; FMA pipe 48 %, shared memory 53 %) and by
+// the latency of staging and output with one CTA per SM.
 
-// Half h of a site vector in a work buffer: units 3h .. 3h+2.
-__device__ inline void ld_hbuf(const float4* buf, int Hd, int i, int h, Half<float>& v) {
-#pragma unroll
-  for (int u = 0; u < 3; ++u) {
-    float4 q = buf[(3 * h + u) * Hd + i];
-    int k = 2 * u;
-    v.c[k / 3][k % 3] = mk(q.x, q.y);
-    v.c[(k + 1) / 3][(k + 1) % 3] = mk(q.z, q.w);
-  }
-}
-__device__ inline void st_hbuf(float4* buf, int Hd, int i, int h, const Half<float>& v) {
-#pragma unroll
-  for (int u = 0; u < 3; ++u) {
-    int k = 2 * u;
-    buf[(3 * h + u) * Hd + i] = make_float4(v.c[k / 3][k % 3].re, v.c[k / 3][k % 3].im, v.c[(k + 1) / 3][(k + 1) % 3].re,
-                                            v.c[(k + 1) / 3][(k + 1) % 3].im);
-  }
-}
-__device__ inline void half_of(const Spinor<float>& s, int h, Half<float>& o) {
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) o.c[a][c] = h ? s.c[2 + a][c] : s.c[a][c];
-}
+constexpr int ZERO_SLOTS = 8;
 
-// Clover block H (36 reals) of site r.
-template <typename MT> struct BlockLoad;
-template <> struct BlockLoad<__half> {
-  template <int H>
-  __device__ static void load(const MatBlock<__half>& M, int r, float m[36]) {
-    // 72 halves in 9 units of 8; block H holds halves 36 H .. 36 H + 35 (units 4 H .. 4 H + 4)
-#pragma unroll
-    for (int u = 0; u < 5; ++u) {
-      uint4 v = M.cm[(4 * H + u) * M.Vd + r];
-      uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        float2 f = h2f(w[e]);
-        const int k = 8 * u + 2 * e - 4 * H;   // position inside the block
-        if (k >= 0 && k < 36) { m[k] = f.x; m[k + 1] = f.y; }
-      }
-    }
-  }
-};
-template <> struct BlockLoad<float> {
-  template <int H>
-  __device__ static void load(const MatBlock<float>& M, int r, float m[36]) {
-#pragma unroll
-    for (int u = 0; u < 9; ++u) {
-      float4 v = M.cm[(9 * H + u) * M.Vd + r];
-      m[4 * u] = v.x; m[4 * u + 1] = v.y; m[4 * u + 2] = v.z; m[4 * u + 3] = v.w;
-    }
-  }
-};
-
-template <typename MT>
-__device__ inline void block_apply(const MatBlock<MT>& M, int r, int h, const Half<float>& x, Half<float>& y) {
-  float m[36];
-  if (h == 0) BlockLoad<MT>::template load<0>(M, r, m);
-  else BlockLoad<MT>::template load<1>(M, r, m);
-  cx<float> v[6], w[6];
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) v[3 * s + c] = x.c[s][c];
-  clover_block_mul(m, v, w);
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) y.c[s][c] = w[3 * s + c];
-}
-
-// acc: this thread's partial sum over its two directions.  The other thread of the site
-// holds the rest.  Returns the full sum of chirality half h.  buf is scratch here.
-__device__ inline void exchange(const Spinor<float>& acc, int h, float4* buf, int Hd, int i, Half<float>& own) {
-  Half<float> give, mine, got;
-  half_of(acc, 1 - h, give);
-  half_of(acc, h, mine);
-  st_hbuf(buf, Hd, i, 1 - h, give);
-  __syncthreads();
-  ld_hbuf(buf, Hd, i, h, got);
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) own.c[a][c] = mine.c[a][c] + got.c[a][c];
-}
-
-// Store half h of the even-site residual; FP16 needs the norm of the whole site, which
-// the two threads share through nrm (2 Hd floats of shared memory).
-template <typename VT> struct EvenHalfStore;
-template <> struct EvenHalfStore<float> {
-  __device__ static void store(const EvenStore<float>& E, float*, long long d, int Hd, int i, int h,
-                               const Half<float>& v) {
-    st_hbuf(E.p + d * 6 * Hd, Hd, i, h, v);
-  }
-};
-template <> struct EvenHalfStore<__half> {
-  __device__ static void store(const EvenStore<__half>& E, float* nrm, long long d, int Hd, int i, int h,
-                               const Half<float>& v) {
-    float m = 0.f;
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) m = fmaxf(m, fmaxf(fabsf(v.c[a][c].re), fabsf(v.c[a][c].im)));
-    nrm[h * Hd + i] = m;
-    __syncthreads();
-    m = fmaxf(nrm[i], nrm[Hd + i]);
-    float inv = m > 0.f ? 1.f / m : 0.f;
-    if (h == 0) E.norm[d * Hd + i] = m;
-    uint2* q = reinterpret_cast<uint2*>(E.p);
-#pragma unroll
-    for (int t = 0; t < 3; ++t) {
-      int k = 2 * t;            // complex pair (k, k+1) of this half
-      int pair = 3 * h + t;     // pair number inside the site's 12 complex numbers
-      int u = pair >> 1, j = pair & 1;
-      q[((d * 3 + u) * Hd + i) * 2 + j] =
-          make_uint2(f2h(v.c[k / 3][k % 3].re * inv, v.c[k / 3][k % 3].im * inv),
-                     f2h(v.c[(k + 1) / 3][(k + 1) % 3].re * inv, v.c[(k + 1) / 3][(k + 1) % 3].im * inv));
-    }
-  }
-};
-
-// ------------------------------------------------------------------ face code, run-time direction
-// Face coupling and face output run once per visit; with the direction as a loop variable
-// (only the spin projection and reconstruction are selected per direction, warp-uniform)
-// their code stays small.
-__device__ inline void project_rt(int mu, int dir, const Spinor<float>& p, Half<float>& h) {
-  // forward hop uses (1 - gamma_mu), backward (1 + gamma_mu)
-  switch (2 * mu + (dir < 0)) {
-    case 0: project<0, -1>(p, h); break;
-    case 1: project<0, +1>(p, h); break;
-    case 2: project<1, -1>(p, h); break;
-    case 3: project<1, +1>(p, h); break;
-    case 4: project<2, -1>(p, h); break;
-    case 5: project<2, +1>(p, h); break;
-    case 6: project<3, -1>(p, h); break;
-    default: project<3, +1>(p, h); break;
-  }
-}
-__device__ inline void recon_rt(int mu, int dir, Spinor<float>& acc, const Half<float>& h) {
-  switch (2 * mu + (dir < 0)) {
-    case 0: accum_recon<0, -1>(acc, h); break;
-    case 1: accum_recon<0, +1>(acc, h); break;
-    case 2: accum_recon<1, -1>(acc, h); break;
-    case 3: accum_recon<1, +1>(acc, h); break;
-    case 4: accum_recon<2, -1>(acc, h); break;
-    case 5: accum_recon<2, +1>(acc, h); break;
-    case 6: accum_recon<3, -1>(acc, h); break;
-    default: accum_recon<3, +1>(acc, h); break;
-  }
-}
-
-// U_mu(site r) for dir > 0, U_mu(site r)^dag for dir < 0.
-template <typename MT>
-__device__ inline void link_rt(const MatBlock<MT>& M, int mu, int r, int dir, Link<float>& U) {
-  Link<float> L;
-  M.link(mu, r, L);
-  if (dir > 0) {
-    U = L;
+template <int MU>
+__device__ __forceinline__ void frame_project(const Spinor<float>& p, float st, Half<float>& o) {
+  if constexpr (MU < 3) {
+    project<MU, -1>(p, o);
   } else {
 #pragma unroll
-    for (int a2 = 0; a2 < 3; ++a2)
+    for (int s = 0; s < 2; ++s)
 #pragma unroll
-      for (int b2 = 0; b2 < 3; ++b2) U.e[a2][b2] = mk(L.e[b2][a2].re, -L.e[b2][a2].im);
+      for (int c = 0; c < 3; ++c)
+        o.c[s][c] = mk(fmaf(st, p.c[2 + s][c].re, p.c[s][c].re), fmaf(st, p.c[2 + s][c].im, p.c[s][c].im));
+  }
+}
+template <int MU>
+__device__ __forceinline__ void frame_recon(Spinor<float>& acc, float st, const Half<float>& u) {
+  if constexpr (MU < 3) {
+    accum_recon<MU, -1>(acc, u);
+  } else {
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        acc.c[s][c] = acc.c[s][c] + u.c[s][c];
+        acc.c[2 + s][c] = mk(fmaf(st, u.c[s][c].re, acc.c[2 + s][c].re), fmaf(st, u.c[s][c].im, acc.c[2 + s][c].im));
+      }
   }
 }
 
-// Masks of the directions whose forward / backward neighbour is inside the domain.
-__device__ inline void inside_masks(const Geom& g, const int l[4], unsigned& fwd, unsigned& bwd) {
-  fwd = bwd = 0;
+// Three units (one chirality half) at site i of a buffer whose units are `stride` apart.
+__device__ __forceinline__ void ld_half3(const float4* q, int stride, cx<float> v[6]) {
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    fwd |= (l[mu] + 1 < g.b[mu] ? 1u : 0u) << mu;
-    bwd |= (l[mu] > 0 ? 1u : 0u) << mu;
+  for (int u = 0; u < 3; ++u) {
+    const float4 w = q[u * stride];
+    v[2 * u] = mk(w.x, w.y);
+    v[2 * u + 1] = mk(w.z, w.w);
   }
+}
+__device__ __forceinline__ void st_half3(float4* q, int stride, const Half<float>& v) {
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    const int k = 2 * u;
+    q[u * stride] = make_float4(v.c[k / 3][k % 3].re, v.c[k / 3][k % 3].im, v.c[(k + 1) / 3][(k + 1) % 3].re,
+                                v.c[(k + 1) / 3][(k + 1) % 3].im);
+  }
+}
+__device__ __forceinline__ void ld_half3(const float4* q, int stride, Half<float>& v) {
+  cx<float> w[6];
+  ld_half3(q, stride, w);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) v.c[k / 3][k % 3] = w[k];
 }
 
-// acc += couplings to the neighbouring domains from their face buffers (see face_hop_mu).
-template <typename MT>
-__device__ inline void face_hops_rt(const Geom& g, int d, const int n[4], const int l[4], unsigned fwd, unsigned bwd,
-                                    int r_self, const float4* faces, const MatBlock<MT>& M, Spinor<float>& acc) {
-  int fidx[4];
+// own half of the sum over the two lanes of a site
+__device__ __forceinline__ void join_halves(const Spinor<float>& acc, Half<float>& own) {
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) fidx[mu] = face_index(g, l, mu);
-#pragma unroll 1
-  for (int k = 0; k < 8; ++k) {
-    const int mu = k >> 1;
-    const int dir = (k & 1) ? -1 : 1;
-    if ((((dir > 0 ? fwd : bwd) >> mu) & 1u)) continue;   // neighbour inside: not a face hop
-    long long dn;
-    int fi;
-    switch (mu) {   // register arrays are only indexed with constants
-      case 0: dn = neighbour_domain(g, d, n, 0, dir); fi = fidx[0]; break;
-      case 1: dn = neighbour_domain(g, d, n, 1, dir); fi = fidx[1]; break;
-      case 2: dn = neighbour_domain(g, d, n, 2, dir); fi = fidx[2]; break;
-      default: dn = neighbour_domain(g, d, n, 3, dir); fi = fidx[3]; break;
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      own.c[s][c] = mk(acc.c[s][c].re + __shfl_xor_sync(0xffffffffu, acc.c[2 + s][c].re, 16),
+                       acc.c[s][c].im + __shfl_xor_sync(0xffffffffu, acc.c[2 + s][c].im, 16));
+}
+// the site's whole spinor in this lane's frame from the two lanes' own halves
+__device__ __forceinline__ void join_frame(const Half<float>& own, Spinor<float>& v) {
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      v.c[s][c] = own.c[s][c];
+      v.c[2 + s][c] = mk(__shfl_xor_sync(0xffffffffu, own.c[s][c].re, 16),
+                         __shfl_xor_sync(0xffffffffu, own.c[s][c].im, 16));
     }
-    const float4* q = faces + (dn * g.face_block + g.face_off[2 * mu + (dir > 0 ? 0 : 1)] + fi) * 3;
-    Half<float> h, uh;
-    ld_half(q, h);
-    if (dir > 0) {
-      Link<float> U;
-      M.link(mu, r_self, U);
-      su3_mul(U, h, uh);
-    } else {
-      uh = h;
-    }
-    recon_rt(mu, dir, acc, uh);
-  }
 }
 
-// Projected half-spinors of dl on this site's faces (see face_write_mu).
-template <typename MT>
-__device__ inline void face_write_rt(const Geom& g, long long d, const int l[4], unsigned fwd, unsigned bwd,
-                                     int r_self, float4* faces, const MatBlock<MT>& M, const Spinor<float>& dl) {
-  int fidx[4];
+// One chirality half of a stored spinor (N sites from p on).  The half-precision form is
+// [2][N] 16-byte units (the first four numbers of half h), then [N][2] 8-byte units, scaled
+// by the site's norm.
+template <typename T> struct HalfField;
+template <> struct HalfField<float> {
+  float4* p;
+  __device__ HalfField(void* base, float*, long long first, int) : p((float4*)base + first * 6) {}
+  __device__ void load(int N, int r, int h, Half<float>& v) const { ld_half3(p + 3 * h * N + r, N, v); }
+  __device__ void store(int N, int r, int h, const Half<float>& v) const { st_half3(p + 3 * h * N + r, N, v); }
+  __device__ void prefetch(int N, int r, int h) const {
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) fidx[mu] = face_index(g, l, mu);
-#pragma unroll 1
-  for (int k = 0; k < 8; ++k) {
-    const int mu = k >> 1;
-    const int side = k & 1;          // 0: -mu face (l_mu = 0), 1: +mu face (l_mu = b_mu - 1)
-    if (side == 0 ? ((bwd >> mu) & 1u) : ((fwd >> mu) & 1u)) continue;
-    int fi;
-    switch (mu) {
-      case 0: fi = fidx[0]; break;
-      case 1: fi = fidx[1]; break;
-      case 2: fi = fidx[2]; break;
-      default: fi = fidx[3]; break;
-    }
-    Half<float> h, uh;
-    // -mu face: P^-_mu dl for the neighbour's forward hop; +mu face: U^dag P^+_mu dl
-    project_rt(mu, side == 0 ? 1 : -1, dl, h);
-    if (side == 1) {
-      Link<float> U;
-      link_rt(M, mu, r_self, -1, U);
-      su3_mul(U, h, uh);
-    } else {
-      uh = h;
-    }
-    st_half(faces + (d * g.face_block + g.face_off[2 * mu + side] + fi) * 3, uh);
+    for (int u = 0; u < 3; ++u) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + (3 * h + u) * N + r));
   }
-}
+};
+template <> struct HalfField<__half> {
+  uint4* p;
+  float* norm;
+  __device__ HalfField(void* base, float* n, long long first, int) : p((uint4*)base + first * 3), norm(n + first) {}
+  __device__ void load(int N, int r, int h, Half<float>& v) const {
+    const float n = norm[r];
+    const uint4 a = p[h * N + r];
+    const uint2 b = reinterpret_cast<const uint2*>(p + 2 * N)[2 * r + h];
+    const uint32_t w[6] = {a.x, a.y, a.z, a.w, b.x, b.y};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const float2 f = h2f(w[k]);
+      v.c[k / 3][k % 3] = mk(f.x * n, f.y * n);
+    }
+  }
+  __device__ void store(int N, int r, int h, const Half<float>& v) const {
+    float m = 0.f;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) m = fmaxf(m, fmaxf(fabsf(v.c[k / 3][k % 3].re), fabsf(v.c[k / 3][k % 3].im)));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    const float inv = m > 0.f ? 1.f / m : 0.f;
+    if (h == 0) norm[r] = m;
+    uint32_t w[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w[k] = f2h(v.c[k / 3][k % 3].re * inv, v.c[k / 3][k % 3].im * inv);
+    p[h * N + r] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint2*>(p + 2 * N)[2 * r + h] = make_uint2(w[4], w[5]);
+  }
+  __device__ void prefetch(int N, int r, int h) const {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p + h * N + r));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const uint2*>(p + 2 * N) + 2 * r + h));
+  }
+};
 
 // ------------------------------------------------------------------ packed FP16 arithmetic
 // Optional form of the domain solve's two products, in half2 arithmetic (two FP16 lanes
@@ -847,21 +789,17 @@ __device__ inline void unpack_h2(const HalfH2& o, Half<float>& h) {
   }
 }
 
-// o = U h (DAG false) or U^dag h (DAG true); u: the 9 (re, im) words of U, stride Vd.
-template <bool DAG>
-__device__ inline void su3_h2(const __half2* u, int Vd, const HalfH2& h, HalfH2& o) {
-  __half2 U[9];
+// o = U h; w: the nine (re, im) words of U in the order D0, D1, D2.
+__device__ inline void su3_h2(const uint32_t w[9], const HalfH2& h, HalfH2& o) {
+  __half2 U[3][3];
 #pragma unroll
-  for (int e = 0; e < 9; ++e) U[e] = u[e * Vd];
+  for (int k = 0; k < 9; ++k) U[link_row(k)][link_col(k)] = as_h2(w[k]);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     __half2 re, im;
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      const __half2 e = DAG ? U[3 * b + a] : U[3 * a + b];
-      const __half2 er = __low2half2(e), ei = __high2half2(e);
-      // U h:     re += er h.re - ei h.im,  im += er h.im + ei h.re
-      // U^dag h: re += er h.re + ei h.im,  im += er h.im - ei h.re
+      const __half2 er = __low2half2(U[a][b]), ei = __high2half2(U[a][b]);
       if (b == 0) {
         re = __hmul2(er, h.re[b]);
         im = __hmul2(er, h.im[b]);
@@ -869,41 +807,31 @@ __device__ inline void su3_h2(const __half2* u, int Vd, const HalfH2& h, HalfH2&
         re = __hfma2(er, h.re[b], re);
         im = __hfma2(er, h.im[b], im);
       }
-      re = __hfma2(DAG ? ei : __hneg2(ei), h.im[b], re);
-      im = __hfma2(DAG ? __hneg2(ei) : ei, h.re[b], im);
+      re = __hfma2(__hneg2(ei), h.im[b], re);
+      im = __hfma2(ei, h.re[b], im);
     }
     o.re[a] = re;
     o.im[a] = im;
   }
 }
 
-// y = H x for block H of site r; the block's 18 words are 3 pairs of diagonal entries
-// and the 15 lower entries (re, im) in the order of tri(i, j).
-template <int H>
-__device__ inline void clover_block_h2(const MatBlock<__half>& M, int r, const __half2 x[6], __half2 y[6]) {
-  uint32_t w[20];   // units 4H .. 4H+4 of the site; block word k is w[2H + k]
-#pragma unroll
-  for (int u = 0; u < 5; ++u) {
-    uint4 v = M.cm[(4 * H + u) * M.Vd + r];
-    w[4 * u] = v.x;
-    w[4 * u + 1] = v.y;
-    w[4 * u + 2] = v.z;
-    w[4 * u + 3] = v.w;
-  }
+// y = H x; the block's 18 words are 3 pairs of diagonal entries and the 15 lower entries
+// (re, im) in the order of tri(i, j).
+__device__ inline void clover_block_h2(const uint32_t w[18], const __half2 x[6], __half2 y[6]) {
   const __half2 sgn = __floats2half2_rn(-1.f, 1.f);
   __half2 xs[6];   // i x = (-im, re)
 #pragma unroll
   for (int j = 0; j < 6; ++j) xs[j] = __hmul2(__lowhigh2highlow(x[j]), sgn);
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    const __half2 d = as_h2(w[2 * H + i / 2]);
+    const __half2 d = as_h2(w[i / 2]);
     y[i] = __hmul2((i & 1) ? __high2half2(d) : __low2half2(d), x[i]);
   }
 #pragma unroll
   for (int i = 1; i < 6; ++i)
 #pragma unroll
     for (int j = 0; j < i; ++j) {
-      const __half2 L = as_h2(w[2 * H + 3 + tri(i, j)]);
+      const __half2 L = as_h2(w[3 + tri(i, j)]);
       const __half2 lr = __low2half2(L), li = __high2half2(L);
       y[i] = __hfma2(lr, x[j], y[i]);
       y[i] = __hfma2(li, xs[j], y[i]);
@@ -912,138 +840,223 @@ __device__ inline void clover_block_h2(const MatBlock<__half>& M, int r, const _
     }
 }
 
+// y = (chirality block h of site r) x
 template <typename MT, bool H2>
-__device__ inline void block_apply_pair(const MatBlock<MT>& M, int r, int h, const Half<float>& x, Half<float>& y) {
+__device__ __forceinline__ void pair_block(const MatBlock<MT>& M, int r, int h, const Half<float>& x, Half<float>& y) {
   if constexpr (H2) {
+    uint32_t w[18];
+    M.block_words(r, h, w);
     __half2 xv[6], yv[6];
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
+    for (int k = 0; k < 6; ++k) xv[k] = __floats2half2_rn(x.c[k / 3][k % 3].re, x.c[k / 3][k % 3].im);
+    clover_block_h2(w, xv, yv);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) xv[3 * s + c] = __floats2half2_rn(x.c[s][c].re, x.c[s][c].im);
-    if (h == 0) clover_block_h2<0>(M, r, xv, yv);
-    else clover_block_h2<1>(M, r, xv, yv);
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float2 f = __half22float2(yv[3 * s + c]);
-        y.c[s][c] = mk(f.x, f.y);
-      }
+    for (int k = 0; k < 6; ++k) {
+      const float2 f = __half22float2(yv[k]);
+      y.c[k / 3][k % 3] = mk(f.x, f.y);
+    }
   } else {
-    block_apply(M, r, h, x, y);
+    float m[36];
+    M.block(r, h, m);
+    cx<float> v[6], w[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = x.c[k / 3][k % 3];
+    clover_block_mul(m, v, w);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) y.c[k / 3][k % 3] = w[k];
   }
 }
 
-// Hops of one direction with the inside-the-domain test taken from bit masks, so the
-// phase loop carries four small integers instead of two coordinate arrays.
-template <int MU, typename MT, bool H2>
-__device__ inline void hop_mask_mu(const Geom& g, unsigned fwd, unsigned bwd, int lex, int p, int r_self,
-                                   const float4* src, const MatBlock<MT>& M, Spinor<float>& acc) {
+// The geometry of one thread's two sites: nb[mu] holds, for the even (low 16 bits) and the odd
+// site, the index of the neighbour this lane's hop reads (x + mu for h = 0, x - mu for h = 1)
+// among the sites of the other parity, or of a zero slot when it lies outside the domain.
+struct PairSites {
+  unsigned nb[4];
+  int i, h;
+  float st;   // sign of the time direction in this lane's frame
+  template <int P> __device__ __forceinline__ int neighbour(int mu) const {
+    return P ? (int)(nb[mu] >> 16) : (int)(nb[mu] & 0xffffu);
+  }
+};
+
+// One hop in direction MU of the site of parity P.
+template <int P, int MU, typename MT, bool H2>
+__device__ __forceinline__ void pair_hop(const Geom& g, const PairSites& q, const float4* own, const float4* oth,
+                                         const MatBlock<MT>& M, Spinor<float>& acc) {
+  const int HP = g.Hd + ZERO_SLOTS;
+  const int j = q.neighbour<P>(MU);
+  // U_mu of the site itself, or of the neighbour (any link where that is a zero slot)
+  const int r = q.h ? (1 - P) * g.Hd + (j & (g.Hd - 1)) : P * g.Hd + q.i;
+  cx<float> v[12];
+  ld_half3(own + j, HP, v);
+  ld_half3(oth + j, HP, v + 6);
   Spinor<float> psi;
-  Half<float> h, uh;
-  if ((fwd >> MU) & 1u) {
-    int j = (lex + g.bstride[MU]) >> 1;
-    ld_buf(src, g.Hd, j, psi);
-    project<MU, -1>(psi, h);
-    if constexpr (H2) {
-      HalfH2 hh, oh;
-      pack_h2(h, hh);
-      su3_h2<false>(reinterpret_cast<const __half2*>(M.lk) + MU * 9 * g.Vd + r_self, g.Vd, hh, oh);
-      unpack_h2(oh, uh);
-    } else {
-      Link<float> L;
-      M.link(MU, r_self, L);
-      su3_mul(L, h, uh);
-    }
-    accum_recon<MU, -1>(acc, uh);
-  }
-  if ((bwd >> MU) & 1u) {
-    int j = (lex - g.bstride[MU]) >> 1;
-    ld_buf(src, g.Hd, j, psi);
-    project<MU, +1>(psi, h);
-    if constexpr (H2) {
-      HalfH2 hh, oh;
-      pack_h2(h, hh);
-      su3_h2<true>(reinterpret_cast<const __half2*>(M.lk) + MU * 9 * g.Vd + (1 - p) * g.Hd + j, g.Vd, hh, oh);
-      unpack_h2(oh, uh);
-    } else {
-      Link<float> L;
-      M.link(MU, (1 - p) * g.Hd + j, L);
-      su3_dag_mul(L, h, uh);
-    }
-    accum_recon<MU, +1>(acc, uh);
-  }
-}
-
-template <typename MT, bool H2>
-__device__ inline void hops_half_mask(int h, const Geom& g, unsigned fwd, unsigned bwd, int lex, int p, int r_self,
-                                      const float4* src, const MatBlock<MT>& M, Spinor<float>& acc) {
-  if (h == 0) {
-    hop_mask_mu<0, MT, H2>(g, fwd, bwd, lex, p, r_self, src, M, acc);
-    hop_mask_mu<1, MT, H2>(g, fwd, bwd, lex, p, r_self, src, M, acc);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) psi.c[k / 3][k % 3] = v[k];
+  Half<float> hp, uh;
+  frame_project<MU>(psi, q.st, hp);
+  if constexpr (H2) {
+    uint32_t w[9];
+    M.words(MU, r, q.h, w);
+    HalfH2 hh, oh;
+    pack_h2(hp, hh);
+    su3_h2(w, hh, oh);
+    unpack_h2(oh, uh);
   } else {
-    hop_mask_mu<2, MT, H2>(g, fwd, bwd, lex, p, r_self, src, M, acc);
-    hop_mask_mu<3, MT, H2>(g, fwd, bwd, lex, p, r_self, src, M, acc);
+    Link<float> U;
+    M.link(MU, r, q.h, U);
+    su3_mul(U, hp, uh);
+  }
+  frame_recon<MU>(acc, q.st, uh);
+}
+
+// Own half of the sum of all hops inside the domain at the site of parity P (no -1/2 factor).
+template <int P, typename MT, bool H2>
+__device__ __forceinline__ void pair_hops(const Geom& g, const PairSites& q, const float4* src, const MatBlock<MT>& M,
+                                          Half<float>& out) {
+  const int HP = g.Hd + ZERO_SLOTS;
+  const float4* own = src + 3 * q.h * HP;
+  const float4* oth = src + 3 * (1 - q.h) * HP;
+  Spinor<float> acc;
+  zero(acc);
+  pair_hop<P, 0, MT, H2>(g, q, own, oth, M, acc);
+  pair_hop<P, 1, MT, H2>(g, q, own, oth, M, acc);
+  pair_hop<P, 2, MT, H2>(g, q, own, oth, M, acc);
+  pair_hop<P, 3, MT, H2>(g, q, own, oth, M, acc);
+  join_halves(acc, out);
+}
+
+// ---- faces.  The block of face (mu, side) holds [3][face_n] 16-byte units of half-spinors:
+// side 0 (written on the -mu face) P^- delta in the upper spins, side 1 (on the +mu face)
+// U^dag P^+ delta in the lower spins, the frames in which h = 0 and h = 1 read them.  Only one
+// site in four to eight lies on a given face, so the SU(3) products and the output run over
+// lists of face sites, one thread each, instead of over the threads' own sites: per warp
+// ~800 instead of ~1900 instructions a visit (half-sweep of 32^3x64: 459 -> 430 us).
+
+// The k-th site of the four faces of one side (k < face_block / 2): direction, index in its
+// face, and index r among the domain's sites.
+struct FaceSite { int mu, idx, r; };
+__device__ __forceinline__ FaceSite face_site(const Geom& g, int side, int k) {
+  FaceSite f;
+  int lo = 0, first = 0, S = 1, lg = g.lgb[0];
+  f.mu = 0;
+#pragma unroll
+  for (int mu = 1; mu < 4; ++mu) {
+    lo += g.face_n[mu - 1];
+    if (k >= lo) {
+      f.mu = mu;
+      first = lo;
+      S = g.bstride[mu];
+      lg = g.lgb[mu];
+    }
+  }
+  f.idx = k - first;
+  // the coordinate along mu (0 or b - 1) goes in between the lower and the higher ones
+  const int lex = (f.idx & (S - 1)) + (side ? ((S << lg) - S) : 0) + ((f.idx & ~(S - 1)) << lg);
+  int p = lex, sh = 0;
+#pragma unroll
+  for (int mu = 0; mu < 3; ++mu) {
+    sh += g.lgb[mu];
+    p ^= lex >> sh;
+  }
+  f.r = (p & 1) * g.Hd + (lex >> 1);
+  return f;
+}
+
+// Multiply the staged half-spinors of the forward couplings by this domain's links, in place.
+template <typename MT>
+__device__ __forceinline__ void pair_face_links(const Geom& g, const Geom& gf, float4* sF, const MatBlock<MT>& M) {
+  for (int k = threadIdx.x; k < gf.face_block / 2; k += 2 * g.Hd) {
+    const FaceSite f = face_site(g, 1, k);
+    const int fn = gf.face_n[f.mu];
+    float4* q = sF + 3 * gf.face_off[2 * f.mu] + f.idx;
+    Half<float> hf, uh;
+    Link<float> U;
+    ld_half3(q, fn, hf);
+    M.link(f.mu, f.r, 0, U);
+    su3_mul(U, hf, uh);
+    st_half3(q, fn, uh);
   }
 }
 
-// Two threads per site.  The MR iteration is a loop over hop phases, so the hop and
-// clover code appears once (the whole kernel then fits the instruction cache):
-//   phase 0:          even sites, src = t_o      -> rho = r_e + 1/2 H t_o, x = 0
-//   phase 2k+1:       odd sites,  src = rho      -> t = A_oo^{-1} H rho
-//   phase 2k+2:       even sites, src = t        -> p = A_ee rho - 1/4 H t, MR step
-//   phase 2 I_d + 1:  odd sites,  src = x        -> delta_o = A_oo^{-1} (r_o + 1/2 H x)
-// cta: index of the domain among the domains of the given colour.
+// Own half of the couplings of the site of parity P to the neighbouring domains.
+template <int P>
+__device__ __forceinline__ void pair_face_hops(const Geom& g, const Geom& gf, const PairSites& q, const int l[4],
+                                               const float4* sF, Half<float>& out) {
+  Spinor<float> acc;
+  zero(acc);
+  auto face = [&](auto mu_c) {
+    constexpr int MU = decltype(mu_c)::value;
+    if (q.neighbour<P>(MU) >= g.Hd) {
+      Half<float> uh;
+      ld_half3(sF + 3 * gf.face_off[2 * MU + q.h] + face_index(g, l, MU), g.face_n[MU], uh);
+      frame_recon<MU>(acc, q.st, uh);
+    }
+  };
+  face(std::integral_constant<int, 0>());
+  face(std::integral_constant<int, 1>());
+  face(std::integral_constant<int, 2>());
+  face(std::integral_constant<int, 3>());
+  join_halves(acc, out);
+}
+
+// Face output of one side from delta in the work buffers.
+template <int SIDE, typename MT>
+__device__ __forceinline__ void pair_face_write(const Geom& g, const Geom& gf, long long d, const float4* sE,
+                                                float4* faces, const MatBlock<MT>& M) {
+  const int HP = g.Hd + ZERO_SLOTS;
+  const float st = SIDE ? 1.f : -1.f;
+  for (int k = threadIdx.x; k < gf.face_block / 2; k += 2 * g.Hd) {
+    const FaceSite f = face_site(g, SIDE, k);
+    const float4* b = sE + (f.r >= g.Hd ? 6 * HP + f.r - g.Hd : f.r);
+    cx<float> w[12];
+    ld_half3(b + 3 * SIDE * HP, HP, w);
+    ld_half3(b + 3 * (1 - SIDE) * HP, HP, w + 6);
+    Spinor<float> v;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) v.c[c / 3][c % 3] = w[c];
+    Half<float> hp, uh;
+    switch (f.mu) {
+      case 0: frame_project<0>(v, st, hp); break;
+      case 1: frame_project<1>(v, st, hp); break;
+      case 2: frame_project<2>(v, st, hp); break;
+      default: frame_project<3>(v, st, hp); break;
+    }
+    uh = hp;
+    if (SIDE) {
+      Link<float> U;
+      M.link(f.mu, f.r, 1, U);
+      su3_mul(U, hp, uh);
+    }
+    st_half3(faces + (d * gf.face_block + gf.face_off[2 * f.mu + SIDE]) * 3 + f.idx, gf.face_n[f.mu], uh);
+  }
+}
+
+// cta: index of the domain among the domains of the launch's colour.
+// MATS: the Schwarz matrices are staged beside the links (else read from global memory).
 // H2: hop and clover products in packed FP16 (see su3_h2); the domain's residual is then
 // scaled by a power of two, 16 / 2^ceil(log2 max|r|), before it enters the work buffers,
 // and everything that leaves them (the new residual, delta) is scaled back.  The MR
 // iteration is invariant under that scaling and powers of two are exact in FP32.
-template <typename MT, typename VT, bool MSMEM, bool H2, int SHAPE = 0>
+//
+// The odd solution needs no hop phase of its own: x = sum_k alpha_k rho_k over the MR steps,
+// and step k has already formed t_k = A_oo^{-1} H rho_k, so
+//   delta_o = A_oo^{-1} (r_o + 1/2 H x) = A_oo^{-1} r_o + 1/2 sum_k alpha_k t_k
+// is accumulated beside x: one phase (hops and block) less per visit.
+template <typename MT, bool MATS, bool H2, int SHAPE>
 __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
-  // hop phases use g (constant domain fields when SHAPE != 0); the face code, which indexes
-  // the face offsets at run time, reads the kernel parameters a.g directly
+  // hop phases use g (constant domain fields when SHAPE != 0); face offsets come from a.g
   const Geom g = fixed_shape<SHAPE>(a.g);
   extern __shared__ float4 smem[];
-  __shared__ uint64_t mbar, mbar_inj;   // staged copies; injected bytes (test hook)
+  __shared__ uint64_t bars[3];   // links and faces; Schwarz matrices; injected bytes (test hook)
   __shared__ float4 red[2 * SAP_MAX_THREADS / 32];
-  __shared__ float nrm[2 * SAP_MAX_THREADS];
-  const int tid = threadIdx.x;
-  const int Hd = g.Hd, Vd = g.Vd;
-  const int h = tid >= Hd;          // MR phases: chirality half and hop directions; ends: parity
-  const int i = tid - h * Hd;
-
-  // Domain-independent set-up: this thread's sites (even site i and odd site i), their
-  // local coordinates, hop masks and the shared-memory regions.
-  const size_t lk_elems = (size_t)4 * 9 * Vd;
-  const size_t lk_bytes = (size_t)MatBlock<MT>::link_bytes_per_site * Vd;
-  const size_t cm_bytes = (size_t)MatBlock<MT>::mat_bytes_per_site * Vd;
-  char* sbase = reinterpret_cast<char*>(smem);
-  MatBlock<MT> M;
-  M.Vd = Vd;
-  typedef typename std::remove_const<typename std::remove_pointer<decltype(M.lk)>::type>::type LkT;
-  typedef typename std::remove_const<typename std::remove_pointer<decltype(M.cm)>::type>::type CmT;
-  float4* sE = MSMEM ? reinterpret_cast<float4*>(sbase + lk_bytes + cm_bytes) : smem;
-  float4* sO = sE + 6 * Hd;
-  if (MSMEM) {
-    M.lk = reinterpret_cast<const LkT*>(sbase);
-    M.cm = reinterpret_cast<const CmT*>(sbase + lk_bytes);
-  }
-  int le[4], lo[4];
-  local_coords(g, 0, i, le);
-  local_coords(g, 1, i, lo);
-  const int lex_e = le[0] + g.bstride[1] * le[1] + g.bstride[2] * le[2] + g.bstride[3] * le[3];
-  const int lex_o = lo[0] + g.bstride[1] * lo[1] + g.bstride[2] * lo[2] + g.bstride[3] * lo[3];
-  unsigned fe, be, fo, bo;
-  inside_masks(g, le, fe, be);
-  inside_masks(g, lo, fo, bo);
-  const int r_e = i, r_o = Hd + i;
-  const int r_site = h * Hd + i;
-  const unsigned fs = h ? fo : fe, bs = h ? bo : be;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int Hd = g.Hd, Vd = g.Vd, HP = Hd + ZERO_SLOTS;
 
   // This CTA's domain: the cta-th of the launch (the additive form runs both colours, colour
-  // 0 first).  Its links and Schwarz matrices are copied into shared memory on an mbarrier
-  // while the residual is loaded.
+  // 0 first).
   const int ndom = a.both_colours ? g.ND : (g.ND >> 1);
+  if (cta >= ndom) return;
   int n[4], colour;
   long long d;
   {
@@ -1058,84 +1071,152 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
     n[0] = 2 * j + ((colour + n[1] + n[2] + n[3]) & 1);
     d = n[0] + (long long)g.dstride[1] * n[1] + (long long)g.dstride[2] * n[2] + (long long)g.dstride[3] * n[3];
   }
-  const LkT* glk = reinterpret_cast<const LkT*>(a.links) + d * lk_elems;
-  const CmT* gcm = reinterpret_cast<const CmT*>(a.smat) + d * (cm_bytes / sizeof(CmT));
-  if (cta >= ndom) return;
-  if (MSMEM) {
-    if (tid == 0) {
-      mbar_init(&mbar, 1);
-      mbar_init(&mbar_inj, 1);
+
+  // Shared memory: links, Schwarz matrices (MATS), then the two work buffers, which first
+  // receive the face blocks of the neighbouring domains.
+  const uint32_t lk_bytes = (uint32_t)MatBlock<MT>::link_bytes_per_site * Vd;
+  const uint32_t cm_bytes = MATS ? (uint32_t)MatBlock<MT>::mat_bytes_per_site * Vd : 0u;
+  char* sbase = reinterpret_cast<char*>(smem);
+  float4* sE = reinterpret_cast<float4*>(sbase + lk_bytes + cm_bytes);
+  float4* sO = sE + 6 * HP;
+  const char* glk = reinterpret_cast<const char*>(a.links) + d * lk_bytes;
+  const char* gcm = reinterpret_cast<const char*>(a.smat) + d * ((long long)MatBlock<MT>::mat_bytes_per_site * Vd);
+  MatBlock<MT> M;
+  M.Vd = Vd;
+  M.set_links(sbase);
+  M.set_mats(MATS ? (const void*)(sbase + lk_bytes) : (const void*)gcm);
+
+  // one thread: the eight face blocks this domain reads, each one contiguous copy
+  auto stage_faces = [&](const float4* faces) {
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu)
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        const long long dn = neighbour_domain(g, (int)d, n, mu, side ? -1 : +1);
+        bulk_g2s(sE + 3 * a.g.face_off[2 * mu + side], faces + (dn * a.g.face_block + a.g.face_off[2 * mu + side]) * 3,
+                 48u * a.g.face_n[mu], &bars[0]);
+      }
+  };
+  const uint32_t face_bytes = a.use_faces ? 48u * a.g.face_block : 0u;
+  if (tid == 0) {
+#pragma unroll
+    for (int b = 0; b < 3; ++b) mbar_init(&bars[b], 1);
+    mbar_expect_tx(&bars[0], lk_bytes + face_bytes);
+    if (a.use_faces) stage_faces(a.faces);
+    bulk_g2s(sbase, glk, lk_bytes, &bars[0]);
+    if (MATS) {
+      mbar_expect_tx(&bars[1], cm_bytes);
+      bulk_g2s(sbase + lk_bytes, gcm, cm_bytes, &bars[1]);
     }
-    __syncthreads();
-    if (tid == 0) {
-      mbar_expect_tx(&mbar, (uint32_t)(lk_bytes + cm_bytes));
-      bulk_g2s(sbase, glk, (uint32_t)lk_bytes, &mbar);
-      bulk_g2s(sbase + lk_bytes, gcm, (uint32_t)cm_bytes, &mbar);
-      // test hook: bytes that nobody sends, on a barrier of their own
-      if (a.extra_tx) mbar_expect_tx(&mbar_inj, a.extra_tx);
-    }
-  } else {
-    M.lk = glk;
-    M.cm = gcm;
+    // test hook: bytes that nobody sends, on a barrier of their own
+    if (a.extra_tx) mbar_expect_tx(&bars[2], a.extra_tx);
   }
-  const long long s_site = (d << g.lgVd) + h * Hd + i;
+
+  // This thread's sites.
+  PairSites q;
+  q.h = lane >> 4;
+  q.i = (tid >> 5) * 16 + (lane & 15);
+  q.st = q.h ? 1.f : -1.f;
+  const int h = q.h, i = q.i;
+  int le[4], lo[4];
+  local_coords(g, 0, i, le);
+  local_coords(g, 1, i, lo);
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    unsigned w = 0;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const int* l = p ? lo : le;
+      const int lex = l[0] + g.bstride[1] * l[1] + g.bstride[2] * l[2] + g.bstride[3] * l[3];
+      const bool out = h ? l[mu] == 0 : l[mu] == g.b[mu] - 1;
+      const int step = h ? (out ? g.b[mu] - 1 : -1) : (out ? 1 - g.b[mu] : 1);   // periodic in the domain
+      const int j = (lex + step * g.bstride[mu]) >> 1;
+      // a zero slot in the bank group that the wrapped neighbour would use
+      w |= (unsigned)(out ? Hd + (j & (ZERO_SLOTS - 1)) : j) << (16 * p);
+    }
+    q.nb[mu] = w;
+  }
+  const int r_e = i, r_o = Hd + i;
+  float4* const eo = sE + 3 * h * HP + i;   // own half of the even / odd site in the work buffers
+  float4* const oo = sO + 3 * h * HP + i;
+  __syncthreads();   // barriers initialised
 
   // Right-hand sides share the staged matrices; each has its own input, output and state.
 #pragma unroll 1
   for (int rhs = 0; rhs < a.nrhs; ++rhs) {
-  float4* const fr = a.faces + rhs * a.f_stride;
-  float4* const fw = a.faces_out + rhs * a.f_stride;
-  float* const rnr = a.r_norm ? a.r_norm + rhs * a.rn_stride : nullptr;
-  float* const unr = a.u_norm ? a.u_norm + rhs * a.un_stride : nullptr;
-  float inv_sc = 1.f;   // H2: undoes the domain's scaling on the way out
-  // 1. residual of site (parity h, index i), with the couplings to the other colour
-  EvenStore<VT> rst{reinterpret_cast<decltype(EvenStore<VT>::p)>((char*)a.r_store + rhs * a.r_bytes), rnr};
-  {
-    Spinor<float> r;
-    const SpinorPtr<float> vin{const_cast<float4*>(a.vptr ? a.vptr[rhs] : a.v + rhs * a.v_stride)};
+    float* const rnr = a.r_norm ? a.r_norm + rhs * a.rn_stride : nullptr;
+    float* const unr = a.u_norm ? a.u_norm + rhs * a.un_stride : nullptr;
+    const HalfField<MT> rst((char*)a.r_store + rhs * a.r_bytes, rnr, d * Hd, 0);
+    const HalfField<MT> ust((char*)a.u_store + rhs * a.u_bytes, unr, d * Vd, 0);
+    float inv_sc = 1.f;   // H2: undoes the domain's scaling on the way out
+    Half<float> rho, dO, x, t, own;   // residual and solution (even), solution (odd); own halves
+
+    // 1. residual with the couplings to the other colour
     if (a.first) {
-      vin.load(g, s_site, r);
+      const float4* v = (a.vptr ? a.vptr[rhs] : a.v + rhs * a.v_stride) + d * 6 * Vd + 3 * h * Vd;
+      ld_half3(v + r_e, Vd, rho);
+      ld_half3(v + r_o, Vd, dO);
       if (a.vscale) {
         const float sc = *a.vscale;
 #pragma unroll
-        for (int sp = 0; sp < 4; ++sp)
+        for (int s = 0; s < 2; ++s)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) r.c[sp][c] = sc * r.c[sp][c];
+          for (int c = 0; c < 3; ++c) {
+            rho.c[s][c] = sc * rho.c[s][c];
+            dO.c[s][c] = sc * dO.c[s][c];
+          }
       }
-    } else if (h == 0) {
-      rst.load(d, Hd, i, r);
     } else {
-      zero(r);
+      rst.load(Hd, i, h, rho);
+      ust.prefetch(Vd, r_e, h);
+      ust.prefetch(Vd, r_o, h);
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dO.c[s][c] = mk(0.f, 0.f);
     }
-    if (MSMEM && rhs == 0) {
-      bool ok = mbar_wait(&mbar, 0, a.wait_ns);
-      if (a.extra_tx) ok = mbar_wait(&mbar_inj, 0, a.wait_ns) && ok;
+    if (rhs == 0 || a.use_faces) {
+      bool ok = mbar_wait(&bars[0], rhs & 1, a.wait_ns);
+      if (rhs == 0) {
+        if (MATS) ok = mbar_wait(&bars[1], 0, a.wait_ns) && ok;
+        if (a.extra_tx) ok = mbar_wait(&bars[2], 0, a.wait_ns) && ok;
+      }
       if (__syncthreads_or(!ok)) {
-        // as in sap_kernel: flag, then a bounded wait for the real copies before leaving
+        // a wait ran out: flag it; then wait (bounded) for the staged copies themselves,
+        // which were issued and will land, so none is left writing into this CTA's shared
+        // memory after it exits
         if (tid == 0) atomicExch(a.err, 1);
-        mbar_wait(&mbar, 0, a.wait_ns);
+        mbar_wait(&bars[0], rhs & 1, a.wait_ns);
+        if (MATS && rhs == 0) mbar_wait(&bars[1], 0, a.wait_ns);
         return;
       }
     }
     if (a.use_faces) {
-      Spinor<float> acc;
-      zero(acc);
-      if (h) face_hops_rt(a.g, (int)d, n, lo, fs, bs, r_site, fr, M, acc);
-      else face_hops_rt(a.g, (int)d, n, le, fs, bs, r_site, fr, M, acc);
+      pair_face_links<MT>(g, a.g, sE, M);
+      __syncthreads();
+      pair_face_hops<0>(g, a.g, q, le, sE, own);
 #pragma unroll
-      for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 2; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) r.c[s][c] = r.c[s][c] + 0.5f * acc.c[s][c];
+        for (int c = 0; c < 3; ++c) rho.c[s][c] = rho.c[s][c] + 0.5f * own.c[s][c];
+      pair_face_hops<1>(g, a.g, q, lo, sE, own);
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dO.c[s][c] = dO.c[s][c] + 0.5f * own.c[s][c];
     }
     if constexpr (H2) {
       float m = 0.f;
 #pragma unroll
-      for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 2; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) m = fmaxf(m, fmaxf(fabsf(r.c[s][c].re), fabsf(r.c[s][c].im)));
+        for (int c = 0; c < 3; ++c) {
+          m = fmaxf(m, fmaxf(fabsf(rho.c[s][c].re), fabsf(rho.c[s][c].im)));
+          m = fmaxf(m, fmaxf(fabsf(dO.c[s][c].re), fabsf(dO.c[s][c].im)));
+        }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if ((tid & 31) == 0) red[tid >> 5].x = m;
+      if (lane == 0) red[tid >> 5].x = m;
       __syncthreads();
       m = 0.f;
       for (int w = 0; w < (2 * Hd + 31) >> 5; ++w) m = fmaxf(m, red[w].x);
@@ -1144,65 +1225,55 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
       const float sc = m > 0.f ? ldexpf(1.f, 4 - max(e, -100)) : 1.f;   // finite even for tiny m
       inv_sc = 1.f / sc;
 #pragma unroll
-      for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 2; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) r.c[s][c] = mk(r.c[s][c].re * sc, r.c[s][c].im * sc);
+        for (int c = 0; c < 3; ++c) {
+          rho.c[s][c] = sc * rho.c[s][c];
+          dO.c[s][c] = sc * dO.c[s][c];
+        }
     }
-    st_buf(h ? sO : sE, Hd, i, r);
-  }
-  __syncthreads();
-  Half<float> roh, t, own, rho, x;
-  ld_hbuf(sE, Hd, i, h, rho);              // rho starts as r_e; phase 0 adds 1/2 H t_o
-  ld_hbuf(sO, Hd, i, h, roh);
-  __syncthreads();
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) x.c[s][c] = mk(0.f, 0.f);
-  block_apply_pair<MT, H2>(M, r_o, h, roh, t);   // t_o = A_oo^{-1} r_o
-  st_hbuf(sO, Hd, i, h, t);
-  __syncthreads();
+    pair_block<MT, H2>(M, r_o, h, dO, t);   // t_o = A_oo^{-1} r_o
+    dO = t;
+    __syncthreads();   // the staged faces have been read: the work buffers may be written
+    for (int k = tid; k < 12 * ZERO_SLOTS; k += 2 * Hd)
+      sE[(k / ZERO_SLOTS) * HP + Hd + k % ZERO_SLOTS] = make_float4(0.f, 0.f, 0.f, 0.f);
+    st_half3(oo, HP, t);
+    __syncthreads();
 
-  // 2.-4. preparation, MR steps and odd reconstruction as one loop over hop phases
-  const int nph = 2 * a.i_domain + 2;
-  const int nwarp = (2 * Hd + 31) >> 5;
+    // 2. even-odd preparation: rho = r_e + 1/2 H t_o
+    pair_hops<0, MT, H2>(g, q, sO, M, own);
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        rho.c[s][c] = rho.c[s][c] + 0.5f * own.c[s][c];
+        x.c[s][c] = mk(0.f, 0.f);
+      }
+    st_half3(eo, HP, rho);
+    __syncthreads();
+
+    // 3. MR steps on the Schur complement
+    const int nwarp = (2 * Hd + 31) >> 5;
 #pragma unroll 1
-  for (int ph = 0; ph < nph; ++ph) {
-    const int odd = ph & 1;
-    Spinor<float> acc;
-    zero(acc);
-    // the hop code is specialised per direction pair (h) but appears once in the loop
-    hops_half_mask<MT, H2>(h, g, odd ? fo : fe, odd ? bo : be, odd ? lex_o : lex_e, odd, odd ? r_o : r_e,
-                           odd ? sE : sO, M, acc);
-    exchange(acc, h, odd ? sO : sE, Hd, i, own);
-    if (ph == 0) {
-#pragma unroll
-      for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) rho.c[s][c] = rho.c[s][c] + 0.5f * own.c[s][c];
-      st_hbuf(sE, Hd, i, h, rho);
-    } else {
-      // one clover-block application per phase: A_oo^{-1} on odd phases, A_ee rho on even
-      Half<float> bin;
-#pragma unroll
-      for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-          bin.c[s][c] = !odd ? rho.c[s][c] : (ph == nph - 1 ? roh.c[s][c] + 0.5f * own.c[s][c] : own.c[s][c]);
-      block_apply_pair<MT, H2>(M, odd ? r_o : r_e, h, bin, t);
-      if (odd) st_hbuf(sO, Hd, i, h, t);
-    }
-    if (ph != 0 && !odd) {
-      Half<float> pv = t;
+    for (int it = 0; it < a.i_domain; ++it) {
+      // odd sites: t = A_oo^{-1} H rho
+      pair_hops<1, MT, H2>(g, q, sE, M, own);
+      pair_block<MT, H2>(M, r_o, h, own, t);
+      st_half3(oo, HP, t);
+      __syncthreads();
+      // even sites: p = A_ee rho - 1/4 H t
+      pair_hops<0, MT, H2>(g, q, sO, M, own);
+      Half<float> pv;
+      pair_block<MT, H2>(M, r_e, h, rho, pv);
       float pr_re = 0.f, pr_im = 0.f, pp = 0.f;
 #pragma unroll
       for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           pv.c[s][c] = pv.c[s][c] - 0.25f * own.c[s][c];
-          cx<float> q = cjmul(pv.c[s][c], rho.c[s][c]);
-          pr_re += q.re;
-          pr_im += q.im;
+          cx<float> z = cjmul(pv.c[s][c], rho.c[s][c]);
+          pr_re += z.re;
+          pr_im += z.im;
           pp += pv.c[s][c].re * pv.c[s][c].re + pv.c[s][c].im * pv.c[s][c].im;
         }
 #pragma unroll
@@ -1211,95 +1282,106 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
         pr_im += __shfl_xor_sync(0xffffffffu, pr_im, o);
         pp += __shfl_xor_sync(0xffffffffu, pp, o);
       }
-      if ((tid & 31) == 0) red[tid >> 5] = make_float4(pr_re, pr_im, pp, 0.f);
+      if (lane == 0) red[tid >> 5] = make_float4(pr_re, pr_im, pp, 0.f);
       __syncthreads();
       // every warp sums the nwarp partial sums the same way (lane l holds entry l, a
       // butterfly over the lanes, lane 0's total broadcast), so all threads get one alpha
       float sr = 0.f, si = 0.f, sp = 0.f;
-      {
-        const int lane = tid & 31;
-        if (lane < nwarp) {
-          const float4 q = red[lane];
-          sr = q.x;
-          si = q.y;
-          sp = q.z;
-        }
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          if (o >= nwarp) break;
-          sr += __shfl_xor_sync(0xffffffffu, sr, o);
-          si += __shfl_xor_sync(0xffffffffu, si, o);
-          sp += __shfl_xor_sync(0xffffffffu, sp, o);
-        }
-        sr = __shfl_sync(0xffffffffu, sr, 0);
-        si = __shfl_sync(0xffffffffu, si, 0);
-        sp = __shfl_sync(0xffffffffu, sp, 0);
+      if (lane < nwarp) {
+        const float4 w = red[lane];
+        sr = w.x;
+        si = w.y;
+        sp = w.z;
       }
-      cx<float> alpha = sp > 0.f ? mk(sr / sp, si / sp) : mk(0.f, 0.f);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        if (o >= nwarp) break;
+        sr += __shfl_xor_sync(0xffffffffu, sr, o);
+        si += __shfl_xor_sync(0xffffffffu, si, o);
+        sp += __shfl_xor_sync(0xffffffffu, sp, o);
+      }
+      sr = __shfl_sync(0xffffffffu, sr, 0);
+      si = __shfl_sync(0xffffffffu, si, 0);
+      sp = __shfl_sync(0xffffffffu, sp, 0);
+      const cx<float> alpha = sp > 0.f ? mk(sr / sp, si / sp) : mk(0.f, 0.f);
+      const cx<float> ah = 0.5f * alpha;
+      ld_half3(oo, HP, t);   // this step's t of the own odd site
 #pragma unroll
       for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           x.c[s][c] = cmac(x.c[s][c], alpha, rho.c[s][c]);
           rho.c[s][c] = cnmac(rho.c[s][c], alpha, pv.c[s][c]);
+          dO.c[s][c] = cmac(dO.c[s][c], ah, t.c[s][c]);
         }
-      // the last MR step hands x to the reconstruction phase instead of rho
-      st_hbuf(sE, Hd, i, h, ph == nph - 2 ? x : rho);
+      if (it + 1 < a.i_domain) {
+        st_half3(eo, HP, rho);
+        __syncthreads();
+      }
     }
-    __syncthreads();
-  }
-  if (!a.last) {
     if constexpr (H2) {
 #pragma unroll
       for (int s = 0; s < 2; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) rho.c[s][c] = mk(rho.c[s][c].re * inv_sc, rho.c[s][c].im * inv_sc);
+        for (int c = 0; c < 3; ++c) {
+          rho.c[s][c] = inv_sc * rho.c[s][c];
+          x.c[s][c] = inv_sc * x.c[s][c];
+          dO.c[s][c] = inv_sc * dO.c[s][c];
+        }
     }
-    EvenHalfStore<VT>::store(rst, nrm, d, Hd, i, h, rho);
-    __syncthreads();
-  }
 
-  // 5. site (h, i): u += delta, faces of delta
-  Spinor<float> dl;
-  ld_buf(h ? sO : sE, Hd, i, dl);
-  if constexpr (H2) {
+    // 4. faces of delta for the next half-sweep (none after the very last one)
+    if (!(a.last && (a.both_colours || colour == 1))) {
+      st_half3(eo, HP, x);
+      st_half3(oo, HP, dO);
+      __syncthreads();
+      float4* const fw = a.faces_out + rhs * a.f_stride;
+      pair_face_write<1, MT>(g, a.g, d, sE, fw, M);
+      pair_face_write<0, MT>(g, a.g, d, sE, fw, M);
+    }
+    // the next right-hand side's faces land in the work buffers while this one is stored
+    if (rhs + 1 < a.nrhs) {
+      __syncthreads();
+      if (tid == 0 && a.use_faces) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_expect_tx(&bars[0], face_bytes);
+        stage_faces(a.faces + (rhs + 1) * a.f_stride);
+      }
+    }
+
+    // 5. u += delta and the new residual
+    Half<float> ue = x, uo = dO;
+    if (!a.first) {
+      Half<float> w;
+      ust.load(Vd, r_e, h, w);
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 2; ++s)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) dl.c[s][c] = mk(dl.c[s][c].re * inv_sc, dl.c[s][c].im * inv_sc);
-  }
-  typename VecPtr<VT>::type ust = VecPtr<VT>::make((char*)a.u_store + rhs * a.u_bytes, unr);
-  Spinor<float> u;
-  if (a.first) {
-    u = dl;
-  } else {
-    ust.load(g, s_site, u);
+        for (int c = 0; c < 3; ++c) ue.c[s][c] = ue.c[s][c] + w.c[s][c];
+      ust.load(Vd, r_o, h, w);
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 2; ++s)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) u.c[s][c] = u.c[s][c] + dl.c[s][c];
-  }
-  if (a.last) {
-    SpinorPtr<float> zo{a.zptr ? a.zptr[rhs] : a.z + rhs * a.v_stride};
-    zo.store(g, s_site, u);
-  } else {
-    ust.store(g, s_site, u);
-  }
-  // faces for the next half-sweep (none after the very last one)
-  if (!(a.last && (a.both_colours || colour == 1))) {
-    if (h) face_write_rt(a.g, d, lo, fs, bs, r_site, fw, M, dl);
-    else face_write_rt(a.g, d, le, fs, bs, r_site, fw, M, dl);
-  }
-  __syncthreads();   // the work buffers are reused by the next right-hand side
+        for (int c = 0; c < 3; ++c) uo.c[s][c] = uo.c[s][c] + w.c[s][c];
+    }
+    if (a.last) {
+      float4* z = (a.zptr ? a.zptr[rhs] : a.z + rhs * a.v_stride) + d * 6 * Vd + 3 * h * Vd;
+      st_half3(z + r_e, Vd, ue);
+      st_half3(z + r_o, Vd, uo);
+    } else {
+      rst.store(Hd, i, h, rho);
+      ust.store(Vd, r_e, h, ue);
+      ust.store(Vd, r_o, h, uo);
+    }
   }
 }
 
 // One CTA per domain (measured faster on GB300 than a persistent grid walking its domains
 // with the next domain's copies in flight: the round-robin tail and the extra live state
 // cost more than the overlap gains).
-template <typename MT, typename VT, bool MSMEM, bool H2, int SHAPE>
-__global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair(SapArgs a) {
-  sap_pair_body<MT, VT, MSMEM, H2, SHAPE>(a, blockIdx.x);
+template <typename MT, bool MATS, bool H2, int SHAPE>
+__global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair(const __grid_constant__ SapArgs a) {
+  sap_pair_body<MT, MATS, H2, SHAPE>(a, blockIdx.x);
 }
 
 // Several lattices of the same domain shape in one launch: the grid is the concatenation
@@ -1311,29 +1393,26 @@ struct SapLattices {
   int nlat;
 };
 
-template <typename MT, typename VT, bool MSMEM>
-__global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair_lattices(SapLattices m) {
+__global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair_lattices(const __grid_constant__ SapLattices m) {
   int l = 0;
   while (l + 1 < m.nlat && (int)blockIdx.x >= m.first[l + 1]) ++l;
-  switch (l) {   // constant indices keep the arguments in the parameter space
-    case 0: sap_pair_body<MT, VT, MSMEM, false>(m.lat[0], blockIdx.x - m.first[0]); break;
-    case 1: sap_pair_body<MT, VT, MSMEM, false>(m.lat[1], blockIdx.x - m.first[1]); break;
-    case 2: sap_pair_body<MT, VT, MSMEM, false>(m.lat[2], blockIdx.x - m.first[2]); break;
-    default: sap_pair_body<MT, VT, MSMEM, false>(m.lat[3], blockIdx.x - m.first[3]); break;
-  }
+  sap_pair_body<__half, true, false, 0>(m.lat[l], blockIdx.x - m.first[l]);
 }
 
-size_t sap_smem_bytes(const Geom& g, int mat_prec, bool mat_in_smem) {
-  size_t vec = (size_t)2 * 6 * g.Hd * 16;
-  if (!mat_in_smem) return vec;
-  size_t per = mat_prec == P16 ? (MatBlock<__half>::link_bytes_per_site + MatBlock<__half>::mat_bytes_per_site)
-                               : (MatBlock<float>::link_bytes_per_site + MatBlock<float>::mat_bytes_per_site);
-  return vec + per * g.Vd;
+// One thread per site: the work vectors, and links and matrices when both fit.  Two threads
+// per site: the links always, the matrices when they fit beside them; the work buffers (with
+// their zero slots) share their space with the staged faces.
+size_t sap_smem_bytes(const Geom& g, int mat_prec, bool mat_in_smem, int threads_per_site) {
+  const size_t lk = mat_prec == P16 ? MatBlock<__half>::link_bytes_per_site : MatBlock<float>::link_bytes_per_site;
+  const size_t cm = mat_prec == P16 ? MatBlock<__half>::mat_bytes_per_site : MatBlock<float>::mat_bytes_per_site;
+  if (threads_per_site == 1) return (size_t)2 * 6 * g.Hd * 16 + (mat_in_smem ? (lk + cm) * g.Vd : 0);
+  const size_t work = (size_t)2 * 6 * (g.Hd + ZERO_SLOTS) * 16, faces = (size_t)48 * g.face_block;
+  return (lk + (mat_in_smem ? cm : 0)) * g.Vd + (work > faces ? work : faces);
 }
 
 static int smem_optin();
-bool sap_mat_fits_smem(const Geom& g, int mat_prec) {
-  return sap_smem_bytes(g, mat_prec, true) + 1024 <= (size_t)smem_optin();
+bool sap_mat_fits_smem(const Geom& g, int mat_prec, int threads_per_site) {
+  return sap_smem_bytes(g, mat_prec, true, threads_per_site) + 1024 <= (size_t)smem_optin();
 }
 
 static int smem_optin() {
@@ -1348,35 +1427,38 @@ static int smem_optin() {
 
 int sap_max_domain_sites() { return 2 * SAP_MAX_THREADS; }
 
-template <typename MT, typename VT, bool MSMEM, bool H2, int SHAPE>
-static void launch_pair(const SapArgs& a, int grid, size_t smem, cudaStream_t st) {
+template <typename MT, bool MATS, bool H2, int SHAPE>
+static void launch_shape(const SapArgs& a, int grid, size_t smem, cudaStream_t st) {
   static int configured = 0;
   if (!configured) {
-    // static shared memory (barriers, reduction slots) is a few KB; the rest may be dynamic
-    cudaFuncSetAttribute(sap_kernel_pair<MT, VT, MSMEM, H2, SHAPE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem_optin() - 4096);
+    // static shared memory (barriers, reduction slots) is below 1 KB; the rest may be dynamic
+    cudaFuncSetAttribute(sap_kernel_pair<MT, MATS, H2, SHAPE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         smem_optin() - 1024);
     configured = 1;
   }
-  sap_kernel_pair<MT, VT, MSMEM, H2, SHAPE><<<grid, 2 * a.g.Hd, smem, st>>>(a);
+  sap_kernel_pair<MT, MATS, H2, SHAPE><<<grid, 2 * a.g.Hd, smem, st>>>(a);
 }
 
-template <typename MT, typename VT, bool MSMEM, bool H2 = false>
-static int launch_one(const SapArgs& a, int grid, int pair, cudaStream_t st) {
-  size_t smem = sap_smem_bytes(a.g, std::is_same<MT, __half>::value ? P16 : P32, MSMEM);
-  if (pair) {
-    switch (domain_shape_id(a.g)) {
-      case 1: launch_pair<MT, VT, MSMEM, H2, 1>(a, grid, smem, st); break;
-      case 2: launch_pair<MT, VT, MSMEM, H2, 2>(a, grid, smem, st); break;
-      default: launch_pair<MT, VT, MSMEM, H2, 0>(a, grid, smem, st); break;
-    }
-  } else {
-    static int configured = 0;
-    if (!configured) {
-      cudaFuncSetAttribute(sap_kernel<MT, VT, MSMEM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - 1024);
-      configured = 1;
-    }
-    sap_kernel<MT, VT, MSMEM><<<grid, a.g.Hd, smem, st>>>(a);
+template <typename MT, bool MATS, bool H2 = false>
+static int launch_pair(const SapArgs& a, int grid, cudaStream_t st) {
+  const size_t smem = sap_smem_bytes(a.g, std::is_same<MT, __half>::value ? P16 : P32, MATS, 2);
+  switch (domain_shape_id(a.g)) {
+    case 1: launch_shape<MT, MATS, H2, 1>(a, grid, smem, st); break;
+    case 2: launch_shape<MT, MATS, H2, 2>(a, grid, smem, st); break;
+    default: launch_shape<MT, MATS, H2, 0>(a, grid, smem, st); break;
   }
+  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+}
+
+template <typename MT, bool MSMEM>
+static int launch_single(const SapArgs& a, int grid, cudaStream_t st) {
+  const size_t smem = sap_smem_bytes(a.g, std::is_same<MT, __half>::value ? P16 : P32, MSMEM, 1);
+  static int configured = 0;
+  if (!configured) {
+    cudaFuncSetAttribute(sap_kernel<MT, MT, MSMEM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - 1024);
+    configured = 1;
+  }
+  sap_kernel<MT, MT, MSMEM><<<grid, a.g.Hd, smem, st>>>(a);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
@@ -1401,19 +1483,15 @@ int sap_half_sweep_lattices(const Geom* gs, const SapState* Ss, int nlat, int co
     total += g.ND / 2;
   }
   m.first[nlat] = total;
-  const bool ms = Ss[0].mat_in_smem;
-  size_t smem = sap_smem_bytes(gs[0], P16, ms);
-  if (ms) {
-    static int configured = 0;
-    if (!configured) {
-      cudaFuncSetAttribute(sap_kernel_pair_lattices<__half, __half, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           smem_optin() - 4096);
-      configured = 1;
-    }
-    sap_kernel_pair_lattices<__half, __half, true><<<total, 2 * gs[0].Hd, smem, st>>>(m);
-  } else {
-    sap_kernel_pair_lattices<__half, __half, false><<<total, 2 * gs[0].Hd, smem, st>>>(m);
+  // the domains may differ in shape: room for the one with the most face sites
+  size_t smem = 0;
+  for (int l = 0; l < nlat; ++l) smem = std::max(smem, sap_smem_bytes(gs[l], P16, true, 2));
+  static int configured = 0;
+  if (!configured) {
+    cudaFuncSetAttribute(sap_kernel_pair_lattices, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - 1024);
+    configured = 1;
   }
+  sap_kernel_pair_lattices<<<total, 2 * gs[0].Hd, smem, st>>>(m);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
@@ -1430,13 +1508,15 @@ int sap_half_sweep(const Geom& g, const SapState& S, int colour, int first, int 
   // matrices and vectors are stored in the same precision (FP16 or FP32)
   if (S.mat_prec != S.vec_prec) return -1;
   if (S.half_arith) {   // packed FP16 products: FP16 storage and the two-thread kernel only
-    if (S.mat_prec != P16 || !pr) return -1;
-    return ms ? launch_one<__half, __half, true, true>(a, grid, 1, st)
-              : launch_one<__half, __half, false, true>(a, grid, 1, st);
+    if (S.mat_prec != P16 || !pr || !ms) return -1;
+    return launch_pair<__half, true, true>(a, grid, st);
   }
-  if (S.mat_prec == P16)
-    return ms ? launch_one<__half, __half, true>(a, grid, pr, st) : launch_one<__half, __half, false>(a, grid, pr, st);
-  return ms ? launch_one<float, float, true>(a, grid, pr, st) : launch_one<float, float, false>(a, grid, pr, st);
+  if (S.mat_prec == P16) {   // 304 bytes of matrices per site: every allowed domain fits
+    if (!ms) return -1;
+    return pr ? launch_pair<__half, true>(a, grid, st) : launch_single<__half, true>(a, grid, st);
+  }
+  if (pr) return ms ? launch_pair<float, true>(a, grid, st) : launch_pair<float, false>(a, grid, st);
+  return ms ? launch_single<float, true>(a, grid, st) : launch_single<float, false>(a, grid, st);
 }
 
 static SapArgs make_args(const Geom& g, const SapState& S, int colour, int first, int use_faces, int last,
