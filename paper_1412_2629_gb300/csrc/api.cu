@@ -70,6 +70,7 @@ struct SolverBuffers {
   double* h_status = nullptr;          // pinned host mirror
   LsqState* lsq = nullptr;
   int* flag = nullptr;                 // Gram-Schmidt: 1 when a second projection is needed
+  int* ticket = nullptr;               // Gram-Schmidt: last-block ticket, zero between launches
   double* nu2 = nullptr;               // squared norm of the projected vector
   // 1 / |v_i| of the basis vectors as stored: the single-right-hand-side solver leaves each
   // new vector unnormalised (its exact norm comes out of the projection pass) and its
@@ -617,19 +618,6 @@ __global__ void fill_ones_kernel(float* v, int n) {
 // vscale[0] = 1 / sqrt(nu2): the scale of a vector stored unnormalised
 __global__ void set_vscale_kernel(float* vscale, const double* nu2) { vscale[0] = (float)(1.0 / sqrt(*nu2)); }
 
-// After the first projection: |w - V h|^2 is known exactly; ask for a second projection
-// when it is below half of |w|^2.
-__global__ void gs_decide_kernel(const zd* hA, int nv, const double2* nrm_a, zd* hB, int* flag, double* nu2) {
-  double ww = hA[nv].re, v = nrm_a->x;
-  for (int i = 0; i <= nv; ++i) hB[i] = Z(0.0);
-  *nu2 = v;
-  *flag = v < 0.5 * ww ? 1 : 0;
-}
-
-__global__ void gs_decide2_kernel(const int* flag, const double2* nrm_b, double* nu2) {
-  if (*flag) *nu2 = nrm_b->x;
-}
-
 __global__ void arnoldi_finish_kernel(zd* H, zd* R, int ldh, int j, const zd* hA, const zd* hB, const double* nu2,
                                       LsqState* lsq, zd* g, double* status) {
   zd* col = H + (long)j * ldh;
@@ -745,7 +733,7 @@ static void free_solver_buffers(dd_ctx* c, SolverBuffers& s) {
                   (void*)s.f64, (void*)s.r64, (void*)s.canon64, (void*)s.H, (void*)s.R, (void*)s.P, (void*)s.Hn,
                   (void*)s.g, (void*)s.c0, (void*)s.y, (void*)s.hA, (void*)s.hB, (void*)s.cn, (void*)s.theta,
                   (void*)s.cp, (void*)s.partial, (void*)s.partial2, (void*)s.nrm2, (void*)s.status, (void*)s.lsq,
-                  (void*)s.flag, (void*)s.nu2, (void*)s.dW, (void*)s.dflags, (void*)s.vscale, (void*)s.V16,
+                  (void*)s.flag, (void*)s.ticket, (void*)s.nu2, (void*)s.dW, (void*)s.dflags, (void*)s.vscale, (void*)s.V16,
                   (void*)s.vin, (void*)s.one})
     release(c, p);
   if (s.h_status) cudaFreeHost(s.h_status);
@@ -769,9 +757,11 @@ static void release_solver(dd_ctx* c) {
   c->lock_cap = 0;
 }
 
-// Krylov basis, FP64 fields and small dense buffers for basis size m; streams and events
-// only for the context's own solver (the lockstep right-hand sides run on its stream).
-static dd_status alloc_solver_buffers(dd_ctx* c, SolverBuffers& s, int m, bool streams, bool v16 = false) {
+// Krylov basis, FP64 fields and small dense buffers for basis size m.  The side stream runs the
+// restart's small dense step beside the reliable update (1.0 ms of one warp beside 1.4 ms
+// of FP64 operator on 24^3x48); a main stream only for the context's own solver (the
+// lockstep right-hand sides run on the context's).
+static dd_status alloc_solver_buffers(dd_ctx* c, SolverBuffers& s, int m, bool own_stream, bool v16 = false) {
   const Geom& g = c->g;
   long long n4 = g.V * 6;
   size_t vb = (size_t)n4 * 16;
@@ -807,6 +797,8 @@ static dd_status alloc_solver_buffers(dd_ctx* c, SolverBuffers& s, int m, bool s
   TRY(dalloc(c, &s.status, 16 * sizeof(double)));
   TRY(dalloc(c, &s.lsq, sizeof(LsqState)));
   TRY(dalloc(c, &s.flag, 16));
+  TRY(dalloc(c, &s.ticket, 16));
+  TRY(cuda_check(c, cudaMemsetAsync(s.ticket, 0, 16, c->st), "ticket"));
   TRY(dalloc(c, &s.nu2, 16));
   TRY(dalloc(c, &s.dW, deflate_bytes(m)));
   TRY(dalloc(c, &s.vscale, (m + 2) * sizeof(float)));
@@ -814,11 +806,11 @@ static dd_status alloc_solver_buffers(dd_ctx* c, SolverBuffers& s, int m, bool s
   TRY(launched(c));
   TRY(dalloc(c, &s.dflags, 16 * sizeof(int)));
   if (cudaMallocHost(&s.h_status, 8 * sizeof(double)) != cudaSuccess) return fail(c, DD_ERR_OOM, "pinned status");
-  if (streams && (cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking) != cudaSuccess ||
-                  cudaStreamCreateWithFlags(&s.side, cudaStreamNonBlocking) != cudaSuccess ||
-                  cudaEventCreateWithFlags(&s.ev_in, cudaEventDisableTiming) != cudaSuccess ||
-                  cudaEventCreateWithFlags(&s.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-                  cudaEventCreateWithFlags(&s.ev_join, cudaEventDisableTiming) != cudaSuccess))
+  if ((own_stream && cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking) != cudaSuccess) ||
+      cudaStreamCreateWithFlags(&s.side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s.ev_in, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s.ev_join, cudaEventDisableTiming) != cudaSuccess)
     return fail(c, DD_ERR_CUDA, "solver stream");
   s.m = m;
   return DD_OK;
@@ -879,6 +871,19 @@ static dd_status read_status(dd_ctx* c, int n = 4) {
   return cuda_check(c, cudaStreamSynchronize(c->st), "solver step");
 }
 
+// What a Gram-Schmidt projection's last block does: stage 1 after the first pass, 2 after the
+// second.
+static GsTail gs_tail_of(const SolverBuffers& s, int stage) {
+  GsTail t;
+  t.stage = stage;
+  t.ticket = s.ticket;
+  t.hA = s.hA;
+  t.hB = s.hB;
+  t.flag = s.flag;
+  t.nu2 = s.nu2;
+  return t;
+}
+
 // rho2 = |f - A x|^2 into s.nrm2 (device) and return it on the host (s: the context's own
 // solver buffers unless given).
 static dd_status true_residual(dd_ctx* c, double* rho2, SolverBuffers* sp = nullptr) {
@@ -896,7 +901,7 @@ static dd_status true_residual(dd_ctx* c, double* rho2, SolverBuffers* sp = null
 
 // End of a cycle after mm Arnoldi steps, on the device: y from the least-squares problem;
 // the deflated restart's small dense step (one warp, on the second stream beside the
-// reliable update when `side` is set); x64 += Z y; r64 = f - A64 x64 and |r64|^2; then,
+// reliable update); x64 += Z y; r64 = f - A64 x64 and |r64|^2; then,
 // when the deflation succeeded and |r64| is still above target, V <- V P_{k+1} and
 // Z <- Z P_k in place and the projection of r64 onto the new V_{k+1}.  The one host read
 // returns |r64|^2 and whether the deflated restart keeps enough of r64.
@@ -906,24 +911,19 @@ struct CycleEnd {
   int defl_rc = -1;
 };
 
-static dd_status end_cycle(dd_ctx* c, SolverBuffers& s, int mm, const dd_solve_params* p, double nf, bool side,
-                           CycleEnd* out) {
+static dd_status end_cycle(dd_ctx* c, SolverBuffers& s, int mm, const dd_solve_params* p, double nf, CycleEnd* out) {
   const long long n4 = c->g.V * 6;
   const int m = p->m, k = p->k, ldh = m + 1;
   const double defl_tol = 1e-2;
   const int want = k > 0 && mm > k;
   lsq_solve_kernel<<<1, 1, 0, c->st>>>(s.R, ldh, mm, s.g, s.y);
   int nk = 1;
-  cudaStream_t ds = c->st;
   if (want) {
-    if (side && s.side) {
-      cudaEventRecord(s.ev_fork, c->st);
-      cudaStreamWaitEvent(s.side, s.ev_fork, 0);
-      ds = s.side;
-    }
-    launch_deflate(s.H, ldh, mm, k, s.c0, s.y, s.P, s.Hn, s.cn, s.theta, s.dW, s.dflags, ds);
+    cudaEventRecord(s.ev_fork, c->st);
+    cudaStreamWaitEvent(s.side, s.ev_fork, 0);
+    launch_deflate(s.H, ldh, mm, k, s.c0, s.y, s.P, s.Hn, s.cn, s.theta, s.dW, s.dflags, s.side);
     nk++;
-    if (ds != c->st) cudaEventRecord(s.ev_join, ds);
+    cudaEventRecord(s.ev_join, s.side);
   }
   launch_x_update(s.x64, s.Z, mm, n4, (const double2*)s.y, c->st);
   nk++;
@@ -932,7 +932,7 @@ static dd_status end_cycle(dd_ctx* c, SolverBuffers& s, int mm, const dd_solve_p
   launch_norm2_64(s.r64, c->g.V * 12, s.partial, c->st);
   launch_reduce_partials(s.partial, 1, s.nrm2, 0, c->st);
   nk = 2;
-  if (want && ds != c->st) cudaStreamWaitEvent(c->st, s.ev_join, 0);
+  if (want) cudaStreamWaitEvent(c->st, s.ev_join, 0);
   const double tol2 = (p->tol * nf) * (p->tol * nf);
   restart_gate_kernel<<<1, 1, 0, c->st>>>(s.dflags, want, s.nrm2, tol2);
   nk++;
@@ -951,7 +951,7 @@ static dd_status end_cycle(dd_ctx* c, SolverBuffers& s, int mm, const dd_solve_p
       nk += 1 + launch_gs_dot(s.V16, k + 1, n4, s.w, s.partial, gate, 1, c->st, s.vscale);
     else
       nk += 1 + launch_gs_dot(s.V, k + 1, n4, s.w, s.partial, gate, 1, c->st);
-    launch_gs_reduce(s.partial, k + 1, (double2*)s.cp, gate, 1, c->st);
+    launch_gs_reduce(s.partial, k + 1, n4, (double2*)s.cp, gate, 1, c->st);
     nk++;
   }
   restart_decide_kernel<<<1, 1, 0, c->st>>>(s.dflags, want, k, s.cp, s.nrm2, defl_tol, s.status);
@@ -1092,7 +1092,6 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
   const int m = p->m, k = p->k, ldh = m + 1;
   const double tol = p->tol;
   const double nf = sqrt(nf2);
-  const double defl_tol = 1e-2;
   cudaEvent_t e0, e1, e2, e3, e4;
   cudaEventCreate(&e0); cudaEventCreate(&e1); cudaEventCreate(&e2); cudaEventCreate(&e3); cudaEventCreate(&e4);
   cudaEvent_t tstart, tend;
@@ -1159,45 +1158,37 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
         if (h16) {
           // the same Gram-Schmidt over the FP16 basis, projecting w in place; the new basis
           // vector is normalised on its way into V16 (and into vin for the next step)
-          double2* nrm_a = s.nrm2 + 1;
-          double2* nrm_b = s.nrm2 + 2;
           const float* sc = s.vscale;
           int nk = launch_gs_dot(V16(0), j + 1, n4, s.w, s.partial, nullptr, 0, c->st, sc);
-          launch_gs_reduce(s.partial, j + 1, (double2*)s.hA, nullptr, 0, c->st);
-          launch_gs_project(s.w, s.w, V16(0), j + 1, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st, sc);
-          launch_gs_reduce(s.partial2, 0, nrm_a, nullptr, 0, c->st);
-          gs_decide_kernel<<<1, 1, 0, c->st>>>(s.hA, j + 1, nrm_a, s.hB, s.flag, s.nu2);
+          launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
+          launch_gs_project(s.w, s.w, V16(0), j + 1, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st, sc,
+                            gs_tail_of(s, 1));
           nk += launch_gs_dot(V16(0), j + 1, n4, s.w, s.partial, s.flag, 1, c->st, sc);
-          launch_gs_reduce(s.partial, j + 1, (double2*)s.hB, s.flag, 1, c->st);
-          launch_gs_project(s.w, s.w, V16(0), j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc);
-          launch_gs_reduce(s.partial2, 0, nrm_b, s.flag, 1, c->st);
-          gs_decide2_kernel<<<1, 1, 0, c->st>>>(s.flag, nrm_b, s.nu2);
+          launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hB, s.flag, 1, c->st);
+          launch_gs_project(s.w, s.w, V16(0), j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc,
+                            gs_tail_of(s, 2));
           cudaEventRecord(s.ev_fork, c->st);
           cudaStreamWaitEvent(s.side, s.ev_fork, 0);
           arnoldi_finish_kernel<<<1, 1, 0, s.side>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status);
           cudaEventRecord(s.ev_join, s.side);
           launch_basis16_store(V16(j + 1), s.vin, s.w, n4, s.nu2, vs16, c->st);
           cudaStreamWaitEvent(c->st, s.ev_join, 0);
-          return launched(c, nk + 10);
+          return launched(c, nk + 6);
         }
         // Gram-Schmidt: classical projection with the exact norm of the result, repeated
         // once when it cancels more than half of |w| (Daniel-Gragg-Kaufman-Stewart test)
         float4* vn = Vv(j + 1);
-        double2* nrm_a = s.nrm2 + 1;
-        double2* nrm_b = s.nrm2 + 2;
         // the basis vectors are read through their scales (vscale), and the new one stays
         // unnormalised: its exact norm comes out of the projection pass
         const float* sc = s.vscale;
         int nk = launch_gs_dot(Vv(0), j + 1, n4, s.w, s.partial, nullptr, 0, c->st, sc);
-        launch_gs_reduce(s.partial, j + 1, (double2*)s.hA, nullptr, 0, c->st);
-        launch_gs_project(vn, s.w, Vv(0), j + 1, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st, sc);
-        launch_gs_reduce(s.partial2, 0, nrm_a, nullptr, 0, c->st);
-        gs_decide_kernel<<<1, 1, 0, c->st>>>(s.hA, j + 1, nrm_a, s.hB, s.flag, s.nu2);
+        launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
+        launch_gs_project(vn, s.w, Vv(0), j + 1, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st, sc,
+                            gs_tail_of(s, 1));
         nk += launch_gs_dot(Vv(0), j + 1, n4, vn, s.partial, s.flag, 1, c->st, sc);
-        launch_gs_reduce(s.partial, j + 1, (double2*)s.hB, s.flag, 1, c->st);
-        launch_gs_project(vn, vn, Vv(0), j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc);
-        launch_gs_reduce(s.partial2, 0, nrm_b, s.flag, 1, c->st);
-        gs_decide2_kernel<<<1, 1, 0, c->st>>>(s.flag, nrm_b, s.nu2);
+        launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hB, s.flag, 1, c->st);
+        launch_gs_project(vn, vn, Vv(0), j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc,
+                            gs_tail_of(s, 2));
         // the Hessenberg column and its Givens update (one thread) beside the new vector's
         // scale; both only read nu2
         cudaEventRecord(s.ev_fork, c->st);
@@ -1206,7 +1197,7 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
         cudaEventRecord(s.ev_join, s.side);
         set_vscale_kernel<<<1, 1, 0, c->st>>>(s.vscale + j + 1, s.nu2);
         cudaStreamWaitEvent(c->st, s.ev_join, 0);
-        return launched(c, nk + 10);
+        return launched(c, nk + 6);
       }));
       cudaEventRecord(e3, c->st);
       TRY(read_status(c));
@@ -1241,7 +1232,7 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
       fprintf(stderr, "[dd] basis orthogonality max|V^H V - I| = %.3e over %d vectors\n", dev, mm + 1);
     }
     CycleEnd ce;
-    TRY(end_cycle(c, s, mm, p, nf, true, &ce));
+    TRY(end_cycle(c, s, mm, p, nf, &ce));
     rho2 = ce.rho2;
     reliable++;
     rel = sqrt(rho2) / nf;
@@ -1347,21 +1338,17 @@ static dd_status lock_gs(dd_ctx* c, SolverBuffers& s, int j, int m) {
   const long long n4 = c->g.V * 6;
   const int ldh = m + 1;
   float4* vn = s.V + (long long)(j + 1) * n4;
-  double2* nrm_a = s.nrm2 + 1;
-  double2* nrm_b = s.nrm2 + 2;
   int nk = launch_gs_dot(s.V, j + 1, n4, s.w, s.partial, nullptr, 0, c->st);
-  launch_gs_reduce(s.partial, j + 1, (double2*)s.hA, nullptr, 0, c->st);
-  launch_gs_project(vn, s.w, s.V, j + 1, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st);
-  launch_gs_reduce(s.partial2, 0, nrm_a, nullptr, 0, c->st);
-  gs_decide_kernel<<<1, 1, 0, c->st>>>(s.hA, j + 1, nrm_a, s.hB, s.flag, s.nu2);
+  launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
+  launch_gs_project(vn, s.w, s.V, j + 1, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st, nullptr,
+                    gs_tail_of(s, 1));
   nk += launch_gs_dot(s.V, j + 1, n4, vn, s.partial, s.flag, 1, c->st);
-  launch_gs_reduce(s.partial, j + 1, (double2*)s.hB, s.flag, 1, c->st);
-  launch_gs_project(vn, vn, s.V, j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st);
-  launch_gs_reduce(s.partial2, 0, nrm_b, s.flag, 1, c->st);
-  gs_decide2_kernel<<<1, 1, 0, c->st>>>(s.flag, nrm_b, s.nu2);
+  launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hB, s.flag, 1, c->st);
+  launch_gs_project(vn, vn, s.V, j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, nullptr,
+                    gs_tail_of(s, 2));
   launch_scale_inplace(vn, n4, s.nu2, c->st);
   arnoldi_finish_kernel<<<1, 1, 0, c->st>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status);
-  TRY(launched(c, nk + 10));
+  TRY(launched(c, nk + 6));
   return cuda_check(c, cudaMemcpyAsync(s.h_status, s.status, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->st),
                     "status");
 }
@@ -1372,7 +1359,7 @@ static dd_status lock_end_cycle(dd_ctx* c, SolverBuffers& s, LockRhs& R, int mm,
   const long long n4 = c->g.V * 6;
   const int m = p->m, k = p->k, ldh = m + 1;
   CycleEnd ce;
-  TRY(end_cycle(c, s, mm, p, R.nf, false, &ce));
+  TRY(end_cycle(c, s, mm, p, R.nf, &ce));
   R.rho2 = ce.rho2;
   R.reliable++;
   R.rel = sqrt(R.rho2) / R.nf;
@@ -1893,29 +1880,25 @@ static dd_status solve_gcr_one(dd_ctx* c, const dd_solve_params* p, double nf2, 
       TRY(apply_internal(c, Zv(k), wk, P32));
       cudaEventRecord(e2, c->st);
       // w_k <- w_k - W beta (classical, with the DGKS second pass); z_k <- z_k - Z beta
-      double2* nrm_a = s.nrm2 + 1;
-      double2* nrm_b = s.nrm2 + 2;
       int nk = launch_gs_dot(Wv(0), k, n4, wk, s.partial, nullptr, 0, c->st);
-      launch_gs_reduce(s.partial, k, (double2*)s.hA, nullptr, 0, c->st);
-      launch_gs_project(Wv(k), wk, Wv(0), k, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st);
-      launch_gs_reduce(s.partial2, 0, nrm_a, nullptr, 0, c->st);
+      launch_gs_reduce(s.partial, k, n4, (double2*)s.hA, nullptr, 0, c->st);
+      launch_gs_project(Wv(k), wk, Wv(0), k, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st, nullptr,
+                    gs_tail_of(s, 1));
       launch_gs_project(Zv(k), Zv(k), Zv(0), k, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st);
-      gs_decide_kernel<<<1, 1, 0, c->st>>>(s.hA, k, nrm_a, s.hB, s.flag, s.nu2);
       nk += launch_gs_dot(Wv(0), k, n4, Wv(k), s.partial, s.flag, 1, c->st);
-      launch_gs_reduce(s.partial, k, (double2*)s.hB, s.flag, 1, c->st);
-      launch_gs_project(Wv(k), Wv(k), Wv(0), k, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st);
-      launch_gs_reduce(s.partial2, 0, nrm_b, s.flag, 1, c->st);
+      launch_gs_reduce(s.partial, k, n4, (double2*)s.hB, s.flag, 1, c->st);
+      launch_gs_project(Wv(k), Wv(k), Wv(0), k, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, nullptr,
+                    gs_tail_of(s, 2));
       launch_gs_project(Zv(k), Zv(k), Zv(0), k, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st);
-      gs_decide2_kernel<<<1, 1, 0, c->st>>>(s.flag, nrm_b, s.nu2);
       launch_scale_inplace(Wv(k), n4, s.nu2, c->st);
       launch_scale_inplace(Zv(k), n4, s.nu2, c->st);
       // alpha_k = <w_k, r>; r <- r - alpha_k w_k with its exact norm
       nk += launch_gs_dot(Wv(k), 1, n4, r, s.partial, nullptr, 0, c->st);
-      launch_gs_reduce(s.partial, 1, (double2*)(alpha + k), nullptr, 0, c->st);
+      launch_gs_reduce(s.partial, 1, n4, (double2*)(alpha + k), nullptr, 0, c->st);
       launch_gs_project(r, r, Wv(k), 1, n4, (const double2*)(alpha + k), s.partial2, nullptr, 0, c->st);
-      launch_gs_reduce(s.partial2, 0, s.nrm2 + 3, nullptr, 0, c->st);
+      launch_gs_reduce(s.partial2, 0, n4, s.nrm2 + 3, nullptr, 0, c->st);
       gcr_status_kernel<<<1, 1, 0, c->st>>>(s.nrm2 + 3, s.nu2, s.status);
-      TRY(launched(c, nk + 17));
+      TRY(launched(c, nk + 13));
       cudaEventRecord(e3, c->st);
       TRY(read_status(c));
       float ms;

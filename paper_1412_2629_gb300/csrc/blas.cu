@@ -43,24 +43,46 @@ __device__ inline void stv(uint2* p, long long q, float4 v, float s) {
   p[q] = make_uint2(f2h(v.x * s, v.y * s), f2h(v.z * s, v.w * s));
 }
 
-// Block reduction of NV complex doubles; thread 0 of the block ends with the sums in s[].
-template <int NV>
-__device__ inline void block_reduce(double2 (&v)[NV], double2* s_out) {
-  __shared__ double2 sh[BT / 32][NV];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// Blocks of a grid-stride kernel over n4 elements: four per SM, fewer when there are not that
+// many elements (an 8^4 field has 96 blocks' worth), where idle threads would only lengthen
+// the FP64 reductions below.
+static int blas_blocks(long long n4) {
+  const long long need = (n4 + BT - 1) / BT;
+  const int most = blas_partials_blocks();
+  return need < most ? (int)need : most;
+}
+
+// Sums of N reals per thread over a warp.  Each butterfly step halves the list: a lane keeps
+// one half, sends the other to its partner and adds what it receives, so 32 lanes spend
+// N / 2 + N / 4 + ... FP64 additions each instead of 5 N.  GB300 adds two FP64 numbers per
+// clock and SM, and with full butterflies the 18 sums of a Gram-Schmidt dot pass took longer
+// than its memory traffic on all but the largest lattices.  Returns whether this lane ends
+// with a sum, v[0], and which one.
+template <int N, int O>
+__device__ __forceinline__ void warp_fold(double* v, int& index, int& count) {
+  constexpr int half = (N + 1) / 2;
+  const bool up = threadIdx.x & O;
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      v[i].x += __shfl_xor_sync(0xffffffffu, v[i].x, o);
-      v[i].y += __shfl_xor_sync(0xffffffffu, v[i].y, o);
-    }
-    if (lane == 0) sh[w][i] = v[i];
+  for (int i = 0; i < half; ++i) {
+    const double lo = v[i], hi = half + i < N ? v[half + i] : 0.0;
+    v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, O);
   }
+  index += up ? half : 0;
+  count = up ? count - half : min(count, half);
+  if constexpr (O > 1) warp_fold<half, O / 2>(v, index, count);
+}
+
+// s_out[k] = sum over the block of v[k], k < N (shared memory).
+template <int N>
+__device__ inline void block_sums(double (&v)[N], double* s_out) {
+  __shared__ double sh[BT / 32][N];
+  int index = 0, count = N;
+  warp_fold<N, 16>(v, index, count);
+  if (count > 0) sh[threadIdx.x >> 5][index] = v[0];
   __syncthreads();
-  if (threadIdx.x < NV) {
-    double2 t = make_double2(0, 0);
-    for (int k = 0; k < BT / 32; ++k) { t.x += sh[k][threadIdx.x].x; t.y += sh[k][threadIdx.x].y; }
+  if (threadIdx.x < N) {
+    double t = 0;
+    for (int k = 0; k < BT / 32; ++k) t += sh[k][threadIdx.x];
     s_out[threadIdx.x] = t;
   }
   __syncthreads();
@@ -84,12 +106,13 @@ __global__ void __launch_bounds__(BT) multi_dot_kernel(const float4* V, int v0, 
       }
     }
   }
-  double2 acc[NV];
+  double acc[2 * NV];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) acc[i] = make_double2(re[i], im[i]);
-  __shared__ double2 out[NV];
-  block_reduce<NV>(acc, out);
-  if (threadIdx.x < NV && v0 + (int)threadIdx.x < nv) partial[(long long)blockIdx.x * ldp + v0 + threadIdx.x] = out[threadIdx.x];
+  for (int i = 0; i < NV; ++i) { acc[2 * i] = re[i]; acc[2 * i + 1] = im[i]; }
+  __shared__ double out[2 * NV];
+  block_sums(acc, out);
+  if (threadIdx.x < NV && v0 + (int)threadIdx.x < nv)
+    partial[(long long)blockIdx.x * ldp + v0 + threadIdx.x] = make_double2(out[2 * threadIdx.x], out[2 * threadIdx.x + 1]);
 }
 
 int launch_multi_dot(const float4* V, int nv, long long n4, const float4* w, double2* partial, cudaStream_t st) {
@@ -128,10 +151,10 @@ __global__ void __launch_bounds__(BT) norm2_64_kernel(const double2* x, long lon
     double2 a = x[q];
     s += a.x * a.x + a.y * a.y;
   }
-  double2 acc[1] = {make_double2(s, 0.0)};
-  __shared__ double2 out[1];
-  block_reduce<1>(acc, out);
-  if (threadIdx.x == 0) partial[blockIdx.x] = out[0];
+  double acc[1] = {s};
+  __shared__ double out[1];
+  block_sums(acc, out);
+  if (threadIdx.x == 0) partial[blockIdx.x] = make_double2(out[0], 0.0);
 }
 void launch_norm2_64(const double2* x, long long n2, double2* partial, cudaStream_t st) {
   norm2_64_kernel<<<blas_partials_blocks(), BT, 0, st>>>(x, n2, partial);
@@ -308,25 +331,25 @@ __global__ void __launch_bounds__(BT, 2) gs_dot_kernel(const float4* __restrict_
         im[i] += d.im;
       }
   }
-  double2 acc[NV + 1];
+  double acc[2 * NV + 1];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
+  for (int i = 0; i < NV; ++i) { acc[2 * i] = re[i]; acc[2 * i + 1] = im[i]; }
+  acc[2 * NV] = ww;
+  __shared__ double out[2 * NV + 1];
+  block_sums(acc, out);
+  if ((int)threadIdx.x < nvc) {
     // stored V_i = v_i / vscale[i]: the product with v_i is the stored one times vscale[i]
-    const double sc = (vscale && i < nvc) ? (double)vscale[v0 + i] : 1.0;
-    acc[i] = make_double2(re[i] * sc, im[i] * sc);
+    const double sc = vscale ? (double)vscale[v0 + threadIdx.x] : 1.0;
+    partial[(long long)qb * ldp + v0 + threadIdx.x] = make_double2(out[2 * threadIdx.x] * sc, out[2 * threadIdx.x + 1] * sc);
   }
-  acc[NV] = make_double2(ww, 0.0);
-  __shared__ double2 out[NV + 1];
-  block_reduce<NV + 1>(acc, out);
-  if ((int)threadIdx.x < nvc) partial[(long long)qb * ldp + v0 + threadIdx.x] = out[threadIdx.x];
-  if (self && threadIdx.x == 0) partial[(long long)qb * ldp + nv] = out[NV];
+  if (self && threadIdx.x == 0) partial[(long long)qb * ldp + nv] = make_double2(out[2 * NV], 0.0);
 }
 
 // partial layout [q-slice][nv + 1]: entries 0..nv-1 are V^H w, entry nv is |w|^2.
 int launch_gs_dot(const float4* V, int nv, long long n4, const float4* w, double2* partial, const int* gate, int want,
                   cudaStream_t st, const float* vscale) {
   const int nch = nv > 0 ? (nv + 7) / 8 : 1;
-  gs_dot_kernel<8, 2><<<blas_partials_blocks() * nch, BT, 0, st>>>(V, nv, nch, n4, w, partial, nv + 1, gate, want,
+  gs_dot_kernel<8, 2><<<blas_blocks(n4) * nch, BT, 0, st>>>(V, nv, nch, n4, w, partial, nv + 1, gate, want,
                                                                    vscale);
   return 1;
 }
@@ -384,24 +407,25 @@ __global__ void __launch_bounds__(BT, 2) gs_dot16_kernel(const uint4* __restrict
         }
     }
   }
-  double2 acc[NV + 1];
+  double acc[2 * NV + 1];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    const double sc = (vscale && i < nvc) ? (double)vscale[v0 + i] : 1.0;
-    acc[i] = make_double2(re[i] * sc, im[i] * sc);
+  for (int i = 0; i < NV; ++i) { acc[2 * i] = re[i]; acc[2 * i + 1] = im[i]; }
+  acc[2 * NV] = ww;
+  __shared__ double out[2 * NV + 1];
+  block_sums(acc, out);
+  if ((int)threadIdx.x < nvc) {
+    // stored V_i = v_i / vscale[i]: the product with v_i is the stored one times vscale[i]
+    const double sc = vscale ? (double)vscale[v0 + threadIdx.x] : 1.0;
+    partial[(long long)qb * ldp + v0 + threadIdx.x] = make_double2(out[2 * threadIdx.x] * sc, out[2 * threadIdx.x + 1] * sc);
   }
-  acc[NV] = make_double2(ww, 0.0);
-  __shared__ double2 out[NV + 1];
-  block_reduce<NV + 1>(acc, out);
-  if ((int)threadIdx.x < nvc) partial[(long long)qb * ldp + v0 + threadIdx.x] = out[threadIdx.x];
-  if (self && threadIdx.x == 0) partial[(long long)qb * ldp + nv] = out[NV];
+  if (self && threadIdx.x == 0) partial[(long long)qb * ldp + nv] = make_double2(out[2 * NV], 0.0);
 }
 
 int launch_gs_dot(const uint2* V, int nv, long long n4, const float4* w, double2* partial, const int* gate, int want,
                   cudaStream_t st, const float* vscale) {
   const int nch = nv > 0 ? (nv + 7) / 8 : 1;
   // n4 is even (six units per site): the basis is read as n4 / 2 pairs of units
-  gs_dot16_kernel<8, 2><<<blas_partials_blocks() * nch, BT, 0, st>>>(reinterpret_cast<const uint4*>(V), nv, nch,
+  gs_dot16_kernel<8, 2><<<blas_blocks(n4) * nch, BT, 0, st>>>(reinterpret_cast<const uint4*>(V), nv, nch,
                                                                      n4 / 2, w, partial, nv + 1, gate, want, vscale);
   return 1;
 }
@@ -422,8 +446,40 @@ __global__ void gs_reduce_kernel(const double2* partial, int nb, int ld, double2
   if (threadIdx.x == 0) out[i] = make_double2(shx[0], shy[0]);
 }
 
-void launch_gs_reduce(const double2* partial, int nv, double2* out, const int* gate, int want, cudaStream_t st) {
-  gs_reduce_kernel<<<nv + 1, 256, 0, st>>>(partial, blas_partials_blocks(), nv + 1, out, gate, want);
+void launch_gs_reduce(const double2* partial, int nv, long long n4, double2* out, const int* gate, int want,
+                      cudaStream_t st) {
+  gs_reduce_kernel<<<nv + 1, 256, 0, st>>>(partial, blas_blocks(n4), nv + 1, out, gate, want);
+}
+
+// The last block of a projection pass to finish (a device-scope ticket taken after a fence;
+// nobody waits) sums the blocks' norms in block order in FP64 and takes the pass's decision:
+// stage 1, after the first projection, asks for a second one when |out|^2 fell below half
+// of |w|^2 = hA[nv] and clears hB; stage 2, after the second, only replaces the norm.  In
+// place of two one-block launches per pass: see launch_gs_project.
+__device__ inline void gs_tail(double nrm, double2* norm_partial, const GsTail& tail, int nv) {
+  double acc[1] = {nrm};
+  __shared__ double o[1];
+  __shared__ int last;
+  block_sums(acc, o);
+  if (threadIdx.x == 0) norm_partial[blockIdx.x] = make_double2(o[0], 0.0);
+  if (tail.stage == 0) return;
+  if (threadIdx.x == 0) {
+    __threadfence();   // this block's norm is visible before its ticket is taken
+    last = atomicAdd(tail.ticket, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  double t = 0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += BT) t += __ldcg(&norm_partial[b].x);
+  acc[0] = t;
+  block_sums(acc, o);
+  if (tail.stage == 1)
+    for (int i = threadIdx.x; i <= nv; i += BT) tail.hB[i] = Z(0.0);
+  if (threadIdx.x == 0) {
+    *tail.nu2 = o[0];
+    if (tail.stage == 1) *tail.flag = o[0] < 0.5 * tail.hA[nv].re ? 1 : 0;
+    *tail.ticket = 0;
+  }
 }
 
 // out = w - V h with |out|^2 partials per block (exact norm of the projected vector).
@@ -436,7 +492,7 @@ constexpr int GP_U = 2, GP_B = 4;
 __global__ void __launch_bounds__(BT) gs_project_kernel(float4* out, const float4* w, const float4* __restrict__ V,
                                                         int nv, long long n4, const double2* h,
                                                         double2* norm_partial, const int* gate, int want,
-                                                        const float* vscale) {
+                                                        const float* vscale, GsTail tail) {
   if (gate && *gate != want) return;
   __shared__ float2 hs[64];
   for (int i = threadIdx.x; i < nv; i += BT) {
@@ -495,15 +551,13 @@ __global__ void __launch_bounds__(BT) gs_project_kernel(float4* out, const float
         nrm += a[u].x * a[u].x + a[u].y * a[u].y + a[u].z * a[u].z + a[u].w * a[u].w;
       }
   }
-  double2 acc[1] = {make_double2(nrm, 0.0)};
-  __shared__ double2 o[1];
-  block_reduce<1>(acc, o);
-  if (threadIdx.x == 0) norm_partial[blockIdx.x] = o[0];
+  gs_tail(nrm, norm_partial, tail, nv);
 }
 
 void launch_gs_project(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
-                       double2* norm_partial, const int* gate, int want, cudaStream_t st, const float* vscale) {
-  gs_project_kernel<<<blas_partials_blocks(), BT, 0, st>>>(out, w, V, nv, n4, h, norm_partial, gate, want, vscale);
+                       double2* norm_partial, const int* gate, int want, cudaStream_t st, const float* vscale,
+                       const GsTail& tail) {
+  gs_project_kernel<<<blas_blocks(n4), BT, 0, st>>>(out, w, V, nv, n4, h, norm_partial, gate, want, vscale, tail);
 }
 
 // out = w - V h over an FP16 basis read in unit pairs (see gs_dot16_kernel); in place
@@ -511,7 +565,7 @@ void launch_gs_project(float4* out, const float4* w, const float4* V, int nv, lo
 __global__ void __launch_bounds__(BT) gs_project16_kernel(float4* out, const float4* w, const uint4* __restrict__ V,
                                                           int nv, long long n8, const double2* h,
                                                           double2* norm_partial, const int* gate, int want,
-                                                          const float* vscale) {
+                                                          const float* vscale, GsTail tail) {
   if (gate && *gate != want) return;
   __shared__ float2 hs[64];
   for (int i = threadIdx.x; i < nv; i += BT) {
@@ -577,16 +631,14 @@ __global__ void __launch_bounds__(BT) gs_project16_kernel(float4* out, const flo
                ah[u].x * ah[u].x + ah[u].y * ah[u].y + ah[u].z * ah[u].z + ah[u].w * ah[u].w;
       }
   }
-  double2 acc[1] = {make_double2(nrm, 0.0)};
-  __shared__ double2 o[1];
-  block_reduce<1>(acc, o);
-  if (threadIdx.x == 0) norm_partial[blockIdx.x] = o[0];
+  gs_tail(nrm, norm_partial, tail, nv);
 }
 
 void launch_gs_project(float4* out, const float4* w, const uint2* V, int nv, long long n4, const double2* h,
-                       double2* norm_partial, const int* gate, int want, cudaStream_t st, const float* vscale) {
-  gs_project16_kernel<<<blas_partials_blocks(), BT, 0, st>>>(out, w, reinterpret_cast<const uint4*>(V), nv, n4 / 2, h,
-                                                             norm_partial, gate, want, vscale);
+                       double2* norm_partial, const int* gate, int want, cudaStream_t st, const float* vscale,
+                       const GsTail& tail) {
+  gs_project16_kernel<<<blas_blocks(n4), BT, 0, st>>>(out, w, reinterpret_cast<const uint4*>(V), nv, n4 / 2, h,
+                                                      norm_partial, gate, want, vscale, tail);
 }
 
 // v16 = FP16 of s w / sqrt(*nu2) and v32 = w / sqrt(*nu2) (the FP32 copy the next Schwarz

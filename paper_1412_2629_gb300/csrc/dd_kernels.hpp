@@ -117,10 +117,22 @@ int launch_recombine(uint2* out, const uint2* V, int nv, int nout, long long n4,
 // projections are taken against v_i.
 int launch_gs_dot(const float4* V, int nv, long long n4, const float4* w, double2* partial, const int* gate, int want,
                   cudaStream_t st, const float* vscale = nullptr);
-void launch_gs_reduce(const double2* partial, int nv, double2* out, const int* gate, int want, cudaStream_t st);
+void launch_gs_reduce(const double2* partial, int nv, long long n4, double2* out, const int* gate, int want,
+                      cudaStream_t st);
+// What the last block of a projection pass does with the squared norm of the result: 0
+// nothing (the blocks' sums stay in norm_partial), 1 nu2, hB = 0 and flag = "project again"
+// (|out|^2 below half of hA[nv] = |w|^2), 2 nu2 only.  ticket: a device int, zero between launches.
+struct GsTail {
+  int stage = 0;
+  int* ticket = nullptr;
+  const zd* hA = nullptr;
+  zd* hB = nullptr;
+  int* flag = nullptr;
+  double* nu2 = nullptr;
+};
 void launch_gs_project(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
                        double2* norm_partial, const int* gate, int want, cudaStream_t st,
-                       const float* vscale = nullptr);
+                       const float* vscale = nullptr, const GsTail& tail = GsTail());
 void launch_scale_inplace(float4* v, long long n4, const double* nu2, cudaStream_t st);
 // The same passes over an FP16 basis (w and the projection's output stay FP32), and the
 // FP16 basis store / load: v16 = FP16(s w / sqrt(nu2)) with the FP32 copy w / sqrt(nu2) in
@@ -128,7 +140,8 @@ void launch_scale_inplace(float4* v, long long n4, const double* nu2, cudaStream
 int launch_gs_dot(const uint2* V, int nv, long long n4, const float4* w, double2* partial, const int* gate, int want,
                   cudaStream_t st, const float* vscale);
 void launch_gs_project(float4* out, const float4* w, const uint2* V, int nv, long long n4, const double2* h,
-                       double2* norm_partial, const int* gate, int want, cudaStream_t st, const float* vscale);
+                       double2* norm_partial, const int* gate, int want, cudaStream_t st, const float* vscale,
+                       const GsTail& tail = GsTail());
 void launch_basis16_store(uint2* v16, float4* v32, const float4* w, long long n4, const double* nu2, float s,
                           cudaStream_t st, const int* gate = nullptr);
 void launch_basis16_load(float4* v32, const uint2* v16, long long n4, float s, cudaStream_t st);

@@ -111,33 +111,51 @@ __global__ void __launch_bounds__(256, 2) apply_A_shape_kernel(Geom g0, LinkPtr<
   out.store(g, s, y);
 }
 
+// Threads per block: `most`, halved until the grid has two blocks per SM (or a block is one
+// warp), so that a small lattice uses the whole chip.  FP64 blocks start at 64 threads: two
+// FP64 lanes per SM are busy with two warps, and on 8^4 the 16 blocks of 256 threads left
+// nine SMs in ten idle (107 -> 49 us cold; FP32 8.3 -> 7.7 us).  24^3x48 gains from the shorter
+// tail too: 1.42 -> 1.37 ms.
+static int block_threads(long long V, int most) {
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    sms = n > 0 ? n : 1;
+  }
+  while (most > 32 && V / most < 2 * sms) most >>= 1;
+  return most;
+}
+
 void launch_apply_A(const Geom& g, GaugeView U, CloverView C, FieldView in, FieldView out, const FieldView* f,
                     cudaStream_t st) {
-  unsigned nb = (unsigned)((g.V + 255) / 256);
+  const int nt = block_threads(g.V, in.prec == P64 ? 64 : 256);
+  const unsigned nb = (unsigned)((g.V + nt - 1) / nt);
   int res = f != nullptr;
   if (in.prec == P32 && domain_shape_id(g) != 0) {
     const LinkPtr<float> L{(const float2*)U.links};
     const CloverPtr<float> Cp{(const float4*)C.m};
     const SpinorPtr<float> vi{(float4*)in.data}, vo{(float4*)out.data}, fi{res ? (float4*)f->data : nullptr};
-    if (domain_shape_id(g) == 1) apply_A_shape_kernel<1><<<nb, 256, 0, st>>>(g, L, Cp, vi, vo, fi, res);
-    else apply_A_shape_kernel<2><<<nb, 256, 0, st>>>(g, L, Cp, vi, vo, fi, res);
+    if (domain_shape_id(g) == 1) apply_A_shape_kernel<1><<<nb, nt, 0, st>>>(g, L, Cp, vi, vo, fi, res);
+    else apply_A_shape_kernel<2><<<nb, nt, 0, st>>>(g, L, Cp, vi, vo, fi, res);
     return;
   }
   if (in.prec == P64) {
     SpinorPtr<double> fi{res ? (double2*)f->data : nullptr};
-    apply_A_kernel<double><<<nb, 256, 0, st>>>(g, LinkPtr<double>{(const double2*)U.links},
+    apply_A_kernel<double><<<nb, nt, 0, st>>>(g, LinkPtr<double>{(const double2*)U.links},
                                                CloverPtr<double>{(const double2*)C.m},
                                                SpinorPtr<double>{(double2*)in.data},
                                                SpinorPtr<double>{(double2*)out.data}, fi, res);
   } else if (in.prec == P32) {
     SpinorPtr<float> fi{res ? (float4*)f->data : nullptr};
-    apply_A_kernel<float><<<nb, 256, 0, st>>>(g, LinkPtr<float>{(const float2*)U.links},
+    apply_A_kernel<float><<<nb, nt, 0, st>>>(g, LinkPtr<float>{(const float2*)U.links},
                                               CloverPtr<float>{(const float4*)C.m},
                                               SpinorPtr<float>{(float4*)in.data}, SpinorPtr<float>{(float4*)out.data},
                                               fi, res);
   } else {
     SpinorPtr<__half> fi{res ? (uint4*)f->data : nullptr, res ? f->norm : nullptr};
-    apply_A_kernel<__half><<<nb, 256, 0, st>>>(g, LinkPtr<__half>{(const uint4*)U.links},
+    apply_A_kernel<__half><<<nb, nt, 0, st>>>(g, LinkPtr<__half>{(const uint4*)U.links},
                                                CloverPtr<__half>{(const uint4*)C.m},
                                                SpinorPtr<__half>{(uint4*)in.data, in.norm},
                                                SpinorPtr<__half>{(uint4*)out.data, out.norm}, fi, res);
