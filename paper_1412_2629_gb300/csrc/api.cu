@@ -526,7 +526,11 @@ static dd_status sap_error_flag(dd_ctx* c) {
   TRY(cuda_check(c, cudaStreamSynchronize(c->st), "sap"));
   if (e) {
     cudaMemsetAsync(c->sap_err, 0, sizeof(int), c->st);
-    return fail(c, DD_ERR_TIMEOUT, "a bounded wait for the domain's staged data ran out");
+    // a projection pass that gave up leaves its ticket short
+    if (c->sv.ticket) cudaMemsetAsync(c->sv.ticket, 0, sizeof(int), c->st);
+    for (SolverBuffers& b : c->lock)
+      if (b.ticket) cudaMemsetAsync(b.ticket, 0, sizeof(int), c->st);
+    return fail(c, DD_ERR_TIMEOUT, "a bounded wait for staged data ran out");
   }
   return DD_OK;
 }
@@ -1183,10 +1187,9 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
         const float* sc = s.vscale;
         int nk = launch_gs_dot(Vv(0), j + 1, n4, s.w, s.partial, nullptr, 0, c->st, sc);
         launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
-        launch_gs_project(vn, s.w, Vv(0), j + 1, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st, sc,
-                            gs_tail_of(s, 1));
-        nk += launch_gs_dot(Vv(0), j + 1, n4, vn, s.partial, s.flag, 1, c->st, sc);
-        launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hB, s.flag, 1, c->st);
+        const int nb = launch_gs_project_dot(vn, s.w, Vv(0), j + 1, n4, (const double2*)s.hA, sc, s.partial, s.partial2,
+                                             c->sap_err, c->st, gs_tail_of(s, 1));
+        launch_gs_reduce_blocks(s.partial, j + 1, nb, (double2*)s.hB, s.flag, 1, c->st);
         launch_gs_project(vn, vn, Vv(0), j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc,
                             gs_tail_of(s, 2));
         // the Hessenberg column and its Givens update (one thread) beside the new vector's
@@ -1340,10 +1343,9 @@ static dd_status lock_gs(dd_ctx* c, SolverBuffers& s, int j, int m) {
   float4* vn = s.V + (long long)(j + 1) * n4;
   int nk = launch_gs_dot(s.V, j + 1, n4, s.w, s.partial, nullptr, 0, c->st);
   launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
-  launch_gs_project(vn, s.w, s.V, j + 1, n4, (const double2*)s.hA, s.partial2, nullptr, 0, c->st, nullptr,
-                    gs_tail_of(s, 1));
-  nk += launch_gs_dot(s.V, j + 1, n4, vn, s.partial, s.flag, 1, c->st);
-  launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hB, s.flag, 1, c->st);
+  const int nb = launch_gs_project_dot(vn, s.w, s.V, j + 1, n4, (const double2*)s.hA, nullptr, s.partial, s.partial2,
+                                       c->sap_err, c->st, gs_tail_of(s, 1));
+  launch_gs_reduce_blocks(s.partial, j + 1, nb, (double2*)s.hB, s.flag, 1, c->st);
   launch_gs_project(vn, vn, s.V, j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, nullptr,
                     gs_tail_of(s, 2));
   launch_scale_inplace(vn, n4, s.nu2, c->st);
@@ -1898,7 +1900,7 @@ static dd_status solve_gcr_one(dd_ctx* c, const dd_solve_params* p, double nf2, 
       launch_gs_project(r, r, Wv(k), 1, n4, (const double2*)(alpha + k), s.partial2, nullptr, 0, c->st);
       launch_gs_reduce(s.partial2, 0, n4, s.nrm2 + 3, nullptr, 0, c->st);
       gcr_status_kernel<<<1, 1, 0, c->st>>>(s.nrm2 + 3, s.nu2, s.status);
-      TRY(launched(c, nk + 13));
+      TRY(launched(c, nk + 12));
       cudaEventRecord(e3, c->st);
       TRY(read_status(c));
       float ms;

@@ -5,7 +5,12 @@
 // terms at most), converts once, and the block and grid reductions run in FP64.  The
 // grid is a fixed multiple of the SM count, so the order of the final FP64 sum is
 // fixed and the result is reproducible run to run.
+#include <cuda.h>
+
+#include <algorithm>
+
 #include "dd_kernels.hpp"
+#include "dd_tma.cuh"
 
 namespace dd {
 
@@ -72,17 +77,17 @@ __device__ __forceinline__ void warp_fold(double* v, int& index, int& count) {
   if constexpr (O > 1) warp_fold<half, O / 2>(v, index, count);
 }
 
-// s_out[k] = sum over the block of v[k], k < N (shared memory).
-template <int N>
+// s_out[k] = sum over the block of NT threads of v[k], k < N (shared memory).
+template <int NT = BT, int N>
 __device__ inline void block_sums(double (&v)[N], double* s_out) {
-  __shared__ double sh[BT / 32][N];
+  __shared__ double sh[NT / 32][N];
   int index = 0, count = N;
   warp_fold<N, 16>(v, index, count);
   if (count > 0) sh[threadIdx.x >> 5][index] = v[0];
   __syncthreads();
   if (threadIdx.x < N) {
     double t = 0;
-    for (int k = 0; k < BT / 32; ++k) t += sh[k][threadIdx.x];
+    for (int k = 0; k < NT / 32; ++k) t += sh[k][threadIdx.x];
     s_out[threadIdx.x] = t;
   }
   __syncthreads();
@@ -450,17 +455,22 @@ void launch_gs_reduce(const double2* partial, int nv, long long n4, double2* out
                       cudaStream_t st) {
   gs_reduce_kernel<<<nv + 1, 256, 0, st>>>(partial, blas_blocks(n4), nv + 1, out, gate, want);
 }
+void launch_gs_reduce_blocks(const double2* partial, int nv, int nb, double2* out, const int* gate, int want,
+                             cudaStream_t st) {
+  gs_reduce_kernel<<<nv + 1, 256, 0, st>>>(partial, nb, nv + 1, out, gate, want);
+}
 
 // The last block of a projection pass to finish (a device-scope ticket taken after a fence;
 // nobody waits) sums the blocks' norms in block order in FP64 and takes the pass's decision:
 // stage 1, after the first projection, asks for a second one when |out|^2 fell below half
 // of |w|^2 = hA[nv] and clears hB; stage 2, after the second, only replaces the norm.  In
 // place of two one-block launches per pass: see launch_gs_project.
+template <int NT>
 __device__ inline void gs_tail(double nrm, double2* norm_partial, const GsTail& tail, int nv) {
   double acc[1] = {nrm};
   __shared__ double o[1];
   __shared__ int last;
-  block_sums(acc, o);
+  block_sums<NT>(acc, o);
   if (threadIdx.x == 0) norm_partial[blockIdx.x] = make_double2(o[0], 0.0);
   if (tail.stage == 0) return;
   if (threadIdx.x == 0) {
@@ -470,11 +480,11 @@ __device__ inline void gs_tail(double nrm, double2* norm_partial, const GsTail& 
   __syncthreads();
   if (!last) return;
   double t = 0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += BT) t += __ldcg(&norm_partial[b].x);
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += NT) t += __ldcg(&norm_partial[b].x);
   acc[0] = t;
-  block_sums(acc, o);
+  block_sums<NT>(acc, o);
   if (tail.stage == 1)
-    for (int i = threadIdx.x; i <= nv; i += BT) tail.hB[i] = Z(0.0);
+    for (int i = threadIdx.x; i <= nv; i += NT) tail.hB[i] = Z(0.0);
   if (threadIdx.x == 0) {
     *tail.nu2 = o[0];
     if (tail.stage == 1) *tail.flag = o[0] < 0.5 * tail.hA[nv].re ? 1 : 0;
@@ -551,13 +561,255 @@ __global__ void __launch_bounds__(BT) gs_project_kernel(float4* out, const float
         nrm += a[u].x * a[u].x + a[u].y * a[u].y + a[u].z * a[u].z + a[u].w * a[u].w;
       }
   }
-  gs_tail(nrm, norm_partial, tail, nv);
+  gs_tail<BT>(nrm, norm_partial, tail, nv);
 }
 
 void launch_gs_project(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
                        double2* norm_partial, const int* gate, int want, cudaStream_t st, const float* vscale,
                        const GsTail& tail) {
   gs_project_kernel<<<blas_blocks(n4), BT, 0, st>>>(out, w, V, nv, n4, h, norm_partial, gate, want, vscale, tail);
+}
+
+// The first projection of a step and the dots of the second one in one pass over the basis:
+// out = w - V h with |out|^2, and partial = V^H out.  Wherever the preconditioner is good, A M v
+// is close to v, the first projection cancels most of |w|^2 and the second is needed in
+// every step; computing its dots here, from the tile that the projection has just read,
+// costs no traffic, so a step reads the basis three times instead of four.
+//
+// One persistent block per SM walks tiles of T float4.  A tile of w and the tiles of all basis
+// vectors arrive by two copies, the second a box of a two-dimensional tensor map (vectors by
+// elements): one bulk copy per vector costs ~50 cycles more than its bytes and held
+// this kernel to 4 TB/s.  A warp of its own issues them several stages ahead.  G groups
+// of four warps take turns at the tiles, so one group's latencies (the wait, the barrier between
+// the two parts) hide behind the others: a group projects its tile in place, one thread per
+// complex number, and then takes the dots, warp u the vectors u, u + 4, ... against the
+// finished tile.  The number of stages is a multiple of G, so a stage always belongs to the
+// same group: waits on a barrier's phase parity are only sound for a waiter that has seen
+// the phase before (copies of different stages may land out of order).
+// Basis of 32^3x64 vectors, 16: 533 us (6.8 TB/s) for 1025 us of the two passes apart, 40: 1248
+// for 2398 us; 24^3x48, 8: 111 for 196 us.
+//
+// Sums: a lane adds at most 64 terms in FP32, as the dot kernels do, and hands them to a
+// two-float sum (TwoSum, exact to the last bits), which is converted to FP64 at the end.
+constexpr int GT = 128;   // threads of a group; 32 more threads issue the copies
+struct TwoFloat {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = hi + x, b = s - hi;
+    lo += (hi - (s - b)) + (x - b);
+    hi = s;
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+__device__ __forceinline__ bool group_or(int group, bool p) {   // barrier over one group
+  int r;
+  asm volatile(
+      "{\n .reg .pred P, Q;\n setp.ne.s32 P, %1, 0;\n barrier.cta.red.or.pred Q, %3, %2, P;\n selp.s32 %0, 1, 0, Q;\n}\n"
+      : "=r"(r)
+      : "r"((int)p), "n"(GT), "r"(group + 1)
+      : "memory");
+  return r != 0;
+}
+
+template <int T, int G, int MOST>   // MOST: the largest number of vectors
+__global__ void __launch_bounds__(G* GT + 32, 1)
+    gs_project_dot_kernel(const __grid_constant__ CUtensorMap basis, float4* out, const float4* w, int nv, long long n4,
+                          const double2* h,
+                          const float* vscale, double2* partial, double2* norm_partial, int stages, int* err,
+                          GsTail tail) {
+  constexpr int K = (MOST + 3) / 4;            // vectors per warp
+  constexpr int E = 2 * T / GT;                // complex numbers per thread
+  constexpr int FLUSH = 2048 / T;              // tiles between flushes of the FP32 sums
+  constexpr unsigned long long LIMIT = 2000000000ull;
+  extern __shared__ __align__(128) float4 sm[];
+  __shared__ float2 hs[64];
+  __shared__ uint64_t full[16], empty[16];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int piece = (nv + 1) * T;             // float4 per stage
+  for (int i = tid; i < nv; i += G * GT + 32) {
+    const double sc = vscale ? (double)vscale[i] : 1.0;   // h_i v_i = (h_i vscale[i]) V_i
+    hs[i] = make_float2((float)(h[i].x * sc), (float)(h[i].y * sc));
+  }
+  const long long ntile = n4 / T;
+  const int mine = (int)((ntile - blockIdx.x + gridDim.x - 1) / gridDim.x);   // tiles of this block
+  if (tid == 0)
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], GT / 32);
+    }
+  __syncthreads();
+
+  TwoFloat snrm;
+  const int group = tid / GT;
+  if (group == G) {
+    int issued = 0;
+    for (int k = 0, s = 0, turn = 0; k < mine; ++k) {
+      // the group has left this stage's previous tile
+      if (!__all_sync(0xffffffffu, turn == 0 || mbar_wait(&empty[s], (turn - 1) & 1, LIMIT))) break;
+      if (lane == 0) {
+        const long long q = (blockIdx.x + (long long)k * gridDim.x) * T;
+        mbar_expect_tx(&full[s], (uint32_t)(piece * 16));
+        bulk_g2s(sm + s * piece, w + q, T * 16, &full[s]);
+        tensor_g2s_2d(sm + s * piece + T, &basis, (int)(2 * q), 0, &full[s]);   // 8-byte elements
+      }
+      __syncwarp();
+      if (++s == stages) {
+        s = 0;
+        ++turn;
+      }
+      issued = k + 1;
+    }
+    // no copy may land in this block's shared memory after it has left (a wait only when a
+    // group gave up)
+    for (int k = max(0, issued - stages); k < issued; ++k) mbar_wait(&full[k % stages], (k / stages) & 1, LIMIT);
+  } else {
+    const int gt = tid - group * GT, warp = gt >> 5;
+    float re[K], im[K], nrm = 0.f;
+    TwoFloat sre[K], sim[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) re[k] = im[k] = 0.f;
+    int left = FLUSH;
+    for (int k = group, s = group, turn = 0; k < mine; k += G) {
+      float4* const st = sm + s * piece;
+      const float4* sv = st + T;
+      const bool ok = mbar_wait(&full[s], turn & 1, LIMIT);
+      float2 a[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) a[e] = reinterpret_cast<const float2*>(st)[gt + GT * e];
+#pragma unroll 4
+      for (int i = 0; i < nv; ++i) {
+        const float2 c = hs[i];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const float2 v = reinterpret_cast<const float2*>(sv + i * T)[gt + GT * e];
+          a[e].x -= c.x * v.x - c.y * v.y;
+          a[e].y -= c.x * v.y + c.y * v.x;
+        }
+      }
+      float2* o = reinterpret_cast<float2*>(out + (blockIdx.x + (long long)k * gridDim.x) * T);
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        o[gt + GT * e] = a[e];
+        reinterpret_cast<float2*>(st)[gt + GT * e] = a[e];
+        nrm += a[e].x * a[e].x + a[e].y * a[e].y;
+      }
+      if (group_or(group, !ok)) {   // a copy did not arrive: flag it and stop
+        if (gt == 0) atomicExch(err, 1);
+        break;
+      }
+#pragma unroll 2
+      for (int e = 0; e < T / 32; ++e) {
+        const float4 p = st[lane + 32 * e];
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          const int i = 4 * j + warp;
+          if (i < nv) {
+            const cx<float> d = dot4(sv[i * T + lane + 32 * e], p);
+            re[j] += d.re;
+            im[j] += d.im;
+          }
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before copies land here again
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[s]);
+      if (--left == 0 || k + G >= mine) {
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          sre[j].add(re[j]);
+          sim[j].add(im[j]);
+          re[j] = im[j] = 0.f;
+        }
+        snrm.add(nrm);
+        nrm = 0.f;
+        left = FLUSH;
+      }
+      s += G;
+      if (s >= stages) {
+        s -= stages;
+        ++turn;
+      }
+    }
+    // each vector's sum over the group's tiles lies in one warp
+    double acc[2 * K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      acc[2 * j] = sre[j].value();
+      acc[2 * j + 1] = sim[j].value();
+    }
+    int index = 0, count = 2 * K;
+    warp_fold<2 * K, 16>(acc, index, count);
+    const int i = 4 * (index >> 1) + warp;
+    double2* row = partial + (long long)(blockIdx.x * G + group) * (nv + 1);
+    if (count > 0 && i < nv) {
+      const double sc = vscale ? (double)vscale[i] : 1.0;
+      reinterpret_cast<double*>(row + i)[index & 1] = acc[0] * sc;
+    }
+    if (gt == 0) row[nv] = make_double2(0.0, 0.0);
+  }
+  gs_tail<G * GT + 32>(snrm.value(), norm_partial, tail, nv);
+}
+
+// Tensor map of nv basis vectors (rows) of n4 float4, in 8-byte elements (a box holds at most 256
+// per dimension): boxes of all rows by T float4.
+static bool basis_map(CUtensorMap* m, const float4* V, int nv, long long n4, int T) {
+  typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static const Encode encode = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return (Encode)f;
+  }();
+  if (!encode) return false;
+  const cuuint64_t dim[2] = {(cuuint64_t)n4 * 2, (cuuint64_t)nv}, stride[1] = {(cuuint64_t)n4 * 16};
+  const cuuint32_t box[2] = {(cuuint32_t)T * 2, (cuuint32_t)nv}, step[2] = {1, 1};
+  return encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<float4*>(V), dim, stride, box, step,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int T, int G, int MOST>
+static int project_dot_launch(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
+                              const float* vscale, double2* partial, double2* norm_partial, int* err, cudaStream_t st,
+                              const GsTail& tail) {
+  const int sms = blas_partials_blocks() / 4;
+  const size_t stage = (size_t)(nv + 1) * T * 16, room = (size_t)208 * 1024;
+  const int stages = (int)std::min<size_t>(16, room / stage) / G * G;
+  static int configured = 0;
+  if (!configured) {
+    cudaFuncSetAttribute(gs_project_dot_kernel<T, G, MOST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
+    configured = 1;
+  }
+  const int nb = (int)std::min<long long>(sms, n4 / T);
+  CUtensorMap basis;
+  if (!basis_map(&basis, V, nv, n4, T)) {   // no tensor maps: the two passes apart
+    launch_gs_project(out, w, V, nv, n4, h, norm_partial, nullptr, 0, st, vscale, tail);
+    launch_gs_dot(V, nv, n4, out, partial, nullptr, 0, st, vscale);
+    return blas_blocks(n4);
+  }
+  gs_project_dot_kernel<T, G, MOST><<<nb, G * GT + 32, stages * stage, st>>>(basis, out, w, nv, n4, h, vscale, partial,
+                                                                             norm_partial, stages, err, tail);
+  return nb * G;
+}
+
+// Tile and groups by the number of vectors: stages of 4 to 64 KB, at least two per group (three
+// for the single group), so that copies are in flight while every group works.  n4 is a
+// multiple of 6144 (V of 1024), hence of every tile.  Returns the number of rows in partial.
+int launch_gs_project_dot(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
+                          const float* vscale, double2* partial, double2* norm_partial, int* err, cudaStream_t st,
+                          const GsTail& tail) {
+  if (nv <= 7) return project_dot_launch<128, 4, 7>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
+  if (nv <= 15) return project_dot_launch<64, 4, 15>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
+  if (nv <= 31) return project_dot_launch<64, 3, 31>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
+  if (nv <= 51) return project_dot_launch<64, 2, 51>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
+  return project_dot_launch<64, 1, 63>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
 }
 
 // out = w - V h over an FP16 basis read in unit pairs (see gs_dot16_kernel); in place
@@ -631,7 +883,7 @@ __global__ void __launch_bounds__(BT) gs_project16_kernel(float4* out, const flo
                ah[u].x * ah[u].x + ah[u].y * ah[u].y + ah[u].z * ah[u].z + ah[u].w * ah[u].w;
       }
   }
-  gs_tail(nrm, norm_partial, tail, nv);
+  gs_tail<BT>(nrm, norm_partial, tail, nv);
 }
 
 void launch_gs_project(float4* out, const float4* w, const uint2* V, int nv, long long n4, const double2* h,
