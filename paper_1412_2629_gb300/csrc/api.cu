@@ -370,6 +370,13 @@ extern "C" dd_status dd_apply_D(dd_ctx* c, const void* in, void* out, int prec, 
     TRY(apply_internal(c, in, out, prec));
   } else {
     if (prec == P16) return fail(c, DD_ERR_INVALID, "FP16 needs the internal layout");
+    // directly on the caller's fields when they allow 16-byte accesses and do not overlap
+    const uintptr_t a = (uintptr_t)in, b = (uintptr_t)out, n = dd_spinor_bytes(c, prec, layout);
+    if (a % 16 == 0 && b % 16 == 0 && (a + n <= b || b + n <= a)) {
+      launch_apply_A_canonical(c->g, gauge_view(c, prec), clover_view(c, prec), in, out, prec, c->st);
+      TRY(launched(c));
+      return cuda_check(c, cudaStreamSynchronize(c->st), "apply_D");
+    }
     TRY(ensure_scratch(c));
     launch_pack_spinor(c->g, in, prec, view(c->g, c->scratch_in, prec), c->st);
     TRY(launched(c));

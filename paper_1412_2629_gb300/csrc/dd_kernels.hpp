@@ -48,6 +48,10 @@ void launch_apply_A_multi_list(const Geom& g, GaugeView U, CloverView C, const f
 void launch_apply_A(const Geom& g, GaugeView U, CloverView C, FieldView in, FieldView out, const FieldView* f,
                     cudaStream_t st);
 
+// out = A in on canonical FP64 or FP32 fields, 16-byte aligned and not overlapping.
+void launch_apply_A_canonical(const Geom& g, GaugeView U, CloverView C, const void* in, void* out, int prec,
+                              cudaStream_t st);
+
 // ---- Schwarz sweep (sap.cu)
 struct SapState {
   int mat_prec;        // P32 or P16: gauge and Schwarz matrices

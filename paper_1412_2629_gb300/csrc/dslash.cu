@@ -162,6 +162,123 @@ void launch_apply_A(const Geom& g, GaugeView U, CloverView C, FieldView in, Fiel
   }
 }
 
+// ------------------------------------------------------------------ canonical fields
+// The operator on the caller's own fields ([t][z][y][x][spin][colour]), without the two layout
+// passes: a thread keeps its place in the domain-major order (links and clover are read as
+// above) and finds its site and the eight neighbours in the canonical field by their index
+// steps.  The strided 16-byte spinor accesses cost L1 wavefronts, which hide behind FP64
+// arithmetic and cost less than the passes in FP32: FP64 24^3x48 1514 -> 1357 us (1350 us on
+// internal fields), FP32 32^3x64 635 -> 413 us (270 internal), FP32 8^4 27 -> 15.6 us.
+template <typename T> struct CanonField;
+template <> struct CanonField<float> {
+  const float4* p;
+  __device__ __forceinline__ void load(long long x, Spinor<float>& v) const {
+#pragma unroll
+    for (int u = 0; u < 6; ++u) {
+      const float4 q = p[6 * x + u];
+      const int k = 2 * u;
+      v.c[k / 3][k % 3] = mk(q.x, q.y);
+      v.c[(k + 1) / 3][(k + 1) % 3] = mk(q.z, q.w);
+    }
+  }
+  __device__ __forceinline__ void store(long long x, const Spinor<float>& v) const {
+#pragma unroll
+    for (int u = 0; u < 6; ++u) {
+      const int k = 2 * u;
+      const_cast<float4*>(p)[6 * x + u] = make_float4(v.c[k / 3][k % 3].re, v.c[k / 3][k % 3].im,
+                                                      v.c[(k + 1) / 3][(k + 1) % 3].re, v.c[(k + 1) / 3][(k + 1) % 3].im);
+    }
+  }
+};
+template <> struct CanonField<double> {
+  const double2* p;
+  __device__ __forceinline__ void load(long long x, Spinor<double>& v) const {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const double2 q = p[12 * x + k];
+      v.c[k / 3][k % 3] = mk(q.x, q.y);
+    }
+  }
+  __device__ __forceinline__ void store(long long x, const Spinor<double>& v) const {
+#pragma unroll
+    for (int k = 0; k < 12; ++k)
+      const_cast<double2*>(p)[12 * x + k] = make_double2(v.c[k / 3][k % 3].re, v.c[k / 3][k % 3].im);
+  }
+};
+
+template <int MU, typename T>
+__device__ __forceinline__ void hop_pair_canon(const Geom& g, const Site& st, long long s, long long x,
+                                               long long stride, const CanonField<T>& in, const LinkPtr<T>& U,
+                                               Spinor<T>& acc) {
+  Spinor<T> psi;
+  Half<T> h, uh;
+  Link<T> L;
+  const int c = st.n[MU] * g.b[MU] + st.l[MU];
+  in.load(c + 1 < g.L[MU] ? x + stride : x - (g.L[MU] - 1) * stride, psi);
+  project<MU, -1>(psi, h);
+  U.load(g, s, MU, L);
+  su3_mul(L, h, uh);
+  accum_recon<MU, -1>(acc, uh);
+  in.load(c > 0 ? x - stride : x + (g.L[MU] - 1) * stride, psi);
+  project<MU, +1>(psi, h);
+  U.load(g, neighbour(g, st, MU, -1), MU, L);
+  su3_dag_mul(L, h, uh);
+  accum_recon<MU, +1>(acc, uh);
+}
+
+template <typename T, int SHAPE>
+__global__ void __launch_bounds__(256) apply_A_canon_kernel(Geom g0, LinkPtr<T> U, CloverPtr<T> C, CanonField<T> in,
+                                                            CanonField<T> out) {
+  const Geom g = fixed_shape<SHAPE>(g0);
+  const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (s >= g.V) return;
+  const Site st = decode(g, s);
+  long long x = 0, stride[4], n = 1;
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    stride[mu] = n;
+    x += (st.n[mu] * g.b[mu] + st.l[mu]) * n;
+    n *= g.L[mu];
+  }
+  Spinor<T> hop;
+  zero(hop);
+  hop_pair_canon<0, T>(g, st, s, x, stride[0], in, U, hop);
+  hop_pair_canon<1, T>(g, st, s, x, stride[1], in, U, hop);
+  hop_pair_canon<2, T>(g, st, s, x, stride[2], in, U, hop);
+  hop_pair_canon<3, T>(g, st, s, x, stride[3], in, U, hop);
+  Spinor<T> v, y;
+  in.load(x, v);
+  T m[72];
+  C.load(g, s, m);
+  clover_mul(m, v, y);
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) y.c[a][b] = y.c[a][b] - T(0.5) * hop.c[a][b];
+  out.store(x, y);
+}
+
+void launch_apply_A_canonical(const Geom& g, GaugeView U, CloverView C, const void* in, void* out, int prec,
+                              cudaStream_t st) {
+  const int nt = block_threads(g.V, prec == P64 ? 64 : 256);
+  const unsigned nb = (unsigned)((g.V + nt - 1) / nt);
+  if (prec == P64) {
+    apply_A_canon_kernel<double, 0><<<nb, nt, 0, st>>>(g, LinkPtr<double>{(const double2*)U.links},
+                                                       CloverPtr<double>{(const double2*)C.m},
+                                                       CanonField<double>{(const double2*)in},
+                                                       CanonField<double>{(const double2*)out});
+    return;
+  }
+  const LinkPtr<float> L{(const float2*)U.links};
+  const CloverPtr<float> Cp{(const float4*)C.m};
+  const CanonField<float> a{(const float4*)in}, b{(const float4*)out};
+  switch (domain_shape_id(g)) {
+    case 1: apply_A_canon_kernel<float, 1><<<nb, nt, 0, st>>>(g, L, Cp, a, b); break;
+    case 2: apply_A_canon_kernel<float, 2><<<nb, nt, 0, st>>>(g, L, Cp, a, b); break;
+    default: apply_A_canon_kernel<float, 0><<<nb, nt, 0, st>>>(g, L, Cp, a, b); break;
+  }
+}
+
 }  // namespace dd
 
 namespace dd {
@@ -200,19 +317,18 @@ __device__ inline void hop_pair_multi(const Geom& g, const Site& st, long long s
   }
 }
 
+// The fields r0 .. r0 + NR - 1 at site s; in_list / out_list: FP32 fields anywhere in memory.
 template <typename T, int NR>
-__global__ void __launch_bounds__(128) apply_A_multi_kernel(Geom g, LinkPtr<T> U, CloverPtr<T> C, SpinorPtr<T> in0,
-                                                             SpinorPtr<T> out0, long long unit_stride,
-                                                             long long norm_stride, int nrhs,
-                                                             const float4* const* in_list, float4* const* out_list) {
+__device__ __forceinline__ void apply_A_multi_site(const Geom& g, long long s, int r0, const LinkPtr<T>& U,
+                                                   const CloverPtr<T>& C, const SpinorPtr<T>& in0,
+                                                   const SpinorPtr<T>& out0, long long unit_stride,
+                                                   long long norm_stride, const float4* const* in_list,
+                                                   float4* const* out_list) {
   typedef typename Arith<T>::type R;
-  long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (s >= g.V) return;
-  const int r0 = blockIdx.y * NR;
   SpinorPtr<T> in[NR], out[NR];
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
-    int rr = r0 + r < nrhs ? r0 + r : nrhs - 1;   // a short last group repeats the last field
+    const int rr = r0 + r;
     in[r] = in0;
     out[r] = out0;
     in[r].p += rr * unit_stride;
@@ -220,7 +336,7 @@ __global__ void __launch_bounds__(128) apply_A_multi_kernel(Geom g, LinkPtr<T> U
     shift_norm(in[r], rr * norm_stride);
     shift_norm(out[r], rr * norm_stride);
     if constexpr (std::is_same<T, float>::value) {
-      if (in_list) {   // FP32 fields anywhere in memory
+      if (in_list) {
         in[r].p = const_cast<float4*>(in_list[rr]);
         out[r].p = out_list[rr];
       }
@@ -238,7 +354,6 @@ __global__ void __launch_bounds__(128) apply_A_multi_kernel(Geom g, LinkPtr<T> U
   C.load(g, s, m);
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
-    if (r0 + r >= nrhs) break;
     Spinor<R> x, y;
     in[r].load(g, s, x);
     clover_mul(m, x, y);
@@ -250,31 +365,64 @@ __global__ void __launch_bounds__(128) apply_A_multi_kernel(Geom g, LinkPtr<T> U
   }
 }
 
+// Blocks that work on the same 128 sites with other fields are neighbours in launch order, so
+// the links and clover blocks come from HBM once and from L2 afterwards; a field left over
+// from the pairs runs alone.  Bound by the latency of the neighbours' loads (L1 and L2): three
+// blocks per SM at 168 registers, with a few spilled, beat two at 255 and four at 128 (six
+// fields of 24^3x48: 355, 430 and 377 us), and three fields per thread gain nothing over two.
+// The domain shape as compile-time constants and the launch order took six fields
+// from 541 to 349 us (169 us of traffic).
+constexpr int MULTI_NR = 2, MULTI_THREADS = 128;
+template <typename T, int SHAPE>
+__global__ void __launch_bounds__(MULTI_THREADS, 3)
+    apply_A_multi_kernel(Geom g0, LinkPtr<T> U, CloverPtr<T> C, SpinorPtr<T> in, SpinorPtr<T> out, long long unit_stride,
+                         long long norm_stride, int nrhs, int groups, const float4* const* in_list,
+                         float4* const* out_list) {
+  const Geom g = fixed_shape<SHAPE>(g0);
+  const long long s = (blockIdx.x / groups) * (long long)MULTI_THREADS + threadIdx.x;
+  if (s >= g.V) return;
+  const int r0 = (blockIdx.x % groups) * MULTI_NR;
+  if (r0 + 1 < nrhs)
+    apply_A_multi_site<T, 2>(g, s, r0, U, C, in, out, unit_stride, norm_stride, in_list, out_list);
+  else
+    apply_A_multi_site<T, 1>(g, s, r0, U, C, in, out, unit_stride, norm_stride, in_list, out_list);
+}
+
+template <typename T>
+static void multi_launch(const Geom& g, LinkPtr<T> U, CloverPtr<T> C, SpinorPtr<T> in, SpinorPtr<T> out,
+                         long long unit_stride, long long norm_stride, int nrhs, const float4* const* in_list,
+                         float4* const* out_list, cudaStream_t st) {
+  const int groups = (nrhs + MULTI_NR - 1) / MULTI_NR;
+  const unsigned nb = (unsigned)((g.V + MULTI_THREADS - 1) / MULTI_THREADS) * groups;
+  auto launch = [&](auto kernel) {
+    kernel<<<nb, MULTI_THREADS, 0, st>>>(g, U, C, in, out, unit_stride, norm_stride, nrhs, groups, in_list, out_list);
+  };
+  switch (domain_shape_id(g)) {
+    case 1: launch(apply_A_multi_kernel<T, 1>); break;
+    case 2: launch(apply_A_multi_kernel<T, 2>); break;
+    default: launch(apply_A_multi_kernel<T, 0>); break;
+  }
+}
+
 void launch_apply_A_multi(const Geom& g, GaugeView U, CloverView C, FieldView in, FieldView out, int nrhs,
                           cudaStream_t st) {
-  const int NR = 2;
-  dim3 grid((unsigned)((g.V + 127) / 128), (unsigned)((nrhs + NR - 1) / NR));
   if (in.prec == P32) {
-    apply_A_multi_kernel<float, NR><<<grid, 128, 0, st>>>(
-        g, LinkPtr<float>{(const float2*)U.links}, CloverPtr<float>{(const float4*)C.m},
-        SpinorPtr<float>{(float4*)in.data}, SpinorPtr<float>{(float4*)out.data}, g.V * 6, 0, nrhs, nullptr, nullptr);
+    multi_launch<float>(g, LinkPtr<float>{(const float2*)U.links}, CloverPtr<float>{(const float4*)C.m},
+                        SpinorPtr<float>{(float4*)in.data}, SpinorPtr<float>{(float4*)out.data}, g.V * 6, 0, nrhs,
+                        nullptr, nullptr, st);
   } else {
     // FP16 fields are V * 52 bytes each (values, then the per-site norms) and follow each
     // other: 13 V / 4 uint4 units or 13 V floats apart (V is a multiple of 64)
-    apply_A_multi_kernel<__half, NR><<<grid, 128, 0, st>>>(
-        g, LinkPtr<__half>{(const uint4*)U.links}, CloverPtr<__half>{(const uint4*)C.m},
-        SpinorPtr<__half>{(uint4*)in.data, in.norm}, SpinorPtr<__half>{(uint4*)out.data, out.norm}, 13 * g.V / 4,
-        13 * g.V, nrhs, nullptr, nullptr);
+    multi_launch<__half>(g, LinkPtr<__half>{(const uint4*)U.links}, CloverPtr<__half>{(const uint4*)C.m},
+                         SpinorPtr<__half>{(uint4*)in.data, in.norm}, SpinorPtr<__half>{(uint4*)out.data, out.norm},
+                         13 * g.V / 4, 13 * g.V, nrhs, nullptr, nullptr, st);
   }
 }
 
 void launch_apply_A_multi_list(const Geom& g, GaugeView U, CloverView C, const float4* const* in,
                                float4* const* out, int nrhs, cudaStream_t st) {
-  const int NR = 2;
-  dim3 grid((unsigned)((g.V + 127) / 128), (unsigned)((nrhs + NR - 1) / NR));
-  apply_A_multi_kernel<float, NR><<<grid, 128, 0, st>>>(
-      g, LinkPtr<float>{(const float2*)U.links}, CloverPtr<float>{(const float4*)C.m}, SpinorPtr<float>{nullptr},
-      SpinorPtr<float>{nullptr}, 0, 0, nrhs, in, out);
+  multi_launch<float>(g, LinkPtr<float>{(const float2*)U.links}, CloverPtr<float>{(const float4*)C.m},
+                      SpinorPtr<float>{nullptr}, SpinorPtr<float>{nullptr}, 0, 0, nrhs, in, out, st);
 }
 
 }  // namespace dd

@@ -20,21 +20,70 @@ __device__ inline long long canon_index(const Geom& g, const int x[4]) {
   return x[0] + (long long)g.L[0] * (x[1] + (long long)g.L[1] * (x[2] + (long long)g.L[2] * x[3]));
 }
 
-template <typename C, typename T>
+// One site of a canonical field, 24 reals in a row, in 16-byte accesses where the field's
+// address allows them (VEC): 24 scalar accesses a site, each of a warp in 32 lines, bound
+// the layout passes (whole calls, FP32 24^3x48: unpacking 91 -> 35 us, packing 40 -> 31 us).
+template <bool VEC> __device__ __forceinline__ void canon_load(const double* q, double v[24]) {
+#pragma unroll
+  for (int k = 0; k < 24; k += 2) {
+    if constexpr (VEC) {
+      const double2 w = *reinterpret_cast<const double2*>(q + k);
+      v[k] = w.x; v[k + 1] = w.y;
+    } else {
+      v[k] = q[k]; v[k + 1] = q[k + 1];
+    }
+  }
+}
+template <bool VEC> __device__ __forceinline__ void canon_load(const float* q, float v[24]) {
+#pragma unroll
+  for (int k = 0; k < 24; k += 4) {
+    if constexpr (VEC) {
+      const float4 w = *reinterpret_cast<const float4*>(q + k);
+      v[k] = w.x; v[k + 1] = w.y; v[k + 2] = w.z; v[k + 3] = w.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[k + e] = q[k + e];
+    }
+  }
+}
+template <bool VEC> __device__ __forceinline__ void canon_store(double* q, const double v[24]) {
+#pragma unroll
+  for (int k = 0; k < 24; k += 2) {
+    if constexpr (VEC) {
+      *reinterpret_cast<double2*>(q + k) = make_double2(v[k], v[k + 1]);
+    } else {
+      q[k] = v[k]; q[k + 1] = v[k + 1];
+    }
+  }
+}
+template <bool VEC> __device__ __forceinline__ void canon_store(float* q, const float v[24]) {
+#pragma unroll
+  for (int k = 0; k < 24; k += 4) {
+    if constexpr (VEC) {
+      *reinterpret_cast<float4*>(q + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) q[k + e] = v[k + e];
+    }
+  }
+}
+
+template <typename C, typename T, bool VEC>
 __global__ void pack_spinor_kernel(Geom g, const C* canon, SpinorPtr<T> out) {
   long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (s >= g.V) return;
   Site st = decode(g, s);
   int x[4];
   site_global(g, st, x);
-  const C* q = canon + 24 * canon_index(g, x);
+  C q[24];
+  canon_load<VEC>(canon + 24 * canon_index(g, x), q);
   Spinor<typename Arith<T>::type> v;
 #pragma unroll
   for (int k = 0; k < 12; ++k) v.c[k / 3][k % 3] = mk<typename Arith<T>::type>(q[2 * k], q[2 * k + 1]);
   out.store(g, s, v);
 }
 
-template <typename T, typename C>
+template <typename T, typename C, bool VEC>
 __global__ void unpack_spinor_kernel(Geom g, SpinorPtr<T> in, C* canon) {
   long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (s >= g.V) return;
@@ -43,37 +92,46 @@ __global__ void unpack_spinor_kernel(Geom g, SpinorPtr<T> in, C* canon) {
   site_global(g, st, x);
   Spinor<typename Arith<T>::type> v;
   in.load(g, s, v);
-  C* q = canon + 24 * canon_index(g, x);
+  C q[24];
 #pragma unroll
   for (int k = 0; k < 12; ++k) { q[2 * k] = (C)v.c[k / 3][k % 3].re; q[2 * k + 1] = (C)v.c[k / 3][k % 3].im; }
+  canon_store<VEC>(canon + 24 * canon_index(g, x), q);
 }
 
 static inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
-template <typename C>
+template <typename C, bool VEC>
 static void pack_dispatch(const Geom& g, const C* canon, FieldView out, cudaStream_t st) {
   unsigned nb = nblk(g.V, 256);
-  if (out.prec == P64) pack_spinor_kernel<C, double><<<nb, 256, 0, st>>>(g, canon, SpinorPtr<double>{(double2*)out.data});
-  else if (out.prec == P32) pack_spinor_kernel<C, float><<<nb, 256, 0, st>>>(g, canon, SpinorPtr<float>{(float4*)out.data});
-  else pack_spinor_kernel<C, __half><<<nb, 256, 0, st>>>(g, canon, SpinorPtr<__half>{(uint4*)out.data, out.norm});
+  if (out.prec == P64) pack_spinor_kernel<C, double, VEC><<<nb, 256, 0, st>>>(g, canon, SpinorPtr<double>{(double2*)out.data});
+  else if (out.prec == P32) pack_spinor_kernel<C, float, VEC><<<nb, 256, 0, st>>>(g, canon, SpinorPtr<float>{(float4*)out.data});
+  else pack_spinor_kernel<C, __half, VEC><<<nb, 256, 0, st>>>(g, canon, SpinorPtr<__half>{(uint4*)out.data, out.norm});
 }
+
+static bool vec_aligned(const void* p) { return (uintptr_t)p % 16 == 0; }
 
 void launch_pack_spinor(const Geom& g, const void* canon, int canon_prec, FieldView out, cudaStream_t st) {
-  if (canon_prec == P64) pack_dispatch(g, (const double*)canon, out, st);
-  else pack_dispatch(g, (const float*)canon, out, st);
+  const bool vec = vec_aligned(canon);
+  if (canon_prec == P64)
+    vec ? pack_dispatch<double, true>(g, (const double*)canon, out, st) : pack_dispatch<double, false>(g, (const double*)canon, out, st);
+  else
+    vec ? pack_dispatch<float, true>(g, (const float*)canon, out, st) : pack_dispatch<float, false>(g, (const float*)canon, out, st);
 }
 
-template <typename C>
+template <typename C, bool VEC>
 static void unpack_dispatch(const Geom& g, FieldView in, C* canon, cudaStream_t st) {
   unsigned nb = nblk(g.V, 256);
-  if (in.prec == P64) unpack_spinor_kernel<double, C><<<nb, 256, 0, st>>>(g, SpinorPtr<double>{(double2*)in.data}, canon);
-  else if (in.prec == P32) unpack_spinor_kernel<float, C><<<nb, 256, 0, st>>>(g, SpinorPtr<float>{(float4*)in.data}, canon);
-  else unpack_spinor_kernel<__half, C><<<nb, 256, 0, st>>>(g, SpinorPtr<__half>{(uint4*)in.data, in.norm}, canon);
+  if (in.prec == P64) unpack_spinor_kernel<double, C, VEC><<<nb, 256, 0, st>>>(g, SpinorPtr<double>{(double2*)in.data}, canon);
+  else if (in.prec == P32) unpack_spinor_kernel<float, C, VEC><<<nb, 256, 0, st>>>(g, SpinorPtr<float>{(float4*)in.data}, canon);
+  else unpack_spinor_kernel<__half, C, VEC><<<nb, 256, 0, st>>>(g, SpinorPtr<__half>{(uint4*)in.data, in.norm}, canon);
 }
 
 void launch_unpack_spinor(const Geom& g, FieldView in, void* canon, int canon_prec, cudaStream_t st) {
-  if (canon_prec == P64) unpack_dispatch(g, in, (double*)canon, st);
-  else unpack_dispatch(g, in, (float*)canon, st);
+  const bool vec = vec_aligned(canon);
+  if (canon_prec == P64)
+    vec ? unpack_dispatch<double, true>(g, in, (double*)canon, st) : unpack_dispatch<double, false>(g, in, (double*)canon, st);
+  else
+    vec ? unpack_dispatch<float, true>(g, in, (float*)canon, st) : unpack_dispatch<float, false>(g, in, (float*)canon, st);
 }
 
 __global__ void pack_gauge_kernel(Geom g, const double* canon, int anti, double2* u64, float2* u32, uint4* u16) {
