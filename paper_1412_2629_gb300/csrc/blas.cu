@@ -633,11 +633,13 @@ __global__ void __launch_bounds__(G* GT + 32, 1)
   }
   const long long ntile = n4 / T;
   const int mine = (int)((ntile - blockIdx.x + gridDim.x - 1) / gridDim.x);   // tiles of this block
-  if (tid == 0)
+  if (tid == 0) {
     for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], GT / 32);
     }
+    mbar_init_fence();
+  }
   __syncthreads();
 
   TwoFloat snrm;

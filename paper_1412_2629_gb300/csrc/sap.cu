@@ -378,6 +378,7 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
     if (tid == 0) {
       mbar_init(&mbar, 1);
       mbar_init(&mbar_inj, 1);
+      mbar_init_fence();
     }
     __syncthreads();
     if (tid == 0) {
@@ -648,6 +649,32 @@ __device__ __forceinline__ void ld_half3(const float4* q, int stride, Half<float
   for (int k = 0; k < 6; ++k) v.c[k / 3][k % 3] = w[k];
 }
 
+// The same in a work buffer, colour by colour: unit c holds colour c of both spins, so a hop needs
+// two units for each colour that it projects and keeps few numbers waiting for their partners.
+__device__ __forceinline__ void ld_work(const float4* q, int stride, Half<float>& v) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float4 w = q[c * stride];
+    v.c[0][c] = mk(w.x, w.y);
+    v.c[1][c] = mk(w.z, w.w);
+  }
+}
+__device__ __forceinline__ void st_work(float4* q, int stride, const Half<float>& v) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) q[c * stride] = make_float4(v.c[0][c].re, v.c[0][c].im, v.c[1][c].re, v.c[1][c].im);
+}
+// a whole site in the frame whose own half starts at `own`
+__device__ __forceinline__ void ld_frame(const float4* own, const float4* oth, int stride, Spinor<float>& v) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float4 a = own[c * stride], b = oth[c * stride];
+    v.c[0][c] = mk(a.x, a.y);
+    v.c[1][c] = mk(a.z, a.w);
+    v.c[2][c] = mk(b.x, b.y);
+    v.c[3][c] = mk(b.z, b.w);
+  }
+}
+
 // own half of the sum over the two lanes of a site
 __device__ __forceinline__ void join_halves(const Spinor<float>& acc, Half<float>& own) {
 #pragma unroll
@@ -848,12 +875,8 @@ __device__ __forceinline__ void pair_hop(const Geom& g, const PairSites& q, cons
   const int j = q.neighbour<P>(MU);
   // U_mu of the site itself, or of the neighbour (any link where that is a zero slot)
   const int r = q.h ? (1 - P) * g.Hd + (j & (g.Hd - 1)) : P * g.Hd + q.i;
-  cx<float> v[12];
-  ld_half3(own + j, HP, v);
-  ld_half3(oth + j, HP, v + 6);
   Spinor<float> psi;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) psi.c[k / 3][k % 3] = v[k];
+  ld_frame(own + j, oth + j, HP, psi);
   Half<float> hp, uh;
   frame_project<MU>(psi, q.st, hp);
   if constexpr (H2) {
@@ -970,12 +993,8 @@ __device__ __forceinline__ void pair_face_write(const Geom& g, const Geom& gf, l
   for (int k = threadIdx.x; k < gf.face_block / 2; k += 2 * g.Hd) {
     const FaceSite f = face_site(g, SIDE, k);
     const float4* b = sE + (f.r >= g.Hd ? 6 * HP + f.r - g.Hd : f.r);
-    cx<float> w[12];
-    ld_half3(b + 3 * SIDE * HP, HP, w);
-    ld_half3(b + 3 * (1 - SIDE) * HP, HP, w + 6);
     Spinor<float> v;
-#pragma unroll
-    for (int c = 0; c < 12; ++c) v.c[c / 3][c % 3] = w[c];
+    ld_frame(b + 3 * SIDE * HP, b + 3 * (1 - SIDE) * HP, HP, v);
     Half<float> hp, uh;
     switch (f.mu) {
       case 0: frame_project<0>(v, st, hp); break;
@@ -1062,8 +1081,8 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
   if (tid == 0) {
 #pragma unroll
     for (int b = 0; b < 3; ++b) mbar_init(&bars[b], 1);
+    mbar_init_fence();
     mbar_expect_tx(&bars[0], lk_bytes + face_bytes);
-    if (a.use_faces) stage_faces(a.faces);
     bulk_g2s(sbase, glk, lk_bytes, &bars[0]);
     if (MATS) {
       mbar_expect_tx(&bars[1], cm_bytes);
@@ -1100,6 +1119,13 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
   const int r_e = i, r_o = Hd + i;
   float4* const eo = sE + 3 * h * HP + i;   // own half of the even / odd site in the work buffers
   float4* const oo = sO + 3 * h * HP + i;
+  // Links and matrices are constant; everything from here on may come from the previous launch.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (tid == 0) {
+    if (a.use_faces) stage_faces(a.faces);
+    // the next half-sweep may start (and stage its links and matrices) where SMs are free
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   __syncthreads();   // barriers initialised
 
   // Right-hand sides share the staged matrices; each has its own input, output and state.
@@ -1198,7 +1224,7 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
     __syncthreads();   // the staged faces have been read: the work buffers may be written
     for (int k = tid; k < 12 * ZERO_SLOTS; k += 2 * Hd)
       sE[(k / ZERO_SLOTS) * HP + Hd + k % ZERO_SLOTS] = make_float4(0.f, 0.f, 0.f, 0.f);
-    st_half3(oo, HP, t);
+    st_work(oo, HP, t);
     __syncthreads();
 
     // 2. even-odd preparation: rho = r_e + 1/2 H t_o
@@ -1210,7 +1236,7 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
         rho.c[s][c] = rho.c[s][c] + 0.5f * own.c[s][c];
         x.c[s][c] = mk(0.f, 0.f);
       }
-    st_half3(eo, HP, rho);
+    st_work(eo, HP, rho);
     __syncthreads();
 
     // 3. MR steps on the Schur complement
@@ -1220,7 +1246,7 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
       // odd sites: t = A_oo^{-1} H rho
       pair_hops<1, MT, H2>(g, q, sE, M, own);
       pair_block<MT, H2>(M, r_o, h, own, t);
-      st_half3(oo, HP, t);
+      st_work(oo, HP, t);
       __syncthreads();
       // even sites: p = A_ee rho - 1/4 H t
       pair_hops<0, MT, H2>(g, q, sO, M, own);
@@ -1266,7 +1292,7 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
       sp = __shfl_sync(0xffffffffu, sp, 0);
       const cx<float> alpha = sp > 0.f ? mk(sr / sp, si / sp) : mk(0.f, 0.f);
       const cx<float> ah = 0.5f * alpha;
-      ld_half3(oo, HP, t);   // this step's t of the own odd site
+      ld_work(oo, HP, t);   // this step's t of the own odd site
 #pragma unroll
       for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -1276,7 +1302,7 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
           dO.c[s][c] = cmac(dO.c[s][c], ah, t.c[s][c]);
         }
       if (it + 1 < a.i_domain) {
-        st_half3(eo, HP, rho);
+        st_work(eo, HP, rho);
         __syncthreads();
       }
     }
@@ -1293,8 +1319,8 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
 
     // 4. faces of delta for the next half-sweep (none after the very last one)
     if (!(a.last && (a.both_colours || colour == 1))) {
-      st_half3(eo, HP, x);
-      st_half3(oo, HP, dO);
+      st_work(eo, HP, x);
+      st_work(oo, HP, dO);
       __syncthreads();
       float4* const fw = a.faces_out + rhs * a.f_stride;
       pair_face_write<1, MT>(g, a.g, d, sE, fw, M);
@@ -1360,6 +1386,29 @@ __global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair_lattic
   sap_pair_body<__half, true, false, 0>(m.lat[l], blockIdx.x - m.first[l]);
 }
 
+// A half-sweep's blocks may start before the previous launch of the stream has ended: they stage
+// their links and matrices and wait (griddepcontrol.wait) before they touch anything else.
+// Launches of a few blocks are bound by such latencies: Schwarz on 8^4, 32 half-sweeps, 669 -> 572
+// us; FP32 storage on 16^3x32 323 -> 295 us; 32^3x64 1720 -> 1693 us by its last wave.  Early
+// blocks take the places that are free, which leaves the SMs unevenly loaded where a launch
+// fills a few of each SM's places once (256 blocks of 128 threads: 23.7 -> 28.6 us), so not there:
+// only with one block per SM, with half the SMs empty, or with at least two waves.
+static cudaLaunchAttribute overlapped_launch(int grid, int threads, size_t smem) {
+  static int sms = 0, per_sm = 0;
+  if (!sms) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  }
+  // 128 registers a thread; smem and 2 KB of shared memory a block
+  const int places = std::max(1, std::min((int)(per_sm / (smem + 2048)), 2 * SAP_MAX_THREADS / threads));
+  cudaLaunchAttribute a = {};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = places == 1 || 2 * grid <= sms || grid >= 2 * sms * places;
+  return a;
+}
+
 // One thread per site: the work vectors, and links and matrices when both fit.  Two threads
 // per site: the links always, the matrices when they fit beside them; the work buffers (with
 // their zero slots) share their space with the staged faces.
@@ -1397,7 +1446,15 @@ static void launch_shape(const SapArgs& a, int grid, size_t smem, cudaStream_t s
                          smem_optin() - 1024);
     configured = 1;
   }
-  sap_kernel_pair<MT, MATS, H2, SHAPE><<<grid, 2 * a.g.Hd, smem, st>>>(a);
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(2 * a.g.Hd);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute early = overlapped_launch(grid, 2 * a.g.Hd, smem);
+  c.attrs = &early;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, sap_kernel_pair<MT, MATS, H2, SHAPE>, a);
 }
 
 template <typename MT, bool MATS, bool H2 = false>
@@ -1452,7 +1509,15 @@ int sap_half_sweep_lattices(const Geom* gs, const SapState* Ss, int nlat, int co
     cudaFuncSetAttribute(sap_kernel_pair_lattices, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - 1024);
     configured = 1;
   }
-  sap_kernel_pair_lattices<<<total, 2 * gs[0].Hd, smem, st>>>(m);
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(total);
+  c.blockDim = dim3(2 * gs[0].Hd);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute early = overlapped_launch(total, 2 * gs[0].Hd, smem);
+  c.attrs = &early;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, sap_kernel_pair_lattices, m);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
