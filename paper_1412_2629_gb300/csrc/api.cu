@@ -357,9 +357,10 @@ static dd_status ensure_scratch(dd_ctx* c) {
   return DD_OK;
 }
 
-static dd_status apply_internal(dd_ctx* c, const void* in, void* out, int prec, const void* f = nullptr) {
+static dd_status apply_internal(dd_ctx* c, const void* in, void* out, int prec, const void* f = nullptr,
+                                const double2* in_norm2 = nullptr) {
   FieldView vi = view(c->g, (void*)in, prec), vo = view(c->g, out, prec), vf = view(c->g, (void*)f, prec);
-  launch_apply_A(c->g, gauge_view(c, prec), clover_view(c, prec), vi, vo, f ? &vf : nullptr, c->st);
+  launch_apply_A(c->g, gauge_view(c, prec), clover_view(c, prec), vi, vo, f ? &vf : nullptr, c->st, in_norm2);
   return launched(c);
 }
 
@@ -702,24 +703,31 @@ __global__ void restart_gate_kernel(int* flags, int want, const double2* nrm2, d
   flags[1] = (want && flags[0] == 0 && nrm2->x > tol2) ? 1 : 0;
 }
 
-// After the projection cp = V_{k+1}^H (r / rho): cp <- rho cp, and whether the deflated
-// restart keeps enough of r: |r - V_{k+1} cp| <= defl_tol |r|.  status[8..11] = |r|^2,
-// decision, the part of r that the projection misses, deflation status.
-__global__ void restart_decide_kernel(const int* flags, int want, int k, zd* cp, const double2* nrm2, double defl_tol,
-                                      double* status) {
+// cp = V_{k+1}^H r = P^H (V^H r) from the projection vr = V^H (r / rho) of the residual onto the
+// cycle's basis (mm + 1 vectors), and whether the deflated restart keeps enough of r:
+// |r - V_{k+1} cp| <= defl_tol |r|.  flags[2] gates the recombination, which a refused restart
+// does not need.  status[8..11] = |r|^2, decision, the part of r that the projection misses,
+// deflation status.  One block of at least k + 1 threads.
+__global__ void restart_decide_kernel(int* flags, int want, int mm, int k, const zd* P, int ldp, const zd* vr, zd* cp,
+                                      const double2* nrm2, double defl_tol, double* status) {
   const double rho2 = nrm2->x;
   int dec = 0;
   double miss = 1.0;
   if (want && flags[1]) {
     const double rho = sqrt(rho2);
-    double pc = 0;
-    for (int i = 0; i <= k; ++i) {
-      cp[i] = rho * cp[i];
-      pc += abs2(cp[i]);
+    if ((int)threadIdx.x <= k) {
+      zd t = Z(0.0);
+      for (int i = 0; i <= mm; ++i) t = t + conj(P[i + (long)threadIdx.x * ldp]) * vr[i];
+      cp[threadIdx.x] = rho * t;
     }
+    __syncthreads();
+    double pc = 0;
+    for (int i = 0; i <= k; ++i) pc += abs2(cp[i]);
     miss = sqrt(fmax(0.0, 1.0 - pc / rho2));
     dec = miss <= defl_tol ? 1 : 0;
   }
+  if (threadIdx.x) return;
+  flags[2] = dec;
   status[8] = rho2;
   status[9] = dec;
   status[10] = miss;
@@ -897,9 +905,17 @@ static GsTail gs_tail_of(const SolverBuffers& s, int stage) {
 
 // rho2 = |f - A x|^2 into s.nrm2 (device) and return it on the host (s: the context's own
 // solver buffers unless given).
-static dd_status true_residual(dd_ctx* c, double* rho2, SolverBuffers* sp = nullptr) {
+static dd_status true_residual(dd_ctx* c, double* rho2, SolverBuffers* sp = nullptr, bool initial = false) {
   SolverBuffers& s = sp ? *sp : c->sv;
-  TRY(apply_internal(c, s.x64, s.r64, P64, s.f64));
+  // a solve's first residual, usually of x = 0: its norm (one read of x) spares the operator
+  const double2* xnorm = nullptr;
+  if (initial) {
+    launch_norm2_64(s.x64, c->g.V * 12, s.partial, c->st);
+    launch_reduce_partials(s.partial, 1, s.nrm2 + 2, 0, c->st);
+    TRY(launched(c, 2));
+    xnorm = s.nrm2 + 2;
+  }
+  TRY(apply_internal(c, s.x64, s.r64, P64, s.f64, xnorm));
   launch_norm2_64(s.r64, c->g.V * 12, s.partial, c->st);
   launch_reduce_partials(s.partial, 1, s.nrm2, 0, c->st);
   TRY(launched(c, 2));
@@ -912,10 +928,12 @@ static dd_status true_residual(dd_ctx* c, double* rho2, SolverBuffers* sp = null
 
 // End of a cycle after mm Arnoldi steps, on the device: y from the least-squares problem;
 // the deflated restart's small dense step (one warp, on the second stream beside the
-// reliable update); x64 += Z y; r64 = f - A64 x64 and |r64|^2; then,
-// when the deflation succeeded and |r64| is still above target, V <- V P_{k+1} and
-// Z <- Z P_k in place and the projection of r64 onto the new V_{k+1}.  The one host read
-// returns |r64|^2 and whether the deflated restart keeps enough of r64.
+// reliable update); x64 += Z y; r64 = f - A64 x64 and |r64|^2; then, when the deflation
+// succeeded and |r64| is still above target, the projection of r64 onto V_{k+1} = V P_{k+1}, and
+// when it keeps enough of r64, V <- V P_{k+1} and Z <- Z P_k in place.  The one host read returns
+// |r64|^2 and that decision.  The projection is taken from V^H r64, so a restart that is
+// refused costs one read of V and not the recombination (24^3x48, m = 16, k = 6: 0.16 ms in
+// place of 0.78 ms).
 struct CycleEnd {
   double rho2 = 0, miss = 1;
   bool deflate = false;
@@ -948,25 +966,26 @@ static dd_status end_cycle(dd_ctx* c, SolverBuffers& s, int mm, const dd_solve_p
   restart_gate_kernel<<<1, 1, 0, c->st>>>(s.dflags, want, s.nrm2, tol2);
   nk++;
   if (want) {
+    const int* gate = s.dflags + 1;
+    launch_r64_to_v32(s.w, s.r64, n4, s.nrm2, c->st, gate);
+    nk += 2;
+    if (s.v16) nk += launch_gs_dot(s.V16, mm + 1, n4, s.w, s.partial, gate, 1, c->st, s.vscale);
+    else nk += launch_gs_dot(s.V, mm + 1, n4, s.w, s.partial, gate, 1, c->st, s.vscale);
+    launch_gs_reduce(s.partial, mm + 1, n4, (double2*)s.hA, gate, 1, c->st);
+  }
+  restart_decide_kernel<<<1, 64, 0, c->st>>>(s.dflags, want, mm, k, s.P, ldh, s.hA, s.cp, s.nrm2, defl_tol, s.status);
+  nk++;
+  if (want) {
     // V <- V P_{k+1}, Z <- Z P_k in place: every output element depends only on the inputs
     // at the same position, which its thread reads before writing
-    const int* gate = s.dflags + 1;
+    const int* gate = s.dflags + 2;
     if (s.v16)
       nk += launch_recombine(s.V16, s.V16, mm + 1, k + 1, n4, (const double2*)s.P, ldh, c->st, gate, s.vscale,
                              s.v16_scale);
     else
       nk += launch_recombine(s.V, s.V, mm + 1, k + 1, n4, (const double2*)s.P, ldh, c->st, gate, s.vscale);
     nk += launch_recombine(s.Z, s.Z, mm, k, n4, (const double2*)s.P, ldh, c->st, gate);
-    launch_r64_to_v32(s.w, s.r64, n4, s.nrm2, c->st, gate);
-    if (s.v16)
-      nk += 1 + launch_gs_dot(s.V16, k + 1, n4, s.w, s.partial, gate, 1, c->st, s.vscale);
-    else
-      nk += 1 + launch_gs_dot(s.V, k + 1, n4, s.w, s.partial, gate, 1, c->st);
-    launch_gs_reduce(s.partial, k + 1, n4, (double2*)s.cp, gate, 1, c->st);
-    nk++;
   }
-  restart_decide_kernel<<<1, 1, 0, c->st>>>(s.dflags, want, k, s.cp, s.nrm2, defl_tol, s.status);
-  nk++;
   TRY(launched(c, nk));
   TRY(cuda_check(c, cudaMemcpyAsync(s.h_status, s.status + 8, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->st),
                  "restart status"));
@@ -1132,7 +1151,7 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
     return launched(c, 4);
   };
 
-  TRY(true_residual(c, &rho2));
+  TRY(true_residual(c, &rho2, nullptr, true));
   reliable++;
   double rel = sqrt(rho2) / nf;
   if (!isfinite(rel)) rc = fail(c, DD_ERR_NONFINITE, "non-finite residual");
@@ -1323,8 +1342,8 @@ static dd_status ensure_lock(dd_ctx* c, int nrhs, int m) {
     if (c->h_lock_ptrs) cudaFreeHost(c->h_lock_ptrs);
     c->lock_ptrs = nullptr;
     c->h_lock_ptrs = nullptr;
-    TRY(dalloc(c, &c->lock_ptrs, 3 * (size_t)nrhs * sizeof(void*)));
-    if (cudaMallocHost(&c->h_lock_ptrs, 3 * (size_t)nrhs * sizeof(void*)) != cudaSuccess)
+    TRY(dalloc(c, &c->lock_ptrs, 4 * (size_t)nrhs * sizeof(void*)));
+    if (cudaMallocHost(&c->h_lock_ptrs, 4 * (size_t)nrhs * sizeof(void*)) != cudaSuccess)
       return fail(c, DD_ERR_OOM, "pinned pointer lists");
     c->lock_cap = nrhs;
   }
@@ -1332,13 +1351,16 @@ static dd_status ensure_lock(dd_ctx* c, int nrhs, int m) {
 }
 
 // z_r = M v_r for na right-hand sides given by device pointer lists.
-static dd_status sap_run_list(dd_ctx* c, const float4* const* vl, float4* const* zl, const dd_sap_params* p, int na) {
+// The inputs are the stored v_r times *vs[r].
+static dd_status sap_run_list(dd_ctx* c, const float4* const* vl, float4* const* zl, const float* const* vs,
+                              const dd_sap_params* p, int na) {
   int prec = sap_prec(p->storage_prec);
   TRY(ensure_sap(c, prec, na));
   if (p->additive) TRY(ensure_faces2(c, prec));
   SapState S = sap_state(c, prec, p, na);
   S.vlist = vl;
   S.zlist = zl;
+  S.vscales = vs;
   return sap_sweeps(c, S, p, nullptr, nullptr, c->sap[prec].faces2);
 }
 
@@ -1348,18 +1370,27 @@ static dd_status lock_gs(dd_ctx* c, SolverBuffers& s, int j, int m) {
   const long long n4 = c->g.V * 6;
   const int ldh = m + 1;
   float4* vn = s.V + (long long)(j + 1) * n4;
-  int nk = launch_gs_dot(s.V, j + 1, n4, s.w, s.partial, nullptr, 0, c->st);
+  const float* sc = s.vscale;
+  int nk = launch_gs_dot(s.V, j + 1, n4, s.w, s.partial, nullptr, 0, c->st, sc);
   launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
-  const int nb = launch_gs_project_dot(vn, s.w, s.V, j + 1, n4, (const double2*)s.hA, nullptr, s.partial, s.partial2,
+  const int nb = launch_gs_project_dot(vn, s.w, s.V, j + 1, n4, (const double2*)s.hA, sc, s.partial, s.partial2,
                                        c->sap_err, c->st, gs_tail_of(s, 1));
   launch_gs_reduce_blocks(s.partial, j + 1, nb, (double2*)s.hB, s.flag, 1, c->st);
-  launch_gs_project(vn, vn, s.V, j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, nullptr,
+  launch_gs_project(vn, vn, s.V, j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc,
                     gs_tail_of(s, 2));
-  launch_scale_inplace(vn, n4, s.nu2, c->st);
-  arnoldi_finish_kernel<<<1, 1, 0, c->st>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status);
+  // the Hessenberg column and its Givens update (one thread) run beside the next right-hand side;
+  // lock_join makes the context's stream wait for them
+  cudaEventRecord(s.ev_fork, c->st);
+  cudaStreamWaitEvent(s.side, s.ev_fork, 0);
+  arnoldi_finish_kernel<<<1, 1, 0, s.side>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status);
+  set_vscale_kernel<<<1, 1, 0, c->st>>>(s.vscale + j + 1, s.nu2);
   TRY(launched(c, nk + 6));
-  return cuda_check(c, cudaMemcpyAsync(s.h_status, s.status, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->st),
-                    "status");
+  TRY(cuda_check(c, cudaMemcpyAsync(s.h_status, s.status, 4 * sizeof(double), cudaMemcpyDeviceToHost, s.side),
+                 "status"));
+  return cuda_check(c, cudaEventRecord(s.ev_join, s.side), "status");
+}
+static dd_status lock_join(dd_ctx* c, SolverBuffers& s) {
+  return cuda_check(c, cudaStreamWaitEvent(c->st, s.ev_join, 0), "status");
 }
 
 // End of a cycle of one right-hand side after mm Arnoldi steps: x64 += Z y, FP64 residual,
@@ -1438,7 +1469,7 @@ static dd_status solve_lockstep(dd_ctx* c, const double* f, double* x, int nrhs,
       continue;
     }
     R[r].nf = sqrt(h.x);
-    TRY(true_residual(c, &R[r].rho2, &s));
+    TRY(true_residual(c, &R[r].rho2, &s, true));
     R[r].reliable++;
     R[r].rel = sqrt(R[r].rho2) / R[r].nf;
     if (!isfinite(R[r].rel)) {
@@ -1467,17 +1498,20 @@ static dd_status solve_lockstep(dd_ctx* c, const double* f, double* x, int nrhs,
       hp[i] = s.V + (long long)R[act[i]].j * n4;
       hp[na + i] = s.Z + (long long)R[act[i]].j * n4;
       hp[2 * na + i] = s.w;
+      hp[3 * na + i] = s.vscale + R[act[i]].j;
     }
-    TRY(cuda_check(c, cudaMemcpyAsync(c->lock_ptrs, hp, 3 * (size_t)na * sizeof(void*), cudaMemcpyHostToDevice, c->st),
+    TRY(cuda_check(c, cudaMemcpyAsync(c->lock_ptrs, hp, 4 * (size_t)na * sizeof(void*), cudaMemcpyHostToDevice, c->st),
                    "pointer lists"));
     cudaEventRecord(e0, c->st);
-    TRY(sap_run_list(c, vl, (float4* const*)(c->lock_ptrs + na), &p->sap, na));
+    TRY(sap_run_list(c, vl, (float4* const*)(c->lock_ptrs + na), (const float* const*)(c->lock_ptrs + 3 * na), &p->sap,
+                     na));
     cudaEventRecord(e1, c->st);
     launch_apply_A_multi_list(g, gauge_view(c, P32), clover_view(c, P32), (const float4* const*)(c->lock_ptrs + na),
                               (float4* const*)(c->lock_ptrs + 2 * na), na, c->st);
     TRY(launched(c));
     cudaEventRecord(e2, c->st);
     for (int r : act) TRY(lock_gs(c, c->lock[r], R[r].j, m));
+    for (int r : act) TRY(lock_join(c, c->lock[r]));
     cudaEventRecord(e3, c->st);
     TRY(cuda_check(c, cudaStreamSynchronize(c->st), "lockstep step"));
     float ms;
@@ -1607,7 +1641,7 @@ static dd_status solve_lattices(dd_ctx** ctxs, int nlat, const double* const* f,
         continue;
       }
       Q.nf = sqrt(h.x);
-      TRY(true_residual(c, &Q.rho2, &s));
+      TRY(true_residual(c, &Q.rho2, &s, true));
       Q.reliable++;
       Q.rel = sqrt(Q.rho2) / Q.nf;
       if (!isfinite(Q.rel)) {
@@ -1644,13 +1678,15 @@ static dd_status solve_lattices(dd_ctx** ctxs, int nlat, const double* const* f,
         hp[i] = s.V + (long long)R[l][act[l][i]].j * n4;
         hp[na + i] = s.Z + (long long)R[l][act[l][i]].j * n4;
         hp[2 * na + i] = s.w;
+        hp[3 * na + i] = s.vscale + R[l][act[l][i]].j;
       }
-      TRY(cuda_check(c, cudaMemcpyAsync(c->lock_ptrs, hp, 3 * (size_t)na * sizeof(void*), cudaMemcpyHostToDevice, st),
+      TRY(cuda_check(c, cudaMemcpyAsync(c->lock_ptrs, hp, 4 * (size_t)na * sizeof(void*), cudaMemcpyHostToDevice, st),
                      "pointer lists"));
       gs[nl] = c->g;
       Ss[nl] = sap_state(c, P16, &p->sap, na);
       Ss[nl].vlist = (const float4* const*)c->lock_ptrs;
       Ss[nl].zlist = (float4* const*)(c->lock_ptrs + na);
+      Ss[nl].vscales = (const float* const*)(c->lock_ptrs + 3 * na);
       lat_of[nl++] = l;
     }
     if (!total) break;
@@ -1675,6 +1711,8 @@ static dd_status solve_lattices(dd_ctx** ctxs, int nlat, const double* const* f,
     cudaEventRecord(e2, st);
     for (int l = 0; l < nlat; ++l)
       for (int r : act[l]) TRY(lock_gs(ctxs[l], ctxs[l]->lock[r], R[l][r].j, m));
+    for (int l = 0; l < nlat; ++l)
+      for (int r : act[l]) TRY(lock_join(ctxs[l], ctxs[l]->lock[r]));
     cudaEventRecord(e3, st);
     TRY(cuda_check(c0, cudaStreamSynchronize(st), "lockstep step"));
     float ms;
@@ -1873,7 +1911,7 @@ static dd_status solve_gcr_one(dd_ctx* c, const dd_solve_params* p, double nf2, 
   float4* r = s.w;
   float4* wk = s.V + (long long)m * n4;   // the (m+1)-th basis slot: the new direction
   zd* alpha = s.y;                          // m + 2 entries
-  TRY(true_residual(c, &rho2));
+  TRY(true_residual(c, &rho2, nullptr, true));
   reliable++;
   double rel = sqrt(rho2) / nf;
   if (!isfinite(rel)) rc = fail(c, DD_ERR_NONFINITE, "non-finite residual");

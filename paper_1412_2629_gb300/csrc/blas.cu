@@ -210,32 +210,52 @@ void launch_r64_to_v32(float4* v, const double2* r, long long n4, const double2*
 // RU independent input loads per thread, which is what keeps HBM busy here.  out may be
 // V itself (in-place recombination): a thread reads all inputs at q before it writes
 // the outputs at q, and no other thread touches q.
+// Bound by issue and shared-memory reads of the coefficients as much as by HBM: in packed FP32
+// multiply-adds 41 -> 9 vectors of 32^3x64 take 2.38 ms (4.2 TB/s), in scalar ones 3.66 ms.
 constexpr int RBT = 128, RU = 8;
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
 template <int NO, typename VT>
 __global__ void __launch_bounds__(RBT) recombine_kernel(VT* out, const VT* V, int nv, int l0, long long n4,
                                                         const double2* P, int ldp, const int* gate,
                                                         const float* vscale, float oscale) {
   if (gate && *gate != 1) return;
-  __shared__ float2 ps[64][NO];
+  __shared__ float4 ps[64][NO];   // coefficients, each part twice: (re, re, im, im)
   for (int t = threadIdx.x; t < nv * NO; t += RBT) {
     int i = t / NO, l = t % NO;
     const double2 c = P[i + (long long)(l0 + l) * ldp];
     const double sc = vscale ? (double)vscale[i] : 1.0;   // stored V_i = v_i / vscale[i]
-    ps[i][l] = make_float2((float)(c.x * sc), (float)(c.y * sc));
+    const float cr = (float)(c.x * sc), ci = (float)(c.y * sc);
+    ps[i][l] = make_float4(cr, cr, ci, ci);
   }
   __syncthreads();
   for (long long q = blockIdx.x * (long long)RBT + threadIdx.x; q < n4; q += (long long)gridDim.x * RBT) {
-    float4 a[NO];
+    // packed FP32 multiply-adds: (re, im) += cr (v.re, v.im) + ci (-v.im, v.re), four issue slots
+    // for an input and an output instead of twelve
+    unsigned long long a[NO][2];
 #pragma unroll
-    for (int l = 0; l < NO; ++l) a[l] = make_float4(0, 0, 0, 0);
+    for (int l = 0; l < NO; ++l) a[l][0] = a[l][1] = 0;
     auto fma_in = [&](int i, float4 v) {
+      const unsigned long long v0 = pack2(v.x, v.y), v1 = pack2(v.z, v.w), w0 = pack2(-v.y, v.x), w1 = pack2(-v.w, v.z);
 #pragma unroll
       for (int l = 0; l < NO; ++l) {
-        float2 c = ps[i][l];
-        a[l].x += c.x * v.x - c.y * v.y;
-        a[l].y += c.x * v.y + c.y * v.x;
-        a[l].z += c.x * v.z - c.y * v.w;
-        a[l].w += c.x * v.w + c.y * v.z;
+        const float4 c = ps[i][l];
+        const unsigned long long cr = pack2(c.x, c.y), ci = pack2(c.z, c.w);
+        a[l][0] = fma2(ci, w0, fma2(cr, v0, a[l][0]));
+        a[l][1] = fma2(ci, w1, fma2(cr, v1, a[l][1]));
       }
     };
     int i = 0;
@@ -248,7 +268,10 @@ __global__ void __launch_bounds__(RBT) recombine_kernel(VT* out, const VT* V, in
     }
     for (; i < nv; ++i) fma_in(i, ldv(V, (long long)i * n4 + q));
 #pragma unroll
-    for (int l = 0; l < NO; ++l) stv(out, (long long)(l0 + l) * n4 + q, a[l], oscale);
+    for (int l = 0; l < NO; ++l) {
+      const float2 lo = unpack2(a[l][0]), hi = unpack2(a[l][1]);
+      stv(out, (long long)(l0 + l) * n4 + q, make_float4(lo.x, lo.y, hi.x, hi.y), oscale);
+    }
   }
 }
 

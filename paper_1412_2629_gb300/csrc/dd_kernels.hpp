@@ -44,9 +44,10 @@ void launch_apply_A_multi(const Geom& g, GaugeView U, CloverView C, FieldView in
 void launch_apply_A_multi_list(const Geom& g, GaugeView U, CloverView C, const float4* const* in,
                                float4* const* out, int nrhs, cudaStream_t st);
 // out = A in, or out = f - A in when f != nullptr.  FP64 and FP32 fields use the matching
-// gauge/clover precision; FP16 fields use FP16 gauge/clover and FP32 arithmetic.
+// gauge/clover precision; FP16 fields use FP16 gauge/clover and FP32 arithmetic.  in_norm2 (FP64
+// residuals; device): |in|^2, and out = f without the operator where it is zero.
 void launch_apply_A(const Geom& g, GaugeView U, CloverView C, FieldView in, FieldView out, const FieldView* f,
-                    cudaStream_t st);
+                    cudaStream_t st, const double2* in_norm2 = nullptr);
 
 // out = A in on canonical FP64 or FP32 fields, 16-byte aligned and not overlapping.
 void launch_apply_A_canonical(const Geom& g, GaugeView U, CloverView C, const void* in, void* out, int prec,
@@ -81,6 +82,7 @@ struct SapState {
   float4* faces_out = nullptr;
   // single right-hand side: the input is v * (*vscale) (device scalar), when set
   const float* vscale = nullptr;
+  const float* const* vscales = nullptr;   // the same for the inputs of vlist (device array)
 };
 // One half-sweep: all domains of `colour`.  first: the residual is the input v (both
 // parities) and u = 0; use_faces: subtract the couplings to the other colour from the

@@ -39,10 +39,17 @@ __device__ inline void hop_pair(const Geom& g, const Site& st, long long s, cons
 
 template <typename T>
 __global__ void __launch_bounds__(256) apply_A_kernel(Geom g, LinkPtr<T> U, CloverPtr<T> C, SpinorPtr<T> in,
-                                                       SpinorPtr<T> out, SpinorPtr<T> f, int residual) {
+                                                       SpinorPtr<T> out, SpinorPtr<T> f, int residual,
+                                                       const double2* in_norm2) {
   typedef typename Arith<T>::type R;
   long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (s >= g.V) return;
+  if (in_norm2 && in_norm2->x == 0.0) {   // f - A 0
+    Spinor<R> fv;
+    f.load(g, s, fv);
+    out.store(g, s, fv);
+    return;
+  }
   Site st = decode(g, s);
   Spinor<R> hop;
   zero(hop);
@@ -129,7 +136,7 @@ static int block_threads(long long V, int most) {
 }
 
 void launch_apply_A(const Geom& g, GaugeView U, CloverView C, FieldView in, FieldView out, const FieldView* f,
-                    cudaStream_t st) {
+                    cudaStream_t st, const double2* in_norm2) {
   const int nt = block_threads(g.V, in.prec == P64 ? 64 : 256);
   const unsigned nb = (unsigned)((g.V + nt - 1) / nt);
   int res = f != nullptr;
@@ -146,19 +153,19 @@ void launch_apply_A(const Geom& g, GaugeView U, CloverView C, FieldView in, Fiel
     apply_A_kernel<double><<<nb, nt, 0, st>>>(g, LinkPtr<double>{(const double2*)U.links},
                                                CloverPtr<double>{(const double2*)C.m},
                                                SpinorPtr<double>{(double2*)in.data},
-                                               SpinorPtr<double>{(double2*)out.data}, fi, res);
+                                               SpinorPtr<double>{(double2*)out.data}, fi, res, res ? in_norm2 : nullptr);
   } else if (in.prec == P32) {
     SpinorPtr<float> fi{res ? (float4*)f->data : nullptr};
     apply_A_kernel<float><<<nb, nt, 0, st>>>(g, LinkPtr<float>{(const float2*)U.links},
                                               CloverPtr<float>{(const float4*)C.m},
                                               SpinorPtr<float>{(float4*)in.data}, SpinorPtr<float>{(float4*)out.data},
-                                              fi, res);
+                                              fi, res, nullptr);
   } else {
     SpinorPtr<__half> fi{res ? (uint4*)f->data : nullptr, res ? f->norm : nullptr};
     apply_A_kernel<__half><<<nb, nt, 0, st>>>(g, LinkPtr<__half>{(const uint4*)U.links},
                                                CloverPtr<__half>{(const uint4*)C.m},
                                                SpinorPtr<__half>{(uint4*)in.data, in.norm},
-                                               SpinorPtr<__half>{(uint4*)out.data, out.norm}, fi, res);
+                                               SpinorPtr<__half>{(uint4*)out.data, out.norm}, fi, res, nullptr);
   }
 }
 

@@ -324,6 +324,7 @@ struct SapArgs {
   const float4* v;
   float4* z;
   const float* vscale;   // if set: the input is v * (*vscale) (a basis vector stored unnormalised)
+  const float* const* vscales;   // the same for the inputs of vptr
   const float4* const* vptr;   // if set: input / output of right-hand side r at vptr[r] / zptr[r]
   float4* const* zptr;
   int* err;
@@ -1143,8 +1144,8 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
       const float4* v = (a.vptr ? a.vptr[rhs] : a.v + rhs * a.v_stride) + d * 6 * Vd + 3 * h * Vd;
       ld_half3(v + r_e, Vd, rho);
       ld_half3(v + r_o, Vd, dO);
-      if (a.vscale) {
-        const float sc = *a.vscale;
+      if (a.vscale || a.vscales) {
+        const float sc = a.vscales ? *a.vscales[rhs] : *a.vscale;
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -1525,7 +1526,7 @@ int sap_half_sweep(const Geom& g, const SapState& S, int colour, int first, int 
                    const float4* v, float4* z, int i_domain, cudaStream_t st) {
   if (g.Hd > SAP_MAX_THREADS || (g.Hd & 31)) return -1;
   // only the pair kernel loops over right-hand sides and reads pointer lists
-  if ((S.nrhs > 1 || S.vlist) && S.threads_per_site != 2) return -1;
+  if ((S.nrhs > 1 || S.vlist || S.vscales) && S.threads_per_site != 2) return -1;
   if (S.both_colours && S.threads_per_site != 2) return -1;   // the additive form: pair kernel only
   SapArgs a = make_args(g, S, colour, first, use_faces, last, v, z, i_domain);
   int grid = S.both_colours ? g.ND : g.ND / 2;
@@ -1566,6 +1567,7 @@ static SapArgs make_args(const Geom& g, const SapState& S, int colour, int first
   a.v = v;
   a.z = z;
   a.vscale = S.vscale;
+  a.vscales = S.vscales;
   a.vptr = S.vlist;
   a.zptr = S.zlist;
   a.err = S.err;
