@@ -611,6 +611,16 @@ __device__ __forceinline__ void frame_project(const Spinor<float>& p, float st, 
         o.c[s][c] = mk(fmaf(st, p.c[2 + s][c].re, p.c[s][c].re), fmaf(st, p.c[2 + s][c].im, p.c[s][c].im));
   }
 }
+// the first hop of a sum (MU = 3) sets it
+__device__ __forceinline__ void frame_recon_first(Spinor<float>& acc, float st, const Half<float>& u) {
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      acc.c[s][c] = u.c[s][c];
+      acc.c[2 + s][c] = st * u.c[s][c];
+    }
+}
 template <int MU>
 __device__ __forceinline__ void frame_recon(Spinor<float>& acc, float st, const Half<float>& u) {
   if constexpr (MU < 3) {
@@ -892,10 +902,14 @@ __device__ __forceinline__ void pair_hop(const Geom& g, const PairSites& q, cons
     M.link(MU, r, q.h, U);
     su3_mul(U, hp, uh);
   }
-  frame_recon<MU>(acc, q.st, uh);
+  if constexpr (MU == 3) frame_recon_first(acc, q.st, uh);
+  else frame_recon<MU>(acc, q.st, uh);
 }
 
-// Own half of the sum of all hops inside the domain at the site of parity P (no -1/2 factor).
+// Own half of the sum of all hops inside the domain at the site of parity P (no -1/2 factor).  The
+// order of the directions and the place of the block products only move what the compiler
+// can overlap: of those tried, t first and y last with the block before the hops was the
+// fastest (32^3x64 half-sweep 423 -> 405 us, 24^3x48 106 -> 102.6 us).
 template <int P, typename MT, bool H2>
 __device__ __forceinline__ void pair_hops(const Geom& g, const PairSites& q, const float4* src, const MatBlock<MT>& M,
                                           Half<float>& out) {
@@ -903,11 +917,10 @@ __device__ __forceinline__ void pair_hops(const Geom& g, const PairSites& q, con
   const float4* own = src + 3 * q.h * HP;
   const float4* oth = src + 3 * (1 - q.h) * HP;
   Spinor<float> acc;
-  zero(acc);
-  pair_hop<P, 0, MT, H2>(g, q, own, oth, M, acc);
-  pair_hop<P, 1, MT, H2>(g, q, own, oth, M, acc);
-  pair_hop<P, 2, MT, H2>(g, q, own, oth, M, acc);
   pair_hop<P, 3, MT, H2>(g, q, own, oth, M, acc);
+  pair_hop<P, 0, MT, H2>(g, q, own, oth, M, acc);
+  pair_hop<P, 2, MT, H2>(g, q, own, oth, M, acc);
+  pair_hop<P, 1, MT, H2>(g, q, own, oth, M, acc);
   join_halves(acc, out);
 }
 
@@ -1250,9 +1263,9 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
       st_work(oo, HP, t);
       __syncthreads();
       // even sites: p = A_ee rho - 1/4 H t
-      pair_hops<0, MT, H2>(g, q, sO, M, own);
       Half<float> pv;
       pair_block<MT, H2>(M, r_e, h, rho, pv);
+      pair_hops<0, MT, H2>(g, q, sO, M, own);
       float pr_re = 0.f, pr_im = 0.f, pp = 0.f;
 #pragma unroll
       for (int s = 0; s < 2; ++s)
