@@ -527,7 +527,8 @@ def main():
     fp32_units = props.multi_processor_count * 128 * 2 * sm_max * 1e6 / 1e12
     # the Schwarz kernel runs inside a seconds-long solve: the sustained FFMA figure
     fp32_peak = peak_sust
-    sap_sha = src_sha(["paper_1412_2629_gb300/csrc/sap.cu", "paper_1412_2629_gb300/csrc/dd_common.cuh"])
+    sap_sha = src_sha(["paper_1412_2629_gb300/csrc/sap.cu", "paper_1412_2629_gb300/csrc/dd_common.cuh",
+                       "paper_1412_2629_gb300/csrc/dd_tma.cuh"])
     dsl_sha = src_sha(["paper_1412_2629_gb300/csrc/dslash.cu", "paper_1412_2629_gb300/csrc/dd_common.cuh"])
     sap_traffic = read_profile("sap_kernel_32x64.txt", sap_sha)
     # full operator inside the solve: one FP32 application per outer iteration
@@ -671,7 +672,7 @@ def kernel_case(args, local):
     else:
         # per right-hand side the batch reads the links and clover once per pair
         per_site = dslash_bytes_per_site("fp32") if nr == 1 else (72 + 72) * 4 / 2 + 48 * 4
-        out = {"case": fp32_operator_kernel(w.domain) if nr == 1 else "apply_A_multi_kernel<float,2>", "nrhs": nr,
+        out = {"case": fp32_operator_kernel(w.domain) if nr == 1 else "apply_A_multi_kernel<float>", "nrhs": nr,
                "lattice": dims, "launch_ms": 1e3 * launch_s,
                "ms_per_rhs": 1e3 * launch_s / nr,
                "gbs_algorithmic": per_site * V * nr / launch_s / 1e9}

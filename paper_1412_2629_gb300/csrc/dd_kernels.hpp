@@ -65,7 +65,7 @@ struct SapState {
   float* u_norm;
   float4* faces;       // projected half-spinors on the 8 faces of every domain (FP32)
   int* err;            // set to 1 when a bounded device wait runs out
-  bool mat_in_smem;    // stage links and Schwarz matrices in shared memory
+  bool mat_in_smem;    // the Schwarz matrices fit into shared memory beside the links
   int threads_per_site = 2;   // 1: one thread per site; 2: hop directions and chirality split
   bool inject_wait_timeout = false;   // test hook: make the bounded wait run out (no fault)
   int nrhs = 1;                // right-hand sides in one launch (their buffers follow each other)

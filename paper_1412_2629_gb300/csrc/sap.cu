@@ -14,14 +14,14 @@
 // D_eo, D_oe are the hops inside the domain with factor -1/2; A_ee is the clover block
 // (diagonal 1/(2 kappa) included), A_oo^{-1} its per-site inverse.
 //
-// Data movement.  The domain's links and Schwarz matrices (clover on even sites,
-// inverse on odd sites) form contiguous blocks in HBM; when they fit, one thread
-// stages both into shared memory with bulk asynchronous copies (TMA engine,
-// completion on an mbarrier) while the others load the residual.  The even-site and
-// odd-site work vectors live in shared memory as FP32; the thread for local index i
-// owns even site i and odd site i and keeps x, rho and r_o in registers, so every MR
-// step runs on chip.  The MR inner products are reduced with warp shuffles and one
-// exchange through shared memory.
+// Data movement.  The domain's links and Schwarz matrices (clover on even sites, inverse on
+// odd sites) form contiguous blocks in HBM, and so does each face of a neighbouring domain;
+// all of them are staged into shared memory with bulk asynchronous copies (TMA engine,
+// completion on mbarriers) while the threads load the residual.  The even-site and odd-site
+// work vectors live in shared memory as FP32; x, rho and the odd solution stay in registers,
+// so every MR step runs on chip.  The MR inner products are reduced with warp shuffles and
+// one exchange through shared memory.  There are two kernels: one thread per site
+// (sap_kernel) and the default with two (sap_kernel_pair).
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
@@ -593,9 +593,11 @@ __global__ void __launch_bounds__(SAP_MAX_THREADS, 1) sap_kernel(SapArgs a) {
 // partial sums exchanged through shared memory, faces read site by site from global memory):
 // half-sweep of 32^3x64 (8x4x4x4 domains, I_domain 4, FP16 storage) 571 -> 430 us, of 24^3x48
 // (4^4, I_domain 3) 162 -> 112 us, FP32 storage 32^3x64 679 -> 474 us; 12.0k -> 10.0k cycles and
-// 2029 -> 1860 instructions per warp and MR step, 28k -> 21k cycles a visit outside them.
-// Bound by instruction issue (74 % in the MR steps; FMA pipe 48 %, shared memory 53 %) and by
-// the latency of staging and output with one CTA per SM.
+// 2029 -> 1860 instructions per warp and MR step, 28k -> 21k cycles a visit outside them (405,
+// 103 and 469 us with the launches overlapped and the order inside a phase chosen, below).
+// Bound by instruction issue and shared-memory wavefronts together (74 % and 63 % busy in the MR
+// steps) and by the latency of staging and output with one CTA per SM.  Cheaper arithmetic
+// alone does not help: SU(3) products in packed FP32 multiply-adds measured 445 us.
 
 constexpr int ZERO_SLOTS = 8;
 
@@ -1377,9 +1379,9 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
   }
 }
 
-// One CTA per domain (measured faster on GB300 than a persistent grid walking its domains
-// with the next domain's copies in flight: the round-robin tail and the extra live state
-// cost more than the overlap gains).
+// One CTA per domain.  A persistent grid that walks its domains, each one's copies issued as the
+// previous one's buffers fall free, measured the same on 32^3x64 (430 us) and slower on 24^3x48
+// (117 instead of 112 us): its loop state spills what the copies gain.
 template <typename MT, bool MATS, bool H2, int SHAPE>
 __global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair(const __grid_constant__ SapArgs a) {
   sap_pair_body<MT, MATS, H2, SHAPE>(a, blockIdx.x);
