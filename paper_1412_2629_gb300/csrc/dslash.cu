@@ -372,37 +372,61 @@ __device__ __forceinline__ void apply_A_multi_site(const Geom& g, long long s, i
   }
 }
 
-// Blocks that work on the same 128 sites with other fields are neighbours in launch order, so
-// the links and clover blocks come from HBM once and from L2 afterwards; a field left over
-// from the pairs runs alone.  Bound by the latency of the neighbours' loads (L1 and L2): three
-// blocks per SM at 168 registers, with a few spilled, beat two at 255 and four at 128 (six
-// fields of 24^3x48: 355, 430 and 377 us), and three fields per thread gain nothing over two.
-// The domain shape as compile-time constants and the launch order took six fields
-// from 541 to 349 us (169 us of traffic).
-constexpr int MULTI_NR = 2, MULTI_THREADS = 128;
+// Blocks that work on the same 128 sites with other pairs of fields are neighbours in launch order,
+// so the links and clover blocks come from HBM once and from L2 afterwards.  Bound by the latency
+// of the neighbours' loads (L1 and L2): three blocks per SM at 168 registers, with a few spilled,
+// beat two at 255 and four at 128 (six fields of 24^3x48: 355, 430 and 377 us; with 4x4x4x8
+// domains, whose shape is not compiled in, three and two blocks: 434 and 541 us), and three
+// fields per thread gain nothing over two.  The domain shape as compile-time constants and the
+// launch order took six fields from 541 to 349 us (169 us of traffic).
+//
+// A field left over from the pairs runs alone, in blocks behind all pairs.  Between the pairs of
+// the same sites its code and theirs, both fully unrolled, evict each other from the instruction
+// caches (8.0 warps waiting for instructions per issue, against 0.7): three FP16 fields of 24^3x48
+// 352 us (4x4x4x8 domains 435), behind the pairs 189 (226); FP32 226 (400) and 216 (293) us; 13
+// FP32 fields of 16^3x32, which gain from the links they share, 149 and 155 us.
+//
+// Both forms below number blocks and fields alike.  Where the compiler knows the shape, the
+// field number as an expression of each branch is 2 % faster (six FP32 fields 344 for 351 us);
+// where it does not, one computed before the branch spills less (429 for 451 us).
+constexpr int MULTI_THREADS = 128;
 template <typename T, int SHAPE>
 __global__ void __launch_bounds__(MULTI_THREADS, 3)
     apply_A_multi_kernel(Geom g0, LinkPtr<T> U, CloverPtr<T> C, SpinorPtr<T> in, SpinorPtr<T> out, long long unit_stride,
-                         long long norm_stride, int nrhs, int groups, const float4* const* in_list,
+                         long long norm_stride, int nrhs, unsigned site_blocks, const float4* const* in_list,
                          float4* const* out_list) {
   const Geom g = fixed_shape<SHAPE>(g0);
-  const long long s = (blockIdx.x / groups) * (long long)MULTI_THREADS + threadIdx.x;
-  if (s >= g.V) return;
-  const int r0 = (blockIdx.x % groups) * MULTI_NR;
-  if (r0 + 1 < nrhs)
-    apply_A_multi_site<T, 2>(g, s, r0, U, C, in, out, unit_stride, norm_stride, in_list, out_list);
-  else
-    apply_A_multi_site<T, 1>(g, s, r0, U, C, in, out, unit_stride, norm_stride, in_list, out_list);
+  const unsigned pairs = (unsigned)nrhs >> 1, paired = site_blocks * pairs;   // pairs of fields, their blocks
+  if constexpr (SHAPE != 0) {
+    const bool alone = blockIdx.x >= paired;
+    const unsigned b = alone ? blockIdx.x - paired : blockIdx.x / pairs;
+    const long long s = b * (long long)MULTI_THREADS + threadIdx.x;
+    if (s >= g.V) return;
+    if (alone)
+      apply_A_multi_site<T, 1>(g, s, 2 * pairs, U, C, in, out, unit_stride, norm_stride, in_list, out_list);
+    else
+      apply_A_multi_site<T, 2>(g, s, 2 * (blockIdx.x % pairs), U, C, in, out, unit_stride, norm_stride, in_list, out_list);
+  } else {
+    const bool pair = blockIdx.x < paired;
+    const unsigned per = pair ? pairs : 1u, x = pair ? blockIdx.x : blockIdx.x - paired;
+    const long long s = (x / per) * (long long)MULTI_THREADS + threadIdx.x;
+    if (s >= g.V) return;
+    const int r0 = pair ? (x % per) * 2 : nrhs - 1;
+    if (r0 + 1 < nrhs)
+      apply_A_multi_site<T, 2>(g, s, r0, U, C, in, out, unit_stride, norm_stride, in_list, out_list);
+    else
+      apply_A_multi_site<T, 1>(g, s, r0, U, C, in, out, unit_stride, norm_stride, in_list, out_list);
+  }
 }
 
 template <typename T>
 static void multi_launch(const Geom& g, LinkPtr<T> U, CloverPtr<T> C, SpinorPtr<T> in, SpinorPtr<T> out,
                          long long unit_stride, long long norm_stride, int nrhs, const float4* const* in_list,
                          float4* const* out_list, cudaStream_t st) {
-  const int groups = (nrhs + MULTI_NR - 1) / MULTI_NR;
-  const unsigned nb = (unsigned)((g.V + MULTI_THREADS - 1) / MULTI_THREADS) * groups;
+  const unsigned nb = (unsigned)((g.V + MULTI_THREADS - 1) / MULTI_THREADS);
   auto launch = [&](auto kernel) {
-    kernel<<<nb, MULTI_THREADS, 0, st>>>(g, U, C, in, out, unit_stride, norm_stride, nrhs, groups, in_list, out_list);
+    kernel<<<nb * (nrhs / 2 + nrhs % 2), MULTI_THREADS, 0, st>>>(g, U, C, in, out, unit_stride, norm_stride, nrhs, nb,
+                                                                 in_list, out_list);
   };
   switch (domain_shape_id(g)) {
     case 1: launch(apply_A_multi_kernel<T, 1>); break;

@@ -151,3 +151,33 @@ def test_lockstep_solve_over_lattices():
             x1 = np.zeros_like(f[r])
             c.dd_solve(f[r], x1, storage_prec=dd.DD_PREC_FP16, **kw)
             assert rel(x[r], x1) <= 1e-8
+
+
+@pytest.mark.parametrize("dom", [(4, 4, 4, 4), (4, 4, 4, 8)], ids=["4444", "4448"])
+@pytest.mark.parametrize("prec", [dd.DD_PREC_FP32, dd.DD_PREC_FP16], ids=["fp32", "fp16"])
+def test_left_over_field_costs_no_more_than_alone(prec, dom):
+    """Three fields in one batch take no longer than a batch of two and a batch of one (15 %
+    for the spread of the timings; interleaved with the pairs' blocks the third field cost 1.3 to
+    1.8 times that).  Best of eight windows of ten synchronous calls; links are the identity."""
+    import time
+    dims = (24, 24, 24, 48)
+    U = torch.zeros(dims[::-1] + (4, 3, 3, 2), dtype=torch.float64, device="cuda")
+    U[..., 0] = torch.eye(3, dtype=torch.float64, device="cuda")
+    c = dd.Context(dims, dom, stream=torch.cuda.current_stream().cuda_stream)
+    c.dd_load_gauge(U, dd.DD_DEVICE)
+    c.dd_build_clover(0.124, 1.5)
+    f = torch.randn(dims[::-1] + (4, 3, 2), dtype=torch.float32, device="cuda")
+    nb = c.dd_spinor_bytes(prec, dd.DD_LAYOUT_INTERNAL)
+    src = torch.empty(3 * nb, dtype=torch.uint8, device="cuda")
+    out = torch.empty_like(src)
+    for r in range(3):
+        c.dd_pack_spinor(f, dd.DD_PREC_FP32, src[r * nb:(r + 1) * nb], prec)
+    best = {n: float("inf") for n in (1, 2, 3)}
+    for _ in range(8):
+        for n in best:
+            c.dd_apply_D_batch(src, out, n, prec)
+            t0 = time.perf_counter()
+            for _ in range(10):
+                c.dd_apply_D_batch(src, out, n, prec)
+            best[n] = min(best[n], time.perf_counter() - t0)
+    assert best[3] <= 1.15 * (best[1] + best[2]), best
