@@ -687,11 +687,7 @@ __global__ void deflate_kernel(const zd* H, int ldh, int mm, int k, const zd* c0
 static void launch_deflate(const zd* H, int ldh, int mm, int k, const zd* c0, const zd* y, zd* P, zd* Hn, zd* cn,
                            zd* theta, void* gscratch, int* flags, cudaStream_t st) {
   constexpr size_t smem_cap = 200 * 1024;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(deflate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cap);
-    configured = true;
-  }
+  allow_smem((const void*)deflate_kernel, smem_cap);
   const size_t b = deflate_bytes(mm);
   const int in_smem = b <= smem_cap;
   deflate_kernel<<<1, 32, in_smem ? b : 0, st>>>(H, ldh, mm, k, c0, y, P, Hn, cn, theta, gscratch, in_smem, flags);
@@ -2364,9 +2360,7 @@ extern "C" dd_status dd_autotune(dd_ctx* c, int storage_prec, int domain_out[4],
   if (st != DD_OK) { release(c, f); return st; }
   fill_random64_kernel<<<blas_partials_blocks(), 256, 0, c->st>>>(f, nreal, 12345);
   st = launched(c);
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_info().sms;
   dd_solve_params sp;
   memset(&sp, 0, sizeof(sp));
   sp.tol = 1e-7;

@@ -16,17 +16,8 @@ namespace dd {
 
 constexpr int BT = 256;           // threads per block
 constexpr int NCHUNK = 8;         // vectors per pass of the multi-dot
-static int g_blocks = 0;
 
-int blas_partials_blocks() {
-  if (!g_blocks) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    g_blocks = 4 * (sms > 0 ? sms : 1);
-  }
-  return g_blocks;
-}
+int blas_partials_blocks() { return 4 * device_info().sms; }
 
 __device__ inline cx<float> dot4(float4 v, float4 w) {  // conj(v) . w over two complex numbers
   return mk(v.x * w.x + v.y * w.y + v.z * w.z + v.w * w.w, v.x * w.y - v.y * w.x + v.z * w.w - v.w * w.z);
@@ -804,21 +795,16 @@ template <int T, int G, int MOST>
 static int project_dot_launch(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
                               const float* vscale, double2* partial, double2* norm_partial, int* err, cudaStream_t st,
                               const GsTail& tail) {
-  const int sms = blas_partials_blocks() / 4;
   const size_t stage = (size_t)(nv + 1) * T * 16, room = (size_t)208 * 1024;
   const int stages = (int)std::min<size_t>(16, room / stage) / G * G;
-  static int configured = 0;
-  if (!configured) {
-    cudaFuncSetAttribute(gs_project_dot_kernel<T, G, MOST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
-    configured = 1;
-  }
-  const int nb = (int)std::min<long long>(sms, n4 / T);
+  const int nb = (int)std::min<long long>(device_info().sms, n4 / T);
   CUtensorMap basis;
   if (!basis_map(&basis, V, nv, n4, T)) {   // no tensor maps: the two passes apart
     launch_gs_project(out, w, V, nv, n4, h, norm_partial, nullptr, 0, st, vscale, tail);
     launch_gs_dot(V, nv, n4, out, partial, nullptr, 0, st, vscale);
     return blas_blocks(n4);
   }
+  allow_smem((const void*)gs_project_dot_kernel<T, G, MOST>, room);
   gs_project_dot_kernel<T, G, MOST><<<nb, G * GT + 32, stages * stage, st>>>(basis, out, w, nv, n4, h, vscale, partial,
                                                                              norm_partial, stages, err, tail);
   return nb * G;

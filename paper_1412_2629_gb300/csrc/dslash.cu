@@ -124,13 +124,7 @@ __global__ void __launch_bounds__(256, 2) apply_A_shape_kernel(Geom g0, LinkPtr<
 // nine SMs in ten idle (107 -> 49 us cold; FP32 8.3 -> 7.7 us).  24^3x48 gains from the shorter
 // tail too: 1.42 -> 1.37 ms.
 static int block_threads(long long V, int most) {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    sms = n > 0 ? n : 1;
-  }
+  const int sms = device_info().sms;
   while (most > 32 && V / most < 2 * sms) most >>= 1;
   return most;
 }

@@ -1410,15 +1410,10 @@ __global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair_lattic
 // fills a few of each SM's places once (256 blocks of 128 threads: 23.7 -> 28.6 us), so not there:
 // only with one block per SM, with half the SMs empty, or with at least two waves.
 static cudaLaunchAttribute overlapped_launch(int grid, int threads, size_t smem) {
-  static int sms = 0, per_sm = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  }
+  const DeviceInfo dev = device_info();
+  const int sms = dev.sms;
   // 128 registers a thread; smem and 2 KB of shared memory a block
-  const int places = std::max(1, std::min((int)(per_sm / (smem + 2048)), 2 * SAP_MAX_THREADS / threads));
+  const int places = std::max(1, std::min((int)(dev.smem_sm / (smem + 2048)), 2 * SAP_MAX_THREADS / threads));
   cudaLaunchAttribute a = {};
   a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   a.val.programmaticStreamSerializationAllowed = places == 1 || 2 * grid <= sms || grid >= 2 * sms * places;
@@ -1436,32 +1431,18 @@ size_t sap_smem_bytes(const Geom& g, int mat_prec, bool mat_in_smem, int threads
   return (lk + (mat_in_smem ? cm : 0)) * g.Vd + (work > faces ? work : faces);
 }
 
-static int smem_optin();
 bool sap_mat_fits_smem(const Geom& g, int mat_prec, int threads_per_site) {
-  return sap_smem_bytes(g, mat_prec, true, threads_per_site) + 1024 <= (size_t)smem_optin();
+  return sap_smem_bytes(g, mat_prec, true, threads_per_site) + 1024 <= (size_t)device_info().smem_block;
 }
 
-static int smem_optin() {
-  static int v = -1;
-  if (v < 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  }
-  return v;
-}
+// Static shared memory (barriers, reduction slots) is below 1 KB; the rest may be dynamic.
+static void allow_sap_smem(const void* kernel) { allow_smem(kernel, device_info().smem_block - 1024); }
 
 int sap_max_domain_sites() { return 2 * SAP_MAX_THREADS; }
 
 template <typename MT, bool MATS, bool H2, int SHAPE>
 static void launch_shape(const SapArgs& a, int grid, size_t smem, cudaStream_t st) {
-  static int configured = 0;
-  if (!configured) {
-    // static shared memory (barriers, reduction slots) is below 1 KB; the rest may be dynamic
-    cudaFuncSetAttribute(sap_kernel_pair<MT, MATS, H2, SHAPE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem_optin() - 1024);
-    configured = 1;
-  }
+  allow_sap_smem((const void*)sap_kernel_pair<MT, MATS, H2, SHAPE>);
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3(grid);
   c.blockDim = dim3(2 * a.g.Hd);
@@ -1487,11 +1468,7 @@ static int launch_pair(const SapArgs& a, int grid, cudaStream_t st) {
 template <typename MT, bool MSMEM>
 static int launch_single(const SapArgs& a, int grid, cudaStream_t st) {
   const size_t smem = sap_smem_bytes(a.g, std::is_same<MT, __half>::value ? P16 : P32, MSMEM, 1);
-  static int configured = 0;
-  if (!configured) {
-    cudaFuncSetAttribute(sap_kernel<MT, MT, MSMEM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - 1024);
-    configured = 1;
-  }
+  allow_sap_smem((const void*)sap_kernel<MT, MT, MSMEM>);
   sap_kernel<MT, MT, MSMEM><<<grid, a.g.Hd, smem, st>>>(a);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
@@ -1520,11 +1497,7 @@ int sap_half_sweep_lattices(const Geom* gs, const SapState* Ss, int nlat, int co
   // the domains may differ in shape: room for the one with the most face sites
   size_t smem = 0;
   for (int l = 0; l < nlat; ++l) smem = std::max(smem, sap_smem_bytes(gs[l], P16, true, 2));
-  static int configured = 0;
-  if (!configured) {
-    cudaFuncSetAttribute(sap_kernel_pair_lattices, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - 1024);
-    configured = 1;
-  }
+  allow_sap_smem((const void*)sap_kernel_pair_lattices);
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3(total);
   c.blockDim = dim3(2 * gs[0].Hd);
