@@ -66,7 +66,7 @@ struct SolverBuffers {
   double2* partial = nullptr;
   double2* partial2 = nullptr;         // per-block norm partials of the Gram-Schmidt projection
   double2* nrm2 = nullptr;
-  double* status = nullptr;            // [0] residual estimate, [1] deflate status
+  double* status = nullptr;            // [0] residual estimate, [2] |w|, [3] projected twice, [4] a wait ran out; [8..] restart
   double* h_status = nullptr;          // pinned host mirror
   LsqState* lsq = nullptr;
   int* flag = nullptr;                 // Gram-Schmidt: 1 when a second projection is needed
@@ -99,8 +99,10 @@ struct dd_ctx {
   bool trace = false;   // DD_TRACE=1 in the environment: one line per solver step on stderr
   // DD_INJECT_WAIT_TIMEOUT=1 at dd_create: the Schwarz kernel's bounded wait for its staged
   // data is made to run out (it expects 16 bytes nobody sends, limit 50 ms), to exercise
-  // the DD_ERR_TIMEOUT path without any fault
+  // the DD_ERR_TIMEOUT path without any fault.  DD_INJECT_GS_TIMEOUT=1: the same in the fused
+  // Gram-Schmidt pass of the solvers
   bool inject_wait_timeout = false;
+  bool inject_gs_timeout = false;
   bool use_graphs = true;   // DD_NO_GRAPHS=1: launch the outer solver's kernels directly
   // gauge
   double* Ucanon = nullptr;
@@ -119,7 +121,7 @@ struct dd_ctx {
   double kappa = 0, csw = 0;
   // schwarz
   SapBuffers sap[3];
-  int* sap_err = nullptr;
+  int* wait_err = nullptr;
   // scratch fields for canonical-layout calls
   void* scratch_in = nullptr;
   void* scratch_out = nullptr;
@@ -255,15 +257,17 @@ extern "C" dd_status dd_create(dd_ctx** out, const int dims[4], const int domain
   c->trace = tr && tr[0] && tr[0] != '0';
   const char* inj = getenv("DD_INJECT_WAIT_TIMEOUT");
   c->inject_wait_timeout = inj && inj[0] && inj[0] != '0';
+  const char* inj_gs = getenv("DD_INJECT_GS_TIMEOUT");
+  c->inject_gs_timeout = inj_gs && inj_gs[0] && inj_gs[0] != '0';
   const char* ng = getenv("DD_NO_GRAPHS");
   c->use_graphs = !(ng && ng[0] && ng[0] != '0');
-  if (dalloc(c, &c->dstatus, 64) != DD_OK || dalloc(c, &c->sap_err, 64) != DD_OK) {
+  if (dalloc(c, &c->dstatus, 64) != DD_OK || dalloc(c, &c->wait_err, 64) != DD_OK) {
     for (void* p : c->allocs) cudaFree(p);
     delete c;
     return DD_ERR_OOM;
   }
   cudaMemsetAsync(c->dstatus, 0, 64, c->st);
-  cudaMemsetAsync(c->sap_err, 0, 64, c->st);
+  cudaMemsetAsync(c->wait_err, 0, 64, c->st);
   *out = c;
   return DD_OK;
 }
@@ -463,7 +467,7 @@ static SapState sap_state(dd_ctx* c, int prec, const dd_sap_params* p, int nrhs)
   S.u_store = b.u_store;
   S.u_norm = b.u_norm;
   S.faces = b.faces;
-  S.err = c->sap_err;
+  S.err = c->wait_err;
   S.threads_per_site = p->threads_per_site ? p->threads_per_site : 2;
   S.mat_in_smem = sap_mat_fits_smem(c->g, prec, S.threads_per_site);
   S.inject_wait_timeout = c->inject_wait_timeout;
@@ -528,19 +532,35 @@ static dd_status check_sap_params(dd_ctx* c, const dd_sap_params* p) {
   return DD_OK;
 }
 
-static dd_status sap_error_flag(dd_ctx* c) {
+static const char* const TIMEOUT_MESSAGE = "a bounded wait for staged data ran out";
+
+// The status of a call that came to `rc`: waits for its work, and reads and clears the word that
+// kernels set when a bounded wait runs out.  Every call that launches such kernels ends here,
+// whatever it came to, so that none leaves the word to a later call; a timeout outranks what
+// followed from it (no convergence, non-finite values), not a CUDA error.
+static dd_status wait_status(dd_ctx* c, dd_status rc = DD_OK) {
+  const std::string before = c->err;
   int e = 0;
-  TRY(cuda_check(c, cudaMemcpyAsync(&e, c->sap_err, sizeof(int), cudaMemcpyDeviceToHost, c->st), "sap status"));
-  TRY(cuda_check(c, cudaStreamSynchronize(c->st), "sap"));
-  if (e) {
-    cudaMemsetAsync(c->sap_err, 0, sizeof(int), c->st);
-    // a projection pass that gave up leaves its ticket short
-    if (c->sv.ticket) cudaMemsetAsync(c->sv.ticket, 0, sizeof(int), c->st);
-    for (SolverBuffers& b : c->lock)
-      if (b.ticket) cudaMemsetAsync(b.ticket, 0, sizeof(int), c->st);
-    return fail(c, DD_ERR_TIMEOUT, "a bounded wait for staged data ran out");
+  dd_status s = cuda_check(c, cudaMemcpyAsync(&e, c->wait_err, sizeof(int), cudaMemcpyDeviceToHost, c->st), "wait status");
+  if (s == DD_OK) s = cuda_check(c, cudaStreamSynchronize(c->st), "wait status");
+  if (s == DD_OK && e) {
+    s = cuda_check(c, cudaMemsetAsync(c->wait_err, 0, sizeof(int), c->st), "wait status");
+    if (s == DD_OK) s = fail(c, DD_ERR_TIMEOUT, TIMEOUT_MESSAGE);
   }
-  return DD_OK;
+  if (s != DD_OK && rc != DD_ERR_CUDA && rc != DD_ERR_OOM) return s;
+  c->err = before;
+  return rc;
+}
+
+// The same for a call on several contexts: every one's word is read and cleared; the message
+// goes to the first.
+static dd_status wait_status(dd_ctx** ctxs, int n, dd_status rc) {
+  for (int l = 0; l < n; ++l) {
+    const dd_status s = wait_status(ctxs[l], rc);
+    if (s != rc && l > 0) ctxs[0]->err = ctxs[l]->err;
+    rc = s;
+  }
+  return rc;
 }
 
 extern "C" dd_status dd_sap_precondition(dd_ctx* c, const float* in, float* out, const dd_sap_params* p, int layout) {
@@ -558,7 +578,7 @@ extern "C" dd_status dd_sap_precondition(dd_ctx* c, const float* in, float* out,
     launch_unpack_spinor(c->g, view(c->g, c->scratch_out, P32), out, P32, c->st);
     TRY(launched(c));
   }
-  return sap_error_flag(c);
+  return wait_status(c);
 }
 
 // ------------------------------------------------------------------ several right-hand sides
@@ -570,7 +590,7 @@ extern "C" dd_status dd_sap_precondition_batch(dd_ctx* c, const float* in, float
   if (p->i_domain == 0) return fail(c, DD_ERR_INVALID, "i_domain must be >= 1");
   if (p->threads_per_site == 1 && nrhs > 1) return fail(c, DD_ERR_INVALID, "batches need threads_per_site 2");
   TRY(sap_run(c, (const float4*)in, (float4*)out, p, nrhs));
-  return sap_error_flag(c);
+  return wait_status(c);
 }
 
 extern "C" dd_status dd_sap_precondition_lattices(dd_ctx** ctxs, const float* const* in, float* const* out, int nlat,
@@ -604,9 +624,8 @@ extern "C" dd_status dd_sap_precondition_lattices(dd_ctx** ctxs, const float* co
         return fail(c0, DD_ERR_CUDA, std::string("Schwarz launch failed: ") + cudaGetErrorString(cudaGetLastError()));
       TRY(launched(c0));
     }
-  TRY(cuda_check(c0, cudaStreamSynchronize(c0->st), "sap_lattices"));
-  for (int l = 0; l < nlat; ++l) TRY(sap_error_flag(ctxs[l]));
-  return DD_OK;
+  // the lattices' words may be read on their own streams once the work on c0's is done
+  return wait_status(ctxs, nlat, cuda_check(c0, cudaStreamSynchronize(c0->st), "sap_lattices"));
 }
 
 extern "C" dd_status dd_apply_D_batch(dd_ctx* c, const void* in, void* out, int nrhs, int prec) {
@@ -631,7 +650,7 @@ __global__ void fill_ones_kernel(float* v, int n) {
 __global__ void set_vscale_kernel(float* vscale, const double* nu2) { vscale[0] = (float)(1.0 / sqrt(*nu2)); }
 
 __global__ void arnoldi_finish_kernel(zd* H, zd* R, int ldh, int j, const zd* hA, const zd* hB, const double* nu2,
-                                      LsqState* lsq, zd* g, double* status) {
+                                      LsqState* lsq, zd* g, double* status, const int* wait_err) {
   zd* col = H + (long)j * ldh;
   for (int i = 0; i <= j; ++i) col[i] = hA[i] + hB[i];
   double h = sqrt(*nu2);
@@ -641,6 +660,7 @@ __global__ void arnoldi_finish_kernel(zd* H, zd* R, int ldh, int j, const zd* hA
   status[0] = lsq_add_column(*lsq, R, ldh, j, j + 2, g);
   status[2] = h;
   status[3] = abs2(hB[0]) > 0 ? 1.0 : 0.0;
+  status[4] = *wait_err;
 }
 
 __global__ void lsq_solve_kernel(const zd* R, int ldh, int n, const zd* g, zd* y) { lsq_solve(R, ldh, n, g, y); }
@@ -1195,7 +1215,8 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
                             gs_tail_of(s, 2));
           cudaEventRecord(s.ev_fork, c->st);
           cudaStreamWaitEvent(s.side, s.ev_fork, 0);
-          arnoldi_finish_kernel<<<1, 1, 0, s.side>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status);
+          arnoldi_finish_kernel<<<1, 1, 0, s.side>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status,
+                                                     c->wait_err);
           cudaEventRecord(s.ev_join, s.side);
           launch_basis16_store(V16(j + 1), s.vin, s.w, n4, s.nu2, vs16, c->st);
           cudaStreamWaitEvent(c->st, s.ev_join, 0);
@@ -1210,7 +1231,7 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
         int nk = launch_gs_dot(Vv(0), j + 1, n4, s.w, s.partial, nullptr, 0, c->st, sc);
         launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
         const int nb = launch_gs_project_dot(vn, s.w, Vv(0), j + 1, n4, (const double2*)s.hA, sc, s.partial, s.partial2,
-                                             c->sap_err, c->st, gs_tail_of(s, 1));
+                                             c->wait_err, c->inject_gs_timeout, c->st, gs_tail_of(s, 1));
         launch_gs_reduce_blocks(s.partial, j + 1, nb, (double2*)s.hB, s.flag, 1, c->st);
         launch_gs_project(vn, vn, Vv(0), j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc,
                             gs_tail_of(s, 2));
@@ -1218,14 +1239,15 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
         // scale; both only read nu2
         cudaEventRecord(s.ev_fork, c->st);
         cudaStreamWaitEvent(s.side, s.ev_fork, 0);
-        arnoldi_finish_kernel<<<1, 1, 0, s.side>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status);
+        arnoldi_finish_kernel<<<1, 1, 0, s.side>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status,
+                                                   c->wait_err);
         cudaEventRecord(s.ev_join, s.side);
         set_vscale_kernel<<<1, 1, 0, c->st>>>(s.vscale + j + 1, s.nu2);
         cudaStreamWaitEvent(c->st, s.ev_join, 0);
         return launched(c, nk + 6);
       }));
       cudaEventRecord(e3, c->st);
-      TRY(read_status(c));
+      TRY(read_status(c, 5));
       float ms;
       cudaEventElapsedTime(&ms, e0, e1); tM += ms * 1e-3;
       cudaEventElapsedTime(&ms, e1, e2); tA += ms * 1e-3;
@@ -1235,6 +1257,7 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
       if (c->trace)
         fprintf(stderr, "[dd] it %d j %d est/rho %.3e h %.3e reorth %d\n", iters, j, est / rho_cycle, s.h_status[2],
                 (int)s.h_status[3]);
+      if (s.h_status[4] != 0.0) { rc = fail(c, DD_ERR_TIMEOUT, TIMEOUT_MESSAGE); break; }
       if (!isfinite(est) || !isfinite(s.h_status[2])) { rc = fail(c, DD_ERR_NONFINITE, "non-finite Arnoldi step"); break; }
       // stop the cycle when the target is met or FP32 vectors cannot resolve further
       if (est <= 0.5 * tol * nf || est <= 2e-6 * rho_cycle || iters >= p->max_iter) { mm = j + 1; break; }
@@ -1304,7 +1327,6 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
     info->flops_nominal += iters * (1848.0 * V + p->sap.i_schwarz * (p->sap.i_domain + 1) * 1848.0 * V) + reliable * 1848.0 * V;
   }
   for (cudaEvent_t e : {e0, e1, e2, e3, e4, tstart, tend}) cudaEventDestroy(e);
-  if (rc == DD_OK) TRY(sap_error_flag(c));
   return rc;
 }
 
@@ -1370,7 +1392,7 @@ static dd_status lock_gs(dd_ctx* c, SolverBuffers& s, int j, int m) {
   int nk = launch_gs_dot(s.V, j + 1, n4, s.w, s.partial, nullptr, 0, c->st, sc);
   launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
   const int nb = launch_gs_project_dot(vn, s.w, s.V, j + 1, n4, (const double2*)s.hA, sc, s.partial, s.partial2,
-                                       c->sap_err, c->st, gs_tail_of(s, 1));
+                                       c->wait_err, c->inject_gs_timeout, c->st, gs_tail_of(s, 1));
   launch_gs_reduce_blocks(s.partial, j + 1, nb, (double2*)s.hB, s.flag, 1, c->st);
   launch_gs_project(vn, vn, s.V, j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc,
                     gs_tail_of(s, 2));
@@ -1378,10 +1400,11 @@ static dd_status lock_gs(dd_ctx* c, SolverBuffers& s, int j, int m) {
   // lock_join makes the context's stream wait for them
   cudaEventRecord(s.ev_fork, c->st);
   cudaStreamWaitEvent(s.side, s.ev_fork, 0);
-  arnoldi_finish_kernel<<<1, 1, 0, s.side>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status);
+  arnoldi_finish_kernel<<<1, 1, 0, s.side>>>(s.H, s.R, ldh, j, s.hA, s.hB, s.nu2, s.lsq, s.g, s.status,
+                                             c->wait_err);
   set_vscale_kernel<<<1, 1, 0, c->st>>>(s.vscale + j + 1, s.nu2);
   TRY(launched(c, nk + 6));
-  TRY(cuda_check(c, cudaMemcpyAsync(s.h_status, s.status, 4 * sizeof(double), cudaMemcpyDeviceToHost, s.side),
+  TRY(cuda_check(c, cudaMemcpyAsync(s.h_status, s.status, 5 * sizeof(double), cudaMemcpyDeviceToHost, s.side),
                  "status"));
   return cuda_check(c, cudaEventRecord(s.ev_join, s.side), "status");
 }
@@ -1518,6 +1541,8 @@ static dd_status solve_lockstep(dd_ctx* c, const double* f, double* x, int nrhs,
       LockRhs& Q = R[r];
       SolverBuffers& s = c->lock[r];
       Q.iters++;
+      if (s.h_status[4] != 0.0) rc = fail(c, DD_ERR_TIMEOUT, TIMEOUT_MESSAGE);
+      if (rc != DD_OK) continue;
       const double est = s.h_status[0];
       if (!isfinite(est) || !isfinite(s.h_status[2])) {
         Q.rc = fail(c, DD_ERR_NONFINITE, "non-finite Arnoldi step");
@@ -1540,7 +1565,7 @@ static dd_status solve_lockstep(dd_ctx* c, const double* f, double* x, int nrhs,
   float ms_total = 0;
   cudaEventElapsedTime(&ms_total, tstart, tend);
   for (cudaEvent_t e : {e0, e1, e2, e3, tstart, tend}) cudaEventDestroy(e);
-  dd_status worst = DD_OK;
+  dd_status worst = rc;
   for (int r = 0; r < nrhs; ++r) {
     SolverBuffers& s = c->lock[r];
     launch_unpack_spinor(g, view(g, s.x64, P64), s.canon64, P64, c->st);
@@ -1565,9 +1590,7 @@ static dd_status solve_lockstep(dd_ctx* c, const double* f, double* x, int nrhs,
     info->t_M = tM;
     info->t_GS = tGS;
     info->t_other = ms_total * 1e-3 - tA - tM - tGS;
-    info->status = worst;
   }
-  if (worst == DD_OK) TRY(sap_error_flag(c));
   return worst;
 }
 
@@ -1654,7 +1677,8 @@ static dd_status solve_lattices(dd_ctx** ctxs, int nlat, const double* const* f,
     }
   }
   std::vector<std::vector<int>> act(nlat);
-  while (true) {
+  dd_status rc = DD_OK;
+  while (rc == DD_OK) {
     int total = 0, nl = 0;
     Geom gs[4];
     SapState Ss[4];
@@ -1720,6 +1744,8 @@ static dd_status solve_lattices(dd_ctx** ctxs, int nlat, const double* const* f,
         LockRhs& Q = R[l][r];
         SolverBuffers& s = ctxs[l]->lock[r];
         Q.iters++;
+        if (s.h_status[4] != 0.0) rc = fail(c0, DD_ERR_TIMEOUT, TIMEOUT_MESSAGE);
+        if (rc != DD_OK) continue;
         const double est = s.h_status[0];
         if (!isfinite(est) || !isfinite(s.h_status[2])) {
           Q.rc = fail(c0, DD_ERR_NONFINITE, "non-finite Arnoldi step");
@@ -1737,7 +1763,7 @@ static dd_status solve_lattices(dd_ctx** ctxs, int nlat, const double* const* f,
   cudaEventSynchronize(tend);
   float ms_total = 0;
   cudaEventElapsedTime(&ms_total, tstart, tend);
-  dd_status worst = DD_OK;
+  dd_status worst = rc;
   for (int l = 0; l < nlat; ++l) {
     dd_ctx* c = ctxs[l];
     const Geom& g = c->g;
@@ -1768,10 +1794,7 @@ static dd_status solve_lattices(dd_ctx** ctxs, int nlat, const double* const* f,
     info->t_M = tM;
     info->t_GS = tGS;
     info->t_other = ms_total * 1e-3 - tA - tM - tGS;
-    info->status = worst;
   }
-  if (worst == DD_OK)
-    for (int l = 0; l < nlat; ++l) TRY(sap_error_flag(ctxs[l]));
   return worst;
 }
 
@@ -1795,7 +1818,9 @@ extern "C" dd_status dd_solve_lattices(dd_ctx** ctxs, int nlat, const double* co
       if (ctxs[q] == ctxs[l]) return fail(c0, DD_ERR_INVALID, "a context appears twice");
   }
   if (info) memset(info, 0, sizeof(*info));
-  return solve_lattices(ctxs, nlat, f, x, nrhs, where, p, info);
+  const dd_status st = wait_status(ctxs, nlat, solve_lattices(ctxs, nlat, f, x, nrhs, where, p, info));
+  if (info) info->status = st;
+  return st;
 }
 
 extern "C" dd_status dd_solve(dd_ctx* c, const double* f, double* x, int nrhs, int where, const dd_solve_params* p,
@@ -1831,8 +1856,11 @@ extern "C" dd_status dd_solve(dd_ctx* c, const double* f, double* x, int nrhs, i
   // several right-hand sides in lockstep, unless the domain solve runs one thread per site
   // (no batched kernel) or DD_SEQUENTIAL_RHS=1 asks for one solve after another
   const char* seq = getenv("DD_SEQUENTIAL_RHS");
-  if (nrhs > 1 && p->sap.threads_per_site != 1 && !(seq && seq[0] == '1'))
-    return solve_lockstep(c, f, x, nrhs, where, p, info);
+  if (nrhs > 1 && p->sap.threads_per_site != 1 && !(seq && seq[0] == '1')) {
+    const dd_status st = wait_status(c, solve_lockstep(c, f, x, nrhs, where, p, info));
+    if (info) info->status = st;
+    return st;
+  }
   const Geom& g = c->g;
   size_t cb = (size_t)g.V * 24 * 8;
   cudaMemcpyKind in_kind = where == DD_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
@@ -1856,7 +1884,7 @@ extern "C" dd_status dd_solve(dd_ctx* c, const double* f, double* x, int nrhs, i
       cudaMemsetAsync(s.x64, 0, field_bytes(g, P64), c->st);
       st = DD_OK;
     } else {
-      st = solve_one(c, p, h.x, info);
+      st = wait_status(c, solve_one(c, p, h.x, info));
     }
     launch_unpack_spinor(g, view(g, s.x64, P64), s.canon64, P64, c->st);
     TRY(launched(c));
@@ -1882,11 +1910,12 @@ __global__ void scale_by_norm_kernel(zd* a, int n, const double2* nrm2) {
   const double rho = sqrt(nrm2->x);
   for (int i = 0; i < n; ++i) a[i] = rho * a[i];
 }
-// status[0] = |r| after the step, status[2] = |w_k| before normalisation
-__global__ void gcr_status_kernel(const double2* nrm_r, const double* nu2, double* status) {
+// status[0] = |r| after the step, status[2] = |w_k| before normalisation, status[4] = a wait ran out
+__global__ void gcr_status_kernel(const double2* nrm_r, const double* nu2, double* status, const int* wait_err) {
   status[0] = sqrt(fmax(nrm_r->x, 0.0));
   status[2] = sqrt(*nu2);
   status[3] = 0.0;
+  status[4] = *wait_err;
 }
 
 static dd_status solve_gcr_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_solve_info* info) {
@@ -1940,10 +1969,10 @@ static dd_status solve_gcr_one(dd_ctx* c, const dd_solve_params* p, double nf2, 
       launch_gs_reduce(s.partial, 1, n4, (double2*)(alpha + k), nullptr, 0, c->st);
       launch_gs_project(r, r, Wv(k), 1, n4, (const double2*)(alpha + k), s.partial2, nullptr, 0, c->st);
       launch_gs_reduce(s.partial2, 0, n4, s.nrm2 + 3, nullptr, 0, c->st);
-      gcr_status_kernel<<<1, 1, 0, c->st>>>(s.nrm2 + 3, s.nu2, s.status);
+      gcr_status_kernel<<<1, 1, 0, c->st>>>(s.nrm2 + 3, s.nu2, s.status, c->wait_err);
       TRY(launched(c, nk + 12));
       cudaEventRecord(e3, c->st);
-      TRY(read_status(c));
+      TRY(read_status(c, 5));
       float ms;
       cudaEventElapsedTime(&ms, e0, e1); tM += ms * 1e-3;
       cudaEventElapsedTime(&ms, e1, e2); tA += ms * 1e-3;
@@ -1952,6 +1981,7 @@ static dd_status solve_gcr_one(dd_ctx* c, const dd_solve_params* p, double nf2, 
       mm = k + 1;
       const double est = s.h_status[0] * sqrt(rho2);
       if (c->trace) fprintf(stderr, "[dd] gcr it %d k %d est/rho %.3e |w| %.3e\n", iters, k, s.h_status[0], s.h_status[2]);
+      if (s.h_status[4] != 0.0) { rc = fail(c, DD_ERR_TIMEOUT, TIMEOUT_MESSAGE); break; }
       if (!isfinite(est) || !isfinite(s.h_status[2])) { rc = fail(c, DD_ERR_NONFINITE, "non-finite GCR step"); break; }
       if (est <= 0.5 * tol * nf || s.h_status[0] <= 2e-6 || iters >= p->max_iter) break;
     }
@@ -1987,7 +2017,6 @@ static dd_status solve_gcr_one(dd_ctx* c, const dd_solve_params* p, double nf2, 
                            reliable * 1848.0 * V;
   }
   for (cudaEvent_t e : {e0, e1, e2, e3, tstart, tend}) cudaEventDestroy(e);
-  if (rc == DD_OK) TRY(sap_error_flag(c));
   return rc;
 }
 
@@ -2020,7 +2049,7 @@ extern "C" dd_status dd_solve_gcr(dd_ctx* c, const double* f, double* x, int whe
   TRY(cuda_check(c, cudaStreamSynchronize(c->st), "norm f"));
   dd_status st = DD_OK;
   if (h.x == 0.0) cudaMemsetAsync(s.x64, 0, field_bytes(g, P64), c->st);
-  else st = solve_gcr_one(c, p, h.x, info);
+  else st = wait_status(c, solve_gcr_one(c, p, h.x, info));
   launch_unpack_spinor(g, view(g, s.x64, P64), s.canon64, P64, c->st);
   TRY(launched(c));
   TRY(cuda_check(c, cudaMemcpyAsync(x, s.canon64, cb, where == DD_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
@@ -2622,7 +2651,7 @@ extern "C" dd_status dd_mg_setup(dd_ctx* c, const double* tv, int where, const d
         }
       }
     }
-  if (rc == DD_OK && p->setup_iters > 0) rc = sap_error_flag(c);
+  if (rc == DD_OK && p->setup_iters > 0) rc = wait_status(c);
   int bad = 0;
   if (rc == DD_OK) rc = cuda_check(c, cudaMemsetAsync(M.state, 0, 16, c->st), "status");
   if (rc == DD_OK) {
@@ -2704,7 +2733,7 @@ extern "C" dd_status dd_mg_precondition(dd_ctx* c, const float* in, float* out, 
     launch_unpack_spinor(c->g, view(c->g, c->scratch_out, P32), out, P32, c->st);
     TRY(launched(c));
   }
-  if (c->mg.smoother.i_schwarz > 0) TRY(sap_error_flag(c));
+  if (c->mg.smoother.i_schwarz > 0) TRY(wait_status(c));
   return cuda_check(c, cudaStreamSynchronize(c->st), "mg precondition");
 }
 

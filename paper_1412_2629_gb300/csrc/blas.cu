@@ -631,14 +631,13 @@ __global__ void __launch_bounds__(G* GT + 32, 1)
     gs_project_dot_kernel(const __grid_constant__ CUtensorMap basis, float4* out, const float4* w, int nv, long long n4,
                           const double2* h,
                           const float* vscale, double2* partial, double2* norm_partial, int stages, int* err,
-                          GsTail tail) {
+                          unsigned long long wait_ns, unsigned extra_tx, GsTail tail) {
   constexpr int K = (MOST + 3) / 4;            // vectors per warp
   constexpr int E = 2 * T / GT;                // complex numbers per thread
   constexpr int FLUSH = 2048 / T;              // tiles between flushes of the FP32 sums
-  constexpr unsigned long long LIMIT = 2000000000ull;
   extern __shared__ __align__(128) float4 sm[];
   __shared__ float2 hs[64];
-  __shared__ uint64_t full[16], empty[16];
+  __shared__ uint64_t full[16], empty[16], injected;
   const int tid = threadIdx.x, lane = tid & 31;
   const int piece = (nv + 1) * T;             // float4 per stage
   for (int i = tid; i < nv; i += G * GT + 32) {
@@ -652,7 +651,9 @@ __global__ void __launch_bounds__(G* GT + 32, 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], GT / 32);
     }
+    mbar_init(&injected, 1);
     mbar_init_fence();
+    if (extra_tx) mbar_expect_tx(&injected, extra_tx);   // test hook: bytes that nobody sends
   }
   __syncthreads();
 
@@ -662,7 +663,7 @@ __global__ void __launch_bounds__(G* GT + 32, 1)
     int issued = 0;
     for (int k = 0, s = 0, turn = 0; k < mine; ++k) {
       // the group has left this stage's previous tile
-      if (!__all_sync(0xffffffffu, turn == 0 || mbar_wait(&empty[s], (turn - 1) & 1, LIMIT))) break;
+      if (!__all_sync(0xffffffffu, turn == 0 || mbar_wait(&empty[s], (turn - 1) & 1, wait_ns))) break;
       if (lane == 0) {
         const long long q = (blockIdx.x + (long long)k * gridDim.x) * T;
         mbar_expect_tx(&full[s], (uint32_t)(piece * 16));
@@ -678,7 +679,7 @@ __global__ void __launch_bounds__(G* GT + 32, 1)
     }
     // no copy may land in this block's shared memory after it has left (a wait only when a
     // group gave up)
-    for (int k = max(0, issued - stages); k < issued; ++k) mbar_wait(&full[k % stages], (k / stages) & 1, LIMIT);
+    for (int k = max(0, issued - stages); k < issued; ++k) mbar_wait(&full[k % stages], (k / stages) & 1, wait_ns);
   } else {
     const int gt = tid - group * GT, warp = gt >> 5;
     float re[K], im[K], nrm = 0.f;
@@ -686,10 +687,11 @@ __global__ void __launch_bounds__(G* GT + 32, 1)
 #pragma unroll
     for (int k = 0; k < K; ++k) re[k] = im[k] = 0.f;
     int left = FLUSH;
+    const bool held = extra_tx && !mbar_wait(&injected, 0, wait_ns);
     for (int k = group, s = group, turn = 0; k < mine; k += G) {
       float4* const st = sm + s * piece;
       const float4* sv = st + T;
-      const bool ok = mbar_wait(&full[s], turn & 1, LIMIT);
+      const bool ok = mbar_wait(&full[s], turn & 1, wait_ns) && !held;
       float2 a[E];
 #pragma unroll
       for (int e = 0; e < E; ++e) a[e] = reinterpret_cast<const float2*>(st)[gt + GT * e];
@@ -793,8 +795,8 @@ static bool basis_map(CUtensorMap* m, const float4* V, int nv, long long n4, int
 
 template <int T, int G, int MOST>
 static int project_dot_launch(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
-                              const float* vscale, double2* partial, double2* norm_partial, int* err, cudaStream_t st,
-                              const GsTail& tail) {
+                              const float* vscale, double2* partial, double2* norm_partial, int* err,
+                              bool inject_timeout, cudaStream_t st, const GsTail& tail) {
   const size_t stage = (size_t)(nv + 1) * T * 16, room = (size_t)208 * 1024;
   const int stages = (int)std::min<size_t>(16, room / stage) / G * G;
   const int nb = (int)std::min<long long>(device_info().sms, n4 / T);
@@ -806,7 +808,9 @@ static int project_dot_launch(float4* out, const float4* w, const float4* V, int
   }
   allow_smem((const void*)gs_project_dot_kernel<T, G, MOST>, room);
   gs_project_dot_kernel<T, G, MOST><<<nb, G * GT + 32, stages * stage, st>>>(basis, out, w, nv, n4, h, vscale, partial,
-                                                                             norm_partial, stages, err, tail);
+                                                                             norm_partial, stages, err,
+                                                                             inject_timeout ? 50000000ull : 2000000000ull,
+                                                                             inject_timeout ? 16u : 0u, tail);
   return nb * G;
 }
 
@@ -814,13 +818,16 @@ static int project_dot_launch(float4* out, const float4* w, const float4* V, int
 // for the single group), so that copies are in flight while every group works.  n4 is a
 // multiple of 6144 (V of 1024), hence of every tile.  Returns the number of rows in partial.
 int launch_gs_project_dot(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
-                          const float* vscale, double2* partial, double2* norm_partial, int* err, cudaStream_t st,
-                          const GsTail& tail) {
-  if (nv <= 7) return project_dot_launch<128, 4, 7>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
-  if (nv <= 15) return project_dot_launch<64, 4, 15>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
-  if (nv <= 31) return project_dot_launch<64, 3, 31>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
-  if (nv <= 51) return project_dot_launch<64, 2, 51>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
-  return project_dot_launch<64, 1, 63>(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, st, tail);
+                          const float* vscale, double2* partial, double2* norm_partial, int* err,
+                          bool inject_timeout, cudaStream_t st, const GsTail& tail) {
+  const auto go = [&](auto launch) {
+    return launch(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, inject_timeout, st, tail);
+  };
+  if (nv <= 7) return go(project_dot_launch<128, 4, 7>);
+  if (nv <= 15) return go(project_dot_launch<64, 4, 15>);
+  if (nv <= 31) return go(project_dot_launch<64, 3, 31>);
+  if (nv <= 51) return go(project_dot_launch<64, 2, 51>);
+  return go(project_dot_launch<64, 1, 63>);
 }
 
 // out = w - V h over an FP16 basis read in unit pairs (see gs_dot16_kernel); in place

@@ -82,3 +82,60 @@ def test_bounded_wait_runs_out_and_context_stays_usable(monkeypatch):
     ok.dd_sap_precondition(src, out, 1, 2, dd.DD_PREC_FP16)
     assert torch.isfinite(out).all()
     c.dd_apply_D(src, torch.empty_like(src), dd.DD_PREC_FP32)
+
+
+def _solves(c, f, **kw):
+    """Each solver on the context `c`, by name, as (solve, right-hand sides)."""
+    two = np.stack([f, f[::-1]])
+    x = np.zeros_like(two)
+    return {"single": (lambda: c.dd_solve(f, x[0], check=False, **kw), 1),
+            "lockstep": (lambda: c.dd_solve(two, x, nrhs=2, check=False, **kw), 2),
+            "gcr": (lambda: c.dd_solve_gcr(f, x[0], check=False, **kw), 1)}
+
+
+@pytest.mark.parametrize("solver", ["single", "lockstep", "gcr"])
+def test_timeout_outranks_the_iteration_limit(solver, monkeypatch):
+    """A solve whose Schwarz launches time out reports that, not what followed from it."""
+    dims, dom = (8, 8, 8, 8), (4, 4, 4, 4)
+    monkeypatch.setenv("DD_INJECT_WAIT_TIMEOUT", "1")
+    c = ctx_for(dims, dom, gauge(dims, 0.5, 5), 0.13, 1.0)
+    solve, n = _solves(c, synth.gaussian_source(dims, 7), tol=1e-10, m=4, max_iter=1, i_schwarz=1, i_domain=2)[solver]
+    info = solve()
+    assert info.status == dd.DD_ERR_TIMEOUT and info.iterations == n
+
+
+def _schwarz(c, f):
+    src = dev(f, torch.float32)
+    out = torch.empty_like(src)
+    c.dd_sap_precondition(src, out, 1, 2, dd.DD_PREC_FP16)
+    return out
+
+
+@pytest.mark.parametrize("solver", ["single", "lockstep"])
+def test_projection_wait_runs_out_and_is_reported_once(solver, monkeypatch):
+    """The fused Gram-Schmidt pass gives up: the solve ends at that step with a timeout, and the
+    next call on the context succeeds."""
+    dims, dom = (8, 8, 8, 8), (4, 4, 4, 4)
+    U, f = gauge(dims, 0.5, 5), synth.gaussian_source(dims, 7)
+    monkeypatch.setenv("DD_INJECT_GS_TIMEOUT", "1")
+    c = ctx_for(dims, dom, U, 0.13, 1.0)
+    solve, n = _solves(c, f, tol=1e-10, m=8, i_schwarz=1, i_domain=2)[solver]
+    info = solve()
+    assert info.status == dd.DD_ERR_TIMEOUT and info.iterations == n
+    monkeypatch.delenv("DD_INJECT_GS_TIMEOUT")
+    assert torch.equal(_schwarz(c, f), _schwarz(ctx_for(dims, dom, U, 0.13, 1.0), f))
+
+
+def test_projection_wait_runs_out_on_two_lattices(monkeypatch):
+    """Every lattice's error word is read and cleared, not only the first one's."""
+    shapes, dom = [(8, 8, 8, 8), (16, 8, 8, 8)], (4, 4, 4, 4)
+    Us = [gauge(d, 0.5, 5) for d in shapes]
+    fs = [synth.gaussian_source(d, 7) for d in shapes]
+    monkeypatch.setenv("DD_INJECT_GS_TIMEOUT", "1")
+    ctxs = [ctx_for(d, dom, U, 0.13, 1.0) for d, U in zip(shapes, Us)]
+    info = dd.dd_solve_lattices(ctxs, fs, [np.zeros_like(f) for f in fs], tol=1e-10, m=8, i_schwarz=1, i_domain=2,
+                                check=False)
+    assert info.status == dd.DD_ERR_TIMEOUT and info.iterations == 2
+    monkeypatch.delenv("DD_INJECT_GS_TIMEOUT")
+    for c, d, U, f in zip(ctxs, shapes, Us, fs):
+        assert torch.equal(_schwarz(c, f), _schwarz(ctx_for(d, dom, U, 0.13, 1.0), f))
