@@ -707,7 +707,8 @@ __global__ void deflate_kernel(const zd* H, int ldh, int mm, int k, const zd* c0
 static void launch_deflate(const zd* H, int ldh, int mm, int k, const zd* c0, const zd* y, zd* P, zd* Hn, zd* cn,
                            zd* theta, void* gscratch, int* flags, cudaStream_t st) {
   constexpr size_t smem_cap = 200 * 1024;
-  allow_smem((const void*)deflate_kernel, smem_cap);
+  static SmemAllowed allowed;
+  allow_smem(allowed, device_info(), (const void*)deflate_kernel, smem_cap);
   const size_t b = deflate_bytes(mm);
   const int in_smem = b <= smem_cap;
   deflate_kernel<<<1, 32, in_smem ? b : 0, st>>>(H, ldh, mm, k, c0, y, P, Hn, cn, theta, gscratch, in_smem, flags);

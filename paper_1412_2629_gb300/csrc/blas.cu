@@ -799,14 +799,16 @@ static int project_dot_launch(float4* out, const float4* w, const float4* V, int
                               bool inject_timeout, cudaStream_t st, const GsTail& tail) {
   const size_t stage = (size_t)(nv + 1) * T * 16, room = (size_t)208 * 1024;
   const int stages = (int)std::min<size_t>(16, room / stage) / G * G;
-  const int nb = (int)std::min<long long>(device_info().sms, n4 / T);
+  const DeviceInfo& dev = device_info();
+  const int nb = (int)std::min<long long>(dev.sms, n4 / T);
   CUtensorMap basis;
   if (!basis_map(&basis, V, nv, n4, T)) {   // no tensor maps: the two passes apart
     launch_gs_project(out, w, V, nv, n4, h, norm_partial, nullptr, 0, st, vscale, tail);
     launch_gs_dot(V, nv, n4, out, partial, nullptr, 0, st, vscale);
     return blas_blocks(n4);
   }
-  allow_smem((const void*)gs_project_dot_kernel<T, G, MOST>, room);
+  static SmemAllowed allowed;
+  allow_smem(allowed, dev, (const void*)gs_project_dot_kernel<T, G, MOST>, room);
   gs_project_dot_kernel<T, G, MOST><<<nb, G * GT + 32, stages * stage, st>>>(basis, out, w, nv, n4, h, vscale, partial,
                                                                              norm_partial, stages, err,
                                                                              inject_timeout ? 50000000ull : 2000000000ull,

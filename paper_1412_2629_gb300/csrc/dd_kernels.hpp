@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "dd_common.cuh"
 #include "smalldense.cuh"
 
@@ -27,15 +29,19 @@ struct CloverView { const void* m; int prec; };
 // ---- device (device.cu)
 // Limits of the current device.  Where they cannot be read: one SM and the shared memory that
 // every device has, so that sizes stay positive and the launch reports the error.
+constexpr int MAX_DEVICES = 64;
 struct DeviceInfo {
+  int id = -1;
   int sms = 1;                    // multiprocessors
   int smem_block = 48 * 1024;     // largest dynamic shared memory of a block
   int smem_sm = 48 * 1024;        // shared memory of a multiprocessor
 };
-DeviceInfo device_info();
-// Lets `kernel` use up to `bytes` of dynamic shared memory on the current device (needed above
-// 48 KB, before every launch: the attribute is the device's).  A refusal shows at the launch.
-void allow_smem(const void* kernel, size_t bytes);
+const DeviceInfo& device_info();
+// Lets `kernel` use up to `bytes` of dynamic shared memory on the current device `dev` (needed
+// above 48 KB, before every launch: the attribute is the device's).  `done`: one static object for
+// each kernel.  A refusal shows at the launch.
+struct SmemAllowed { std::atomic<unsigned long long> devices{0}; };   // bit per device
+void allow_smem(SmemAllowed& done, const DeviceInfo& dev, const void* kernel, size_t bytes);
 
 // ---- layout (layout_clover.cu)
 void launch_pack_spinor(const Geom& g, const void* canon, int canon_prec, FieldView out, cudaStream_t st);

@@ -496,7 +496,8 @@ __global__ void __launch_bounds__(CLOVER_THREADS, 2)
 void launch_build_clover(const Geom& g, const double* canon, double kappa, double csw, double2* c64, float4* c32,
                          uint4* c16, float4* s32, uint4* s16, int* status, cudaStream_t st) {
   const size_t smem = sizeof(double) * 54 * CLOVER_THREADS;
-  allow_smem((const void*)build_clover_kernel, smem);
+  static SmemAllowed allowed;
+  allow_smem(allowed, device_info(), (const void*)build_clover_kernel, smem);
   build_clover_kernel<<<nblk(g.V, CLOVER_THREADS), CLOVER_THREADS, smem, st>>>(g, canon, kappa, csw, c64, c32, c16, s32,
                                                                              s16, status);
 }

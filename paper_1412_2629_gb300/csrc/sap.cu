@@ -1409,8 +1409,7 @@ __global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair_lattic
 // blocks take the places that are free, which leaves the SMs unevenly loaded where a launch
 // fills a few of each SM's places once (256 blocks of 128 threads: 23.7 -> 28.6 us), so not there:
 // only with one block per SM, with half the SMs empty, or with at least two waves.
-static cudaLaunchAttribute overlapped_launch(int grid, int threads, size_t smem) {
-  const DeviceInfo dev = device_info();
+static cudaLaunchAttribute overlapped_launch(const DeviceInfo& dev, int grid, int threads, size_t smem) {
   const int sms = dev.sms;
   // 128 registers a thread; smem and 2 KB of shared memory a block
   const int places = std::max(1, std::min((int)(dev.smem_sm / (smem + 2048)), 2 * SAP_MAX_THREADS / threads));
@@ -1436,19 +1435,23 @@ bool sap_mat_fits_smem(const Geom& g, int mat_prec, int threads_per_site) {
 }
 
 // Static shared memory (barriers, reduction slots) is below 1 KB; the rest may be dynamic.
-static void allow_sap_smem(const void* kernel) { allow_smem(kernel, device_info().smem_block - 1024); }
+static void allow_sap_smem(SmemAllowed& done, const DeviceInfo& dev, const void* kernel) {
+  allow_smem(done, dev, kernel, dev.smem_block - 1024);
+}
 
 int sap_max_domain_sites() { return 2 * SAP_MAX_THREADS; }
 
 template <typename MT, bool MATS, bool H2, int SHAPE>
 static void launch_shape(const SapArgs& a, int grid, size_t smem, cudaStream_t st) {
-  allow_sap_smem((const void*)sap_kernel_pair<MT, MATS, H2, SHAPE>);
+  static SmemAllowed allowed;
+  const DeviceInfo& dev = device_info();
+  allow_sap_smem(allowed, dev, (const void*)sap_kernel_pair<MT, MATS, H2, SHAPE>);
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3(grid);
   c.blockDim = dim3(2 * a.g.Hd);
   c.dynamicSmemBytes = smem;
   c.stream = st;
-  cudaLaunchAttribute early = overlapped_launch(grid, 2 * a.g.Hd, smem);
+  cudaLaunchAttribute early = overlapped_launch(dev, grid, 2 * a.g.Hd, smem);
   c.attrs = &early;
   c.numAttrs = 1;
   cudaLaunchKernelEx(&c, sap_kernel_pair<MT, MATS, H2, SHAPE>, a);
@@ -1468,7 +1471,8 @@ static int launch_pair(const SapArgs& a, int grid, cudaStream_t st) {
 template <typename MT, bool MSMEM>
 static int launch_single(const SapArgs& a, int grid, cudaStream_t st) {
   const size_t smem = sap_smem_bytes(a.g, std::is_same<MT, __half>::value ? P16 : P32, MSMEM, 1);
-  allow_sap_smem((const void*)sap_kernel<MT, MT, MSMEM>);
+  static SmemAllowed allowed;
+  allow_sap_smem(allowed, device_info(), (const void*)sap_kernel<MT, MT, MSMEM>);
   sap_kernel<MT, MT, MSMEM><<<grid, a.g.Hd, smem, st>>>(a);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
@@ -1497,13 +1501,15 @@ int sap_half_sweep_lattices(const Geom* gs, const SapState* Ss, int nlat, int co
   // the domains may differ in shape: room for the one with the most face sites
   size_t smem = 0;
   for (int l = 0; l < nlat; ++l) smem = std::max(smem, sap_smem_bytes(gs[l], P16, true, 2));
-  allow_sap_smem((const void*)sap_kernel_pair_lattices);
+  static SmemAllowed allowed;
+  const DeviceInfo& dev = device_info();
+  allow_sap_smem(allowed, dev, (const void*)sap_kernel_pair_lattices);
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3(total);
   c.blockDim = dim3(2 * gs[0].Hd);
   c.dynamicSmemBytes = smem;
   c.stream = st;
-  cudaLaunchAttribute early = overlapped_launch(total, 2 * gs[0].Hd, smem);
+  cudaLaunchAttribute early = overlapped_launch(dev, total, 2 * gs[0].Hd, smem);
   c.attrs = &early;
   c.numAttrs = 1;
   cudaLaunchKernelEx(&c, sap_kernel_pair_lattices, m);
