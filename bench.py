@@ -62,11 +62,12 @@ def sap_visit_flops(b, i_domain):
     return useful, nominal
 
 
-def dslash_bytes_per_site(prec):
-    """Algorithmic bytes of one full operator application per site: 4 links (18 reals),
-    clover (72 reals), input and output spinors (24 reals each) = 192 reals; FP16
-    storage adds the two 4-byte spinor norms."""
-    return {"fp64": 192 * 8, "fp32": 192 * 4, "fp16": 192 * 2 + 8}[prec]
+def dslash_bytes_per_site(prec, nrhs=1):
+    """Algorithmic bytes of one full operator application per site and right-hand side: 4 links
+    (18 reals) and the clover (72 reals), read once for all nrhs of a batch, and input and output
+    spinors (24 reals each) = 192 reals for one; FP16 storage adds the two 4-byte spinor norms."""
+    real, norms = {"fp64": (8, 0), "fp32": (4, 0), "fp16": (2, 8)}[prec]
+    return (144 / nrhs + 48) * real + norms
 
 
 # ------------------------------------------------------------------ clocks
@@ -670,8 +671,7 @@ def kernel_case(args, local):
                "launch_ms": 1e3 * launch_s, "tflops_useful": nr * useful * V / 2 / launch_s / 1e12,
                "gflops_nominal": nr * nominal * V / 2 / launch_s / 1e9}
     else:
-        # per right-hand side the batch reads the links and clover once per pair
-        per_site = dslash_bytes_per_site("fp32") if nr == 1 else (72 + 72) * 4 / 2 + 48 * 4
+        per_site = dslash_bytes_per_site("fp32", nr)
         out = {"case": fp32_operator_kernel(w.domain) if nr == 1 else "apply_A_multi_kernel<float>", "nrhs": nr,
                "lattice": dims, "launch_ms": 1e3 * launch_s,
                "ms_per_rhs": 1e3 * launch_s / nr,

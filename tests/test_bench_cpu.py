@@ -24,6 +24,13 @@ def test_operator_bytes_per_site(bench):
     assert bench.dslash_bytes_per_site("fp16") == 392   # plus two 4-byte spinor norms
 
 
+def test_batch_operator_bytes_per_site(bench):
+    # links and clover once per call, whatever the number of right-hand sides
+    for n in (1, 2, 5, 6):
+        assert n * bench.dslash_bytes_per_site("fp32", n) == pytest.approx((144 + 48 * n) * 4)
+        assert n * bench.dslash_bytes_per_site("fp16", n) == pytest.approx((144 + 48 * n) * 2 + 8 * n)
+
+
 def test_paper_flop_counts(bench):
     # 8 hops x 168 = 1344 for the hopping term, 504 for the clover term, 1848 in all
     assert 8 * bench.FLOP_HOP + bench.FLOP_CLOVER == bench.FLOP_A == 1848
