@@ -642,10 +642,6 @@ __global__ void fill_value_kernel(float* v, int n, float x) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = x;
 }
 
-__global__ void fill_ones_kernel(float* v, int n) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = 1.f;
-}
-
 // vscale[0] = 1 / sqrt(nu2): the scale of a vector stored unnormalised
 __global__ void set_vscale_kernel(float* vscale, const double* nu2) { vscale[0] = (float)(1.0 / sqrt(*nu2)); }
 

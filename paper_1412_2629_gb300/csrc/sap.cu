@@ -697,17 +697,6 @@ __device__ __forceinline__ void join_halves(const Spinor<float>& acc, Half<float
       own.c[s][c] = mk(acc.c[s][c].re + __shfl_xor_sync(0xffffffffu, acc.c[2 + s][c].re, 16),
                        acc.c[s][c].im + __shfl_xor_sync(0xffffffffu, acc.c[2 + s][c].im, 16));
 }
-// the site's whole spinor in this lane's frame from the two lanes' own halves
-__device__ __forceinline__ void join_frame(const Half<float>& own, Spinor<float>& v) {
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      v.c[s][c] = own.c[s][c];
-      v.c[2 + s][c] = mk(__shfl_xor_sync(0xffffffffu, own.c[s][c].re, 16),
-                         __shfl_xor_sync(0xffffffffu, own.c[s][c].im, 16));
-    }
-}
 
 // One chirality half of a stored spinor (N sites from p on).  The half-precision form is
 // [2][N] 16-byte units (the first four numbers of half h), then [N][2] 8-byte units, scaled
@@ -715,7 +704,7 @@ __device__ __forceinline__ void join_frame(const Half<float>& own, Spinor<float>
 template <typename T> struct HalfField;
 template <> struct HalfField<float> {
   float4* p;
-  __device__ HalfField(void* base, float*, long long first, int) : p((float4*)base + first * 6) {}
+  __device__ HalfField(void* base, float*, long long first) : p((float4*)base + first * 6) {}
   __device__ void load(int N, int r, int h, Half<float>& v) const { ld_half3(p + 3 * h * N + r, N, v); }
   __device__ void store(int N, int r, int h, const Half<float>& v) const { st_half3(p + 3 * h * N + r, N, v); }
   __device__ void prefetch(int N, int r, int h) const {
@@ -726,7 +715,7 @@ template <> struct HalfField<float> {
 template <> struct HalfField<__half> {
   uint4* p;
   float* norm;
-  __device__ HalfField(void* base, float* n, long long first, int) : p((uint4*)base + first * 3), norm(n + first) {}
+  __device__ HalfField(void* base, float* n, long long first) : p((uint4*)base + first * 3), norm(n + first) {}
   __device__ void load(int N, int r, int h, Half<float>& v) const {
     const float n = norm[r];
     const uint4 a = p[h * N + r];
@@ -1149,8 +1138,8 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
   for (int rhs = 0; rhs < a.nrhs; ++rhs) {
     float* const rnr = a.r_norm ? a.r_norm + rhs * a.rn_stride : nullptr;
     float* const unr = a.u_norm ? a.u_norm + rhs * a.un_stride : nullptr;
-    const HalfField<MT> rst((char*)a.r_store + rhs * a.r_bytes, rnr, d * Hd, 0);
-    const HalfField<MT> ust((char*)a.u_store + rhs * a.u_bytes, unr, d * Vd, 0);
+    const HalfField<MT> rst((char*)a.r_store + rhs * a.r_bytes, rnr, d * Hd);
+    const HalfField<MT> ust((char*)a.u_store + rhs * a.u_bytes, unr, d * Vd);
     float inv_sc = 1.f;   // H2: undoes the domain's scaling on the way out
     Half<float> rho, dO, x, t, own;   // residual and solution (even), solution (odd); own halves
 
