@@ -308,6 +308,8 @@ extern "C" dd_status dd_load_gauge(dd_ctx* c, const double* U, int where) {
                  "gauge copy"));
   launch_pack_gauge(g, c->Ucanon, c->anti, c->U64, c->U32, c->U16, c->st);
   TRY(launched(c));
+  // not only for the caller: the Schwarz kernel copies the links before it waits for the previous
+  // launch of its stream, so their writer must have finished before any other work is launched
   TRY(cuda_check(c, cudaStreamSynchronize(c->st), "load_gauge"));
   c->have_gauge = true;
   c->have_clover = false;
@@ -331,6 +333,7 @@ extern "C" dd_status dd_build_clover(dd_ctx* c, double kappa, double csw) {
   TRY(launched(c));
   int bad = 0;
   TRY(cuda_check(c, cudaMemcpyAsync(&bad, c->dstatus, sizeof(int), cudaMemcpyDeviceToHost, c->st), "clover status"));
+  // as in dd_load_gauge: the Schwarz kernel copies its matrices before it waits
   TRY(cuda_check(c, cudaStreamSynchronize(c->st), "build_clover"));
   c->kappa = kappa;
   c->csw = csw;

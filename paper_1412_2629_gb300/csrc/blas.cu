@@ -2,9 +2,9 @@
 // (double2 = one complex number) fields in the internal layout.
 //
 // Inner products: every thread sums its share of the products in FP32 (a few hundred
-// terms at most), converts once, and the block and grid reductions run in FP64.  The
-// grid is a fixed multiple of the SM count, so the order of the final FP64 sum is
-// fixed and the result is reproducible run to run.
+// terms at most), converts once, and the block and grid reductions run in FP64.  The grid
+// follows from the SM count and the field's size alone, so the order of the final FP64 sum
+// is fixed and the result is reproducible run to run.
 #include <cuda.h>
 
 #include <algorithm>

@@ -1124,7 +1124,8 @@ __device__ __forceinline__ void sap_pair_body(const SapArgs& a, int cta) {
   const int r_e = i, r_o = Hd + i;
   float4* const eo = sE + 3 * h * HP + i;   // own half of the even / odd site in the work buffers
   float4* const oo = sO + 3 * h * HP + i;
-  // Links and matrices are constant; everything from here on may come from the previous launch.
+  // Links and matrices were complete before any launch of this stream began (see
+  // overlapped_launch); everything from here on may come from the previous launch.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (tid == 0) {
     if (a.use_faces) stage_faces(a.faces);
@@ -1392,12 +1393,18 @@ __global__ void __launch_bounds__(2 * SAP_MAX_THREADS, 1) sap_kernel_pair_lattic
 }
 
 // A half-sweep's blocks may start before the previous launch of the stream has ended: they stage
-// their links and matrices and wait (griddepcontrol.wait) before they touch anything else.
-// Launches of a few blocks are bound by such latencies: Schwarz on 8^4, 32 half-sweeps, 669 -> 572
-// us; FP32 storage on 16^3x32 323 -> 295 us; 32^3x64 1720 -> 1693 us by its last wave.  Early
-// blocks take the places that are free, which leaves the SMs unevenly loaded where a launch
-// fills a few of each SM's places once (256 blocks of 128 threads: 23.7 -> 28.6 us), so not there:
-// only with one block per SM, with half the SMs empty, or with at least two waves.
+// their links and matrices and wait (griddepcontrol.wait) before they touch anything else.  What
+// they stage is written by dd_load_gauge and dd_build_clover only, which wait for the stream
+// before they return, so no launch that writes it can be the previous one.
+// Launches of a few blocks are bound by such latencies: Schwarz on 8^4, 32 half-sweeps, 640 -> 562
+// us; FP32 storage on 16^3x32, 8 half-sweeps, 309 -> 287 us; 24^3x48, 8 half-sweeps, 868 -> 820 us;
+// 32^3x64, 4 half-sweeps, 1638 -> 1621 us by its last wave.
+// Where a launch fills a few of each SM's places once, early blocks take the places that are
+// free and leave the SMs unevenly loaded: with the next launch let in at a block's start, 256 blocks
+// of 128 threads took 28.6 us for 23.7.  So not there: only with one block per SM, with half the
+// SMs empty, or with at least two waves.  With the next launch let in after the wait, as now, that case
+// gains too (8 half-sweeps of 16^4, 4x4x4x2 domains: 189 us by this rule, 168 without); the
+// sizes between have not been measured.
 static cudaLaunchAttribute overlapped_launch(const DeviceInfo& dev, int grid, int threads, size_t smem) {
   const int sms = dev.sms;
   // 128 registers a thread; smem and 2 KB of shared memory a block
