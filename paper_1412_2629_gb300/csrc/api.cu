@@ -104,6 +104,7 @@ struct dd_ctx {
   bool inject_wait_timeout = false;
   bool inject_gs_timeout = false;
   bool use_graphs = true;   // DD_NO_GRAPHS=1: launch the outer solver's kernels directly
+  bool use_tensor_maps = true;   // DD_NO_TENSOR_MAPS=1: Gram-Schmidt in two passes, as without driver support
   // gauge
   double* Ucanon = nullptr;
   double2* U64 = nullptr;
@@ -261,6 +262,8 @@ extern "C" dd_status dd_create(dd_ctx** out, const int dims[4], const int domain
   c->inject_gs_timeout = inj_gs && inj_gs[0] && inj_gs[0] != '0';
   const char* ng = getenv("DD_NO_GRAPHS");
   c->use_graphs = !(ng && ng[0] && ng[0] != '0');
+  const char* nt = getenv("DD_NO_TENSOR_MAPS");
+  c->use_tensor_maps = !(nt && nt[0] && nt[0] != '0');
   if (dalloc(c, &c->dstatus, 64) != DD_OK || dalloc(c, &c->wait_err, 64) != DD_OK) {
     for (void* p : c->allocs) cudaFree(p);
     delete c;
@@ -919,6 +922,8 @@ static GsTail gs_tail_of(const SolverBuffers& s, int stage) {
   return t;
 }
 
+static GsWait gs_wait_of(const dd_ctx* c) { return GsWait{c->wait_err, c->inject_gs_timeout, c->use_tensor_maps}; }
+
 // rho2 = |f - A x|^2 into s.nrm2 (device) and return it on the host (s: the context's own
 // solver buffers unless given).
 static dd_status true_residual(dd_ctx* c, double* rho2, SolverBuffers* sp = nullptr, bool initial = false) {
@@ -1231,7 +1236,7 @@ static dd_status solve_one(dd_ctx* c, const dd_solve_params* p, double nf2, dd_s
         int nk = launch_gs_dot(Vv(0), j + 1, n4, s.w, s.partial, nullptr, 0, c->st, sc);
         launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
         const int nb = launch_gs_project_dot(vn, s.w, Vv(0), j + 1, n4, (const double2*)s.hA, sc, s.partial, s.partial2,
-                                             c->wait_err, c->inject_gs_timeout, c->st, gs_tail_of(s, 1));
+                                             gs_wait_of(c), c->st, gs_tail_of(s, 1));
         launch_gs_reduce_blocks(s.partial, j + 1, nb, (double2*)s.hB, s.flag, 1, c->st);
         launch_gs_project(vn, vn, Vv(0), j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc,
                             gs_tail_of(s, 2));
@@ -1392,7 +1397,7 @@ static dd_status lock_gs(dd_ctx* c, SolverBuffers& s, int j, int m) {
   int nk = launch_gs_dot(s.V, j + 1, n4, s.w, s.partial, nullptr, 0, c->st, sc);
   launch_gs_reduce(s.partial, j + 1, n4, (double2*)s.hA, nullptr, 0, c->st);
   const int nb = launch_gs_project_dot(vn, s.w, s.V, j + 1, n4, (const double2*)s.hA, sc, s.partial, s.partial2,
-                                       c->wait_err, c->inject_gs_timeout, c->st, gs_tail_of(s, 1));
+                                       gs_wait_of(c), c->st, gs_tail_of(s, 1));
   launch_gs_reduce_blocks(s.partial, j + 1, nb, (double2*)s.hB, s.flag, 1, c->st);
   launch_gs_project(vn, vn, s.V, j + 1, n4, (const double2*)s.hB, s.partial2, s.flag, 1, c->st, sc,
                     gs_tail_of(s, 2));

@@ -795,14 +795,14 @@ static bool basis_map(CUtensorMap* m, const float4* V, int nv, long long n4, int
 
 template <int T, int G, int MOST>
 static int project_dot_launch(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
-                              const float* vscale, double2* partial, double2* norm_partial, int* err,
-                              bool inject_timeout, cudaStream_t st, const GsTail& tail) {
+                              const float* vscale, double2* partial, double2* norm_partial, const GsWait& wait,
+                              cudaStream_t st, const GsTail& tail) {
   const size_t stage = (size_t)(nv + 1) * T * 16, room = (size_t)208 * 1024;
   const int stages = (int)std::min<size_t>(16, room / stage) / G * G;
   const DeviceInfo& dev = device_info();
   const int nb = (int)std::min<long long>(dev.sms, n4 / T);
   CUtensorMap basis;
-  if (!basis_map(&basis, V, nv, n4, T)) {   // no tensor maps: the two passes apart
+  if (!wait.tensor_maps || !basis_map(&basis, V, nv, n4, T)) {   // no tensor maps: the two passes apart
     launch_gs_project(out, w, V, nv, n4, h, norm_partial, nullptr, 0, st, vscale, tail);
     launch_gs_dot(V, nv, n4, out, partial, nullptr, 0, st, vscale);
     return blas_blocks(n4);
@@ -810,9 +810,9 @@ static int project_dot_launch(float4* out, const float4* w, const float4* V, int
   static SmemAllowed allowed;
   allow_smem(allowed, dev, (const void*)gs_project_dot_kernel<T, G, MOST>, room);
   gs_project_dot_kernel<T, G, MOST><<<nb, G * GT + 32, stages * stage, st>>>(basis, out, w, nv, n4, h, vscale, partial,
-                                                                             norm_partial, stages, err,
-                                                                             inject_timeout ? 50000000ull : 2000000000ull,
-                                                                             inject_timeout ? 16u : 0u, tail);
+                                                                             norm_partial, stages, wait.err,
+                                                                             wait.inject_timeout ? 50000000ull : 2000000000ull,
+                                                                             wait.inject_timeout ? 16u : 0u, tail);
   return nb * G;
 }
 
@@ -820,10 +820,10 @@ static int project_dot_launch(float4* out, const float4* w, const float4* V, int
 // for the single group), so that copies are in flight while every group works.  n4 is a
 // multiple of 6144 (V of 1024), hence of every tile.  Returns the number of rows in partial.
 int launch_gs_project_dot(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
-                          const float* vscale, double2* partial, double2* norm_partial, int* err,
-                          bool inject_timeout, cudaStream_t st, const GsTail& tail) {
+                          const float* vscale, double2* partial, double2* norm_partial, const GsWait& wait,
+                          cudaStream_t st, const GsTail& tail) {
   const auto go = [&](auto launch) {
-    return launch(out, w, V, nv, n4, h, vscale, partial, norm_partial, err, inject_timeout, st, tail);
+    return launch(out, w, V, nv, n4, h, vscale, partial, norm_partial, wait, st, tail);
   };
   if (nv <= 7) return go(project_dot_launch<128, 4, 7>);
   if (nv <= 15) return go(project_dot_launch<64, 4, 15>);

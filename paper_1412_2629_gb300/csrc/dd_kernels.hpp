@@ -160,11 +160,15 @@ void launch_gs_project(float4* out, const float4* w, const float4* V, int nv, lo
                        const float* vscale = nullptr, const GsTail& tail = GsTail());
 // The first projection and the second one's dots in one pass over an FP32 basis: out = w - V h
 // (out != w), partial rows [nv + 1] of V^H out.  Returns the number of rows, to be summed by
-// launch_gs_reduce_blocks.  err: set to 1 when a bounded device wait runs out; inject_timeout
-// makes it run out (test hook).
+// launch_gs_reduce_blocks.
+struct GsWait {
+  int* err;                      // set to 1 when a bounded device wait runs out
+  bool inject_timeout = false;   // make it run out (test hook)
+  bool tensor_maps = true;       // false, or where the driver has none: two passes in its place
+};
 int launch_gs_project_dot(float4* out, const float4* w, const float4* V, int nv, long long n4, const double2* h,
-                          const float* vscale, double2* partial, double2* norm_partial, int* err,
-                          bool inject_timeout, cudaStream_t st, const GsTail& tail);
+                          const float* vscale, double2* partial, double2* norm_partial, const GsWait& wait,
+                          cudaStream_t st, const GsTail& tail);
 void launch_gs_reduce_blocks(const double2* partial, int nv, int nb, double2* out, const int* gate, int want,
                              cudaStream_t st);
 void launch_scale_inplace(float4* v, long long n4, const double* nu2, cudaStream_t st);

@@ -8,8 +8,9 @@
 // the links.  The diagonal 1/(2 kappa) is folded into the stored clover.
 // Bytes per site (algorithmic, each field read once): 4 links + clover + in + out =
 // 192 reals; FP32 768 B, FP64 1536 B, FP16 384 B + 8 B of spinor norms.  The stored FP16 links
-// hold one entry of each twice for the Schwarz kernel's loads, so FP16 moves 400 + 8 B; in three
-// vector loads a link instead of nine words all the same faster (24^3x48 150 -> 107 us).
+// hold one entry of each twice for the Schwarz kernel's loads, so FP16 moves 400 + 8 B; with three
+// vector loads a link instead of nine words, and fused products, it is faster all the same
+// (24^3x48 150 -> 107 us).
 #include <type_traits>
 
 #include "dd_kernels.hpp"

@@ -2,8 +2,8 @@
 fused projection-and-dot pass (up to 7, 15, 31, 51 and 63 vectors) contributes, on fields with fewer
 tiles than SMs and on larger ones, in the single and in the lockstep solver.
 
-No cycle ends early at the two kappas.  At 0.25 the first projection cancels little and a second
-one never runs; at 0.16 it runs in (nearly) every step, on the dots of the fused pass.  The basis is
+No cycle ends early on these fields.  At kappa 0.25 the first projection cancels little and a
+second one never runs; at 0.16 it runs in most steps, on the dots of the fused pass.  The basis is
 orthogonal to the accuracy of the last projection's dot products: a thread or lane adds at most
 82 terms in FP32 before FP64 (or a two-float sum) takes over, so |v_i . v_j| stays below
 82 * 2^-24 = 5e-6 (a missing or misplaced term would leave 1e-3 and more)."""
@@ -35,11 +35,14 @@ def test_basis_orthogonality(dims, dom, m, capfd, monkeypatch):
     assert float(got[-1][0]) <= 82 * 2.0 ** -24
 
 
-@pytest.mark.parametrize("dims,dom", [((8, 8, 4, 4), (4, 4, 2, 2)), ((8, 8, 8, 8), (4, 4, 4, 4)),
-                                      ((24, 24, 24, 24), (4, 4, 4, 4))], ids=["8x8x4x4", "8^4", "24^4"])
-def test_orthogonality_with_the_fused_dots(dims, dom, capfd, monkeypatch):
-    """kappa 0.16.  On 24^4 a group of warps hands its FP32 sums on in mid-run: every 2048 float4."""
+@pytest.mark.parametrize("fused", [True, False], ids=["fused", "apart"])
+@pytest.mark.parametrize("dims,dom", [((4, 4, 8, 8), (2, 2, 4, 4)), ((8, 8, 8, 8), (4, 4, 4, 4)),
+                                      ((24, 24, 24, 24), (4, 4, 4, 4))], ids=["4x4x8x8", "8^4", "24^4"])
+def test_orthogonality_with_two_projections(dims, dom, fused, capfd, monkeypatch):
+    """kappa 0.16, with the fused pass and with the two passes that stand in for it without tensor
+    maps.  On 24^4 a group of warps hands its FP32 sums on in mid-run: every 2048 float4."""
     monkeypatch.setenv("DD_TRACE", "2")
+    monkeypatch.setenv("DD_NO_TENSOR_MAPS", "0" if fused else "1")
     if dims[0] == 24:
         sms = torch.cuda.get_device_properties(0).multi_processor_count
         assert np.prod(dims) * 6 // (4 * sms) > 2048, "too few tiles per group for a hand-over before the last one"

@@ -53,7 +53,7 @@ static void run(int dev) {
   for (int nv : {1, 8, 16, 32, 63}) {
     grids().clear();
     const int rows = dd::launch_gs_project_dot(nullptr, nullptr, nullptr, nv, n4, nullptr, nullptr, nullptr, nullptr,
-                                               nullptr, false, nullptr, tail);
+                                               dd::GsWait{nullptr}, nullptr, tail);
     const int groups = nv <= 15 ? 4 : nv <= 31 ? 3 : nv <= 51 ? 2 : 1;
     const std::vector<unsigned> two = {(unsigned)most, (unsigned)(most * ((nv + 7) / 8))}, one = {(unsigned)multiprocessors(dev)};
     if (rows != (tensor_maps() ? multiprocessors(dev) * groups : most) || grids() != (tensor_maps() ? one : two) || cudaGetLastError())
