@@ -983,7 +983,7 @@ def mg_case(args):
         torch.cuda.synchronize()
         return e0.elapsed_time(e1) / reps
 
-    hbm = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("hbm_gbs", 6782.8)
+    hbm = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("hbm_gbs", 6796.9)
     t_r = timed(lambda: ctx.dd_mg_restrict(a, cvec))
     t_p = timed(lambda: ctx.dd_mg_prolong(cvec, b))
     t_c = timed(lambda: ctx.dd_mg_coarse_apply(cvec, cout))
